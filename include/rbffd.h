@@ -156,12 +156,19 @@ int rbffd_weights(const double* xy, const int32_t* idx, int64_t N, int32_t n, in
 /* double-float (warps_per_block 1..4: 2..8 stencils per block); 9 / 10:    */
 /* a quarter of a warp (8 threads), four stencils per warp (4..16 per      */
 /* block).                                                                  */
+/* Where 1 <= m <= 6 and n <= 64 every FP64 null-space configuration (0, 2, */
+/* 3, 7, 9) first runs the refined solve -- float32 elimination, then       */
+/* residuals and sums in 64-bit fixed point, to at least the accuracy of   */
+/* the FP64 elimination -- and the elimination, one warp per stencil, only */
+/* for the stencils whose refinement does not converge fast enough or that */
+/* may be singular; the configurations then give the same bits and take    */
+/* the same time, and autotuning times the default one for all of them.     */
 /* The default is FP64: 2 (two warps per stencil) for m >= 5 when it fits,  */
 /* 9 (a quarter warp, warps_per_block 2) for m <= 2 with n <= 16, 7 (half a */
 /* warp, warps_per_block 2) for other m <= 4 with n <= 32, 0 for other     */
 /* m >= 1, 1 for m = 0.                                                      */
-/* RBFFD_WEIGHTS=ns64 (environment) forces the FP64 null-space form with    */
-/* one warp per stencil, =df its double-float form (1 <= m <= 6), =lu the   */
+/* RBFFD_WEIGHTS=ns64 (environment) forces the FP64 null-space elimination  */
+/* of every stencil, one warp each, =df its double-float form (1 <= m <= 6), =lu the   */
 /* Gaussian elimination.                                                     */
 /* rbffd_weights_autotune times every candidate of the given precision      */
 /* (RBFFD_WEIGHTS_FP64: kernels 0-3, 7, 9; RBFFD_WEIGHTS_DF: 4-6, 8, 10;    */

@@ -28,7 +28,7 @@ CHECKED_LIB_PATH = os.path.join(LIB_DIR, "librbffd_checked.so")
 OBJ_DIR = os.path.join(PKG_DIR, "_build")
 CHECKED_FLAGS = ["-DRBFFD_CHECKED"]
 
-SOURCES = ["api.cu", "knn.cu", "weights.cu", "assemble.cu", "krylov.cu", "batched.cu", "mg.cu", "mg_batch.cu",
+SOURCES = ["api.cu", "knn.cu", "weights.cu", "refined.cu", "assemble.cu", "krylov.cu", "batched.cu", "mg.cu", "mg_batch.cu",
            "explicit.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",

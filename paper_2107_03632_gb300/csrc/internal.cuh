@@ -26,6 +26,15 @@ int coarse_weights(const double* xy, const int32_t* idx, int64_t N, int32_t n, i
 int interp_weights(const double* xy, int64_t Nd, const double* qxy, int64_t Nq, const int32_t* idx, int32_t n,
                    int32_t m, double* w, int32_t* node_status, cudaStream_t st);
 
+// Laplacian weights by float32 elimination and fixed-point refinement
+// (refined.cu), for the sizes refined_applies accepts.  Stencils it does not
+// decide get kWeightsMark (a NaN that no result has) as their first weight,
+// and neither their other weights nor their status are written.
+constexpr unsigned long long kWeightsMark = 0x7ff8726566696e65ull;
+bool refined_applies(int n, int m);
+int refined_weights(const double* xy, const int32_t* idx, int64_t N, int32_t n, int32_t m, double* w,
+                    int32_t* node_status, cudaStream_t st);
+
 // Multigrid hierarchy built by rbffd_mg_setup (lives in the caller's rbffd_mg).
 constexpr int kMgCoarsest = 128;  // dense inverse (one-block Gauss-Jordan) at or below this size
 constexpr int kMgK = 12;          // coarse nodes per interpolation stencil

@@ -1,0 +1,768 @@
+// RBF-FD Laplacian weights by float32 elimination and fixed-point refinement
+// (sm_103a): the FP64 null-space weight solve's fast path.
+//
+// The saddle-point system of a stencil (weights.cu: [Phi P; P^T 0] [w; l] =
+// [f; g] in scaled coordinates) is eliminated once in float32 by the
+// null-space method, and the solution is refined: the residual of the
+// current (w, l) is formed in 64-bit fixed point from kernel values and
+// monomials known to 2^-54 (fixed.cuh), the float32 factors solve for a
+// correction, and the sum is kept in 64-bit fixed point.  Each step reduces
+// the error by the float32 elimination's relative error (1e-3 to 1e-6 on
+// node sets of even density), so three to five solves reach the accuracy of
+// the residual, which is that of the kernel values: more bits than FP64
+// elimination carries.  Largest error per stencil relative to its largest
+// weight, against extended precision (disk of 1,321 nodes, 50 sampled rows;
+// here / FP64 elimination): m = 2, n = 12 1.3e-15 / 1.6e-14; m = 4, n = 30
+// 8.8e-15 / 1.7e-13; m = 6, n = 56 5.2e-13 / 3.5e-12.  A stencil whose corrections do not fall by 8x per step,
+// whose pivots are small, or whose values leave the fixed-point ranges is
+// marked and solved by the FP64 elimination kernel (weights.cu) in a second
+// launch, which also decides every singular case.
+//
+// Why: the FP64 units issue 2 lanes per clock per SM (the float and integer
+// pipes 128 and 64), and the FP64 elimination executes ~105k FP64
+// lane-operations per stencil at m = 6, n = 56.  Here FP64 is left to the
+// shift and scale of the coordinates and the final scaling.
+//
+// One thread per stencil node: NT = 16, 32 or 64 threads per stencil (two
+// stencils per warp, one, or one per two warps).  A thread holds its row of
+// the matrix being eliminated in registers; the pivot row goes through
+// shared memory as 16-byte broadcasts.  Pivot steps rotate the columns by
+// one, so the current column is always register 0 and the step loop needs no
+// unrolling; after s steps the columns are back in place.  Integer sums make
+// the result independent of the order of summation.
+#include "common.cuh"
+#include "fixed.cuh"
+#include "internal.cuh"
+
+#include <algorithm>
+
+namespace rbffd {
+namespace {
+
+// Row stride in floats: a multiple of 4 (16-byte loads) and an odd one, so
+// that the 16-byte loads of eight consecutive rows fall in distinct banks.
+__host__ __device__ constexpr int odd4(int k) { return ((k + 3) / 4 | 1) * 4; }
+__host__ __device__ constexpr int up4(int k) { return (k + 3) / 4 * 4; }
+
+// Shared memory of one stencil (byte offsets).
+//   phi   digits of |x_j - x_k|^3 2^56, entry [t - 1][j] for k = j + t mod n,
+//         t = 1 .. n/2: every pair once (t = n/2 twice for even n), and both
+//         of a thread's accesses in the residual are unit-stride
+//   pd    digits of the monomials 2^56, [j][k], odd stride; W^T before that
+//   A11 [s][LS], X [q][LS] = P2 P1^-1, Tt [q][LS] = (Phi12 - Phi11 X^T)^T,
+//   C [s][LS] = P1^-1, Sm [q][LQ] = (Z^T Phi Z)^-1
+struct RefGeom {
+    int n, q, LQ;
+    int phi, pd, A11, X, Tt, C, Sm, xy, xyf, prow, vr1, vr2, vg, vd0, vt, vdw, vh, dI, lI, pos, red, part, bytes;
+};
+
+RefGeom ref_geom(int NT, int n, int s) {
+    RefGeom g;
+    g.n = n;
+    g.q = n - s;
+    g.LQ = odd4(std::max(g.q, 1));
+    const int LS = odd4(s), LP = s | 1;
+    int off = 0;
+    auto take = [&](int bytes) {
+        const int o = off;
+        off += (bytes + 15) / 16 * 16;
+        return o;
+    };
+    g.phi = take((n / 2) * n * 8);
+    g.pd = take(std::max(n * LP * 8, g.q * LS * 4));
+    g.A11 = take(s * LS * 4);
+    g.X = take(g.q * LS * 4);
+    g.Tt = take(g.q * LS * 4);
+    g.C = take(s * LS * 4);
+    g.Sm = take(g.q * g.LQ * 4);
+    g.xy = take(n * 16);
+    g.xyf = take(n * 8);
+    g.prow = take(2 * (up4(NT) + 4) * 4);
+    g.vr1 = take(LS * 4);
+    g.vr2 = take(g.LQ * 4);
+    g.vg = take(LS * 4);
+    g.vd0 = take(LS * 4);
+    g.vt = take(g.LQ * 4);
+    g.vdw = take((s + g.LQ) * 4);
+    g.vh = take(LS * 4);
+    g.dI = take(2 * n * 4);
+    g.lI = take(LS * 4);
+    g.pos = take(n * 4);
+    g.red = take(64);
+    g.part = take(NT * 16);
+    g.bytes = off;
+    return g;
+}
+
+template <int NT>
+__device__ __forceinline__ unsigned ref_mask() {
+    if constexpr (NT >= 32) return 0xffffffffu;
+    else return ((1u << NT) - 1u) << ((threadIdx.x & 31) & ~(NT - 1));
+}
+
+template <int NT>
+__device__ __forceinline__ void ref_sync() {
+    if constexpr (NT <= 32) __syncwarp(ref_mask<NT>());
+    else __syncthreads();
+}
+
+// Maximum over the stencil's threads; `slot` alternates between consecutive
+// calls so that one barrier per call is enough.
+template <int NT>
+__device__ __forceinline__ unsigned ref_max(unsigned v, unsigned* red, int slot) {
+    v = __reduce_max_sync(ref_mask<NT>(), v);
+    if constexpr (NT > 32) {
+        if ((threadIdx.x & 31) == 0) red[slot * 2 + (threadIdx.x >> 5)] = v;
+        __syncthreads();
+        v = max(red[slot * 2], red[slot * 2 + 1]);
+    }
+    return v;
+}
+
+__device__ __forceinline__ float dot4(const float4& a, const float4& b, float acc) {
+    acc = fmaf(a.x, b.x, acc);
+    acc = fmaf(a.y, b.y, acc);
+    acc = fmaf(a.z, b.z, acc);
+    return fmaf(a.w, b.w, acc);
+}
+
+// sum of a[k] b[k] over k < 4 n4 (rows padded with zeros), two chains
+__device__ __forceinline__ float dotv(const float* a, const float* b, int n4) {
+    const float4* pa = reinterpret_cast<const float4*>(a);
+    const float4* pb = reinterpret_cast<const float4*>(b);
+    float s0 = 0.f, s1 = 0.f;
+    int k = 0;
+#pragma unroll 2
+    for (; k + 1 < n4; k += 2) {
+        s0 = dot4(pa[k], pb[k], s0);
+        s1 = dot4(pa[k + 1], pb[k + 1], s1);
+    }
+    if (k < n4) s0 = dot4(pa[k], pb[k], s0);
+    return s0 + s1;
+}
+
+constexpr float kRefPivot = 1e-5f;   // smaller pivots of P: the FP64 elimination decides
+constexpr float kRefRate = 0.125f;   // slowest accepted reduction per refinement step
+constexpr int kRefMaxSolves = 10;
+constexpr float kRefDone = 0x1p-53f; // predicted error of the sum, relative to max |w|
+
+template <int NT, int M>
+__global__ void __launch_bounds__(NT <= 32 ? 128 : 64) weights_refined_kernel(
+    const double2* __restrict__ xy, const int* __restrict__ idx, int N, const RefGeom g, double* __restrict__ w,
+    int* __restrict__ node_status) {
+    constexpr int S = (M + 1) * (M + 2) / 2;
+    constexpr int LS = odd4(S), S4 = up4(S) / 4, LP = S | 1;
+    constexpr int QM = up4(NT - S + 1);  // register row of the reduced matrix, one column of padding
+    constexpr int RT = NT == 64 ? 4 : 2;  // register tile of the float32 products (rows j)
+    constexpr int CT = NT == 16 ? 2 : 4;  //                                       (rows a)
+    extern __shared__ __align__(16) unsigned char smem_ref[];
+    const int t = threadIdx.x % NT;
+    unsigned char* base = smem_ref + (size_t)(threadIdx.x / NT) * g.bytes;
+    const int n = g.n, q = g.q, LQ = g.LQ, nh = n >> 1, q4 = (q + 3) >> 2;
+    (void)RB_SH(base + g.bytes - 1);
+    int2* phi = reinterpret_cast<int2*>(base + g.phi);
+    int2* pd = reinterpret_cast<int2*>(base + g.pd);
+    float* Wt = reinterpret_cast<float*>(base + g.pd);
+    float* A11 = reinterpret_cast<float*>(base + g.A11);
+    float* X = reinterpret_cast<float*>(base + g.X);
+    float* Tt = reinterpret_cast<float*>(base + g.Tt);
+    float* C = reinterpret_cast<float*>(base + g.C);
+    float* Sm = reinterpret_cast<float*>(base + g.Sm);
+    longlong2* cxy = reinterpret_cast<longlong2*>(base + g.xy);
+    float2* cxf = reinterpret_cast<float2*>(base + g.xyf);
+    float* prow = reinterpret_cast<float*>(base + g.prow);
+    float* vr1 = reinterpret_cast<float*>(base + g.vr1);
+    float* vr2 = reinterpret_cast<float*>(base + g.vr2);
+    float* vg = reinterpret_cast<float*>(base + g.vg);
+    float* vd0 = reinterpret_cast<float*>(base + g.vd0);
+    float* vt = reinterpret_cast<float*>(base + g.vt);
+    float* vdw = reinterpret_cast<float*>(base + g.vdw);
+    float* vy = reinterpret_cast<float*>(base + g.vt);  // after vt is consumed (a barrier between)
+    float* vh = reinterpret_cast<float*>(base + g.vh);
+    int* dI = reinterpret_cast<int*>(base + g.dI);
+    int* lI = reinterpret_cast<int*>(base + g.lI);
+    int* posS = reinterpret_cast<int*>(base + g.pos);
+    unsigned* red = reinterpret_cast<unsigned*>(base + g.red);
+    longlong2* part = reinterpret_cast<longlong2*>(base + g.part);
+    constexpr int PB = up4(NT) + 4;  // floats of one pivot-row buffer
+    const bool mine = t < n;
+    const int spb = blockDim.x / NT;
+
+    for (int node = blockIdx.x * spb + threadIdx.x / NT; node < N; node += gridDim.x * spb) {
+        bool ok = true;  // uniform over the stencil's threads
+        // ---- shift and scale (FP64) ------------------------------------------
+        const double2 c = xy[node];
+        double dx = 0.0, dy = 0.0;
+        unsigned lost = 0;
+        if (mine) {
+            const int sj = idx[(int64_t)node * n + t];
+            const bool in = (unsigned)sj < (unsigned)N;
+            const double2 p = in ? xy[sj] : c;
+            dx = __dadd_rn(p.x, -c.x);
+            dy = __dadd_rn(p.y, -c.y);
+            lost = in ? 0u : 1u;
+        }
+        // largest squared distance, as two 32-bit maxima of its bits
+        const unsigned long long d2 =
+            mine ? (unsigned long long)__double_as_longlong(fma(dx, dx, __dmul_rn(dy, dy))) & 0x7fffffffffffffffull : 0ull;
+        const unsigned top = ref_max<NT>(lost ? 0xffffffffu : (unsigned)(d2 >> 32), red, 0);
+        const unsigned low = ref_max<NT>((unsigned)(d2 >> 32) == top ? (unsigned)d2 : 0u, red, 1);
+        const double dmax = __hiloint2double((int)top, (int)low);
+        ok = top < 0x7ff00000u && seed_range(dmax);
+        double inv_delta2 = 0.0;
+        if (ok) {
+            const double id = rsqrt64(dmax);
+            inv_delta2 = __dmul_rn(id, id);
+            float xf = 0.f, yf = 0.f;
+            int64_t sown = 0;  // |xh| 2^60
+            if (mine) {
+                const double xh = __dmul_rn(dx, id), yh = __dmul_rn(dy, id);
+                const int64_t xi = fx_coord((uint64_t)__double_as_longlong(xh));
+                const int64_t yi = fx_coord((uint64_t)__double_as_longlong(yh));
+                cxy[t] = make_longlong2(xi, yi);
+                xf = (float)xi * 0x1p-61f;
+                yf = (float)yi * 0x1p-61f;
+                cxf[t] = make_float2(xf, yf);
+                const int64_t qi = fx_r2(xi, yi);
+                float qf = fmaf(xf, xf, yf * yf);
+                if (qf < 0x1p-14f) qf = (float)qi * 0x1p-58f;
+                if (qi > 0) sown = fx_sqrt(qi, qf, rsqrtf(qf));
+            }
+
+            // ---- P1^-1 and X = P2 P1^-1: Gauss-Jordan with row pivoting -------
+            float row[S];
+            int pos = -1;
+            row[0] = mine ? 1.f : 0.f;
+            if constexpr (M >= 1) {
+                row[1] = xf;
+                row[2] = yf;
+            }
+#pragma unroll
+            for (int d = 2; d <= M; ++d) {
+                const int cur = d * (d + 1) / 2, prev = (d - 1) * d / 2;
+#pragma unroll
+                for (int i = 0; i < d; ++i) row[cur + i] = xf * row[prev + i];
+                row[cur + d] = yf * row[prev + d - 1];
+            }
+            for (int k = 0; k < S; ++k) {
+                // largest |entry| of the column (ties and the last six bits: lower thread)
+                const unsigned key =
+                    mine && pos < 0 ? ((__float_as_uint(row[0]) & 0x7fffffc0u) | (unsigned)(63 - t)) : 0u;
+                const unsigned best = ref_max<NT>(key, red, 2 + (k & 1));
+                ok = best >= __float_as_uint(kRefPivot) && best < 0x7f800000u;
+                if (!ok) break;
+                const bool piv = t == 63 - (int)(best & 63u);
+                float* pr = prow + (k & 1) * PB;
+                if (piv) {
+                    pos = k;
+                    row[0] = __frcp_rn(row[0]);
+#pragma unroll
+                    for (int j = 0; j < S4; ++j) {
+                        float4 v;
+                        v.x = row[4 * j];
+                        v.y = 4 * j + 1 < S ? row[4 * j + 1 < S ? 4 * j + 1 : 0] : 0.f;
+                        v.z = 4 * j + 2 < S ? row[4 * j + 2 < S ? 4 * j + 2 : 0] : 0.f;
+                        v.w = 4 * j + 3 < S ? row[4 * j + 3 < S ? 4 * j + 3 : 0] : 0.f;
+                        reinterpret_cast<float4*>(pr)[j] = v;
+                    }
+#pragma unroll
+                    for (int j = 1; j < S; ++j) row[j] = 0.f;
+                }
+                ref_sync<NT>();
+                const float f = piv ? row[0] : row[0] * pr[0];
+#pragma unroll
+                for (int j = 0; j < S4; ++j) {
+                    const float4 v = reinterpret_cast<const float4*>(pr)[j];
+                    if (j > 0) row[4 * j - 1] = fmaf(-f, v.x, row[4 * j]);
+                    if (4 * j + 1 < S) row[4 * j] = fmaf(-f, v.y, row[4 * j + 1 < S ? 4 * j + 1 : 0]);
+                    if (4 * j + 2 < S) row[4 * j + 1 < S ? 4 * j + 1 : 0] = fmaf(-f, v.z, row[4 * j + 2 < S ? 4 * j + 2 : 0]);
+                    if (4 * j + 3 < S) row[4 * j + 2 < S ? 4 * j + 2 : 0] = fmaf(-f, v.w, row[4 * j + 3 < S ? 4 * j + 3 : 0]);
+                }
+                row[S - 1] = f;
+            }
+            if (ok) {
+                // permuted position: pivots in pivot order, then the others in node order
+                const unsigned bal = __ballot_sync(ref_mask<NT>(), mine && pos < 0) & ref_mask<NT>();
+                int rank = __popc(bal & ((1u << (threadIdx.x & 31)) - 1u));
+                if constexpr (NT > 32) {
+                    if (t == 0) red[8] = __popc(bal);
+                    __syncthreads();
+                    if (t >= 32) rank += (int)red[8];
+                }
+                if (mine) {
+                    if (pos < 0) pos = S + rank;
+                    RB_AT(posS, t, n) = pos;
+                    float* dst = pos < S ? &RB_AT(C, pos * LS, S * LS) : &RB_AT(X, (pos - S) * LS, q * LS);
+#pragma unroll
+                    for (int j = 0; j < S4; ++j) {
+                        float4 v;
+                        v.x = row[4 * j];
+                        v.y = 4 * j + 1 < S ? row[4 * j + 1 < S ? 4 * j + 1 : 0] : 0.f;
+                        v.z = 4 * j + 2 < S ? row[4 * j + 2 < S ? 4 * j + 2 : 0] : 0.f;
+                        v.w = 4 * j + 3 < S ? row[4 * j + 3 < S ? 4 * j + 3 : 0] : 0.f;
+                        reinterpret_cast<float4*>(dst)[j] = v;
+                    }
+                    // zero diagonal and padding of this row's block
+                    if (pos < S) {
+                        A11[pos * LS + pos] = 0.f;
+                        for (int j = S; j < 4 * S4; ++j) A11[pos * LS + j] = 0.f;
+                    } else {
+                        Sm[(pos - S) * LQ + pos - S] = 0.f;
+                        for (int j = S; j < 4 * S4; ++j) Tt[(pos - S) * LS + j] = Wt[(pos - S) * LS + j] = 0.f;
+                    }
+                }
+            }
+            ref_sync<NT>();
+
+            // ---- kernel values: fixed point for the residual, float32 blocks ----
+            bool close = false;  // two nodes closer than 2^-27 of the radius
+            if (ok && mine) {
+                const longlong2 me = cxy[t];
+                int k = t;
+#pragma unroll 2
+                for (int u = 0; u < nh; ++u) {
+                    k = k + 1 < n ? k + 1 : 0;
+                    const longlong2 o = RB_AT(cxy, k, n);
+                    const float2 of = RB_AT(cxf, k, n);
+                    const int64_t qi = fx_r2(me.x - o.x, me.y - o.y);
+                    const float fx = xf - of.x, fy = yf - of.y;
+                    float qf = fmaf(fx, fx, fy * fy);
+                    if (qf < 0x1p-14f) {
+                        close |= qi < 16;
+                        qf = fmaxf((float)qi * 0x1p-58f, 0x1p-58f);
+                    }
+                    const float ry = rsqrtf(qf);
+                    const Digits v = fx_digits(fx_cube(qi, fx_sqrt(qi, qf, ry)));
+                    phi[u * n + t] = make_int2(v.hi, v.lo);
+                    const float pf = qf * (qf * ry);
+                    const int b = RB_AT(posS, k, n);
+                    const int lo = min(pos, b), hi = max(pos, b);
+                    if (hi < S) {
+                        RB_AT(A11, hi * LS + lo, S * LS) = pf;
+                        RB_AT(A11, lo * LS + hi, S * LS) = pf;
+                    } else if (lo < S) {
+                        RB_AT(Tt, (hi - S) * LS + lo, q * LS) = pf;
+                    } else {
+                        RB_AT(Sm, (hi - S) * LQ + lo - S, q * LQ) = pf;
+                        RB_AT(Sm, (lo - S) * LQ + hi - S, q * LQ) = pf;
+                    }
+                }
+            }
+            ok = ok && ref_max<NT>(close ? 1u : 0u, red, 0) == 0u;  // (a barrier for NT = 64)
+            if constexpr (NT <= 32) ref_sync<NT>();
+
+            if (ok && q > 0) {
+                // ---- U^T = X Phi11; T^T = Phi21 - U^T, W^T = Phi21 - U^T / 2 ------
+                constexpr int TA = (S + CT - 1) / CT;
+                const int tj = (q + RT - 1) / RT;
+                for (int tile = t; tile < tj * TA; tile += NT) {
+                    const int j0 = tile / TA * RT, a0 = (tile - tile / TA * TA) * CT;
+                    float acc[RT][CT];
+#pragma unroll
+                    for (int i = 0; i < RT; ++i)
+#pragma unroll
+                        for (int a = 0; a < CT; ++a) acc[i][a] = 0.f;
+#pragma unroll
+                    for (int k = 0; k < S4; ++k) {
+                        float4 xr[RT], ar[CT];
+#pragma unroll
+                        for (int i = 0; i < RT; ++i)
+                            xr[i] = reinterpret_cast<const float4*>(X + min(j0 + i, q - 1) * LS)[k];
+#pragma unroll
+                        for (int a = 0; a < CT; ++a)
+                            ar[a] = reinterpret_cast<const float4*>(A11 + min(a0 + a, S - 1) * LS)[k];
+#pragma unroll
+                        for (int i = 0; i < RT; ++i)
+#pragma unroll
+                            for (int a = 0; a < CT; ++a) acc[i][a] = dot4(xr[i], ar[a], acc[i][a]);
+                    }
+#pragma unroll
+                    for (int i = 0; i < RT; ++i)
+#pragma unroll
+                        for (int a = 0; a < CT; ++a)
+                            if (j0 + i < q && a0 + a < S) {
+                                const int e = (j0 + i) * LS + a0 + a;
+                                const float v = Tt[e];
+                                Tt[e] = v - acc[i][a];
+                                Wt[e] = fmaf(-0.5f, acc[i][a], v);
+                            }
+                }
+                ref_sync<NT>();
+                // ---- S = Phi22 - X W - (X W)^T, lower tiles and their mirror -------
+                const int nt = (q + RT - 1) / RT;
+                for (int tile = t; tile < nt * (nt + 1) / 2; tile += NT) {
+                    int ti = (int)((sqrtf(8.0f * tile + 1.0f) - 1.0f) * 0.5f);
+                    while (ti * (ti + 1) / 2 > tile) --ti;
+                    while ((ti + 1) * (ti + 2) / 2 <= tile) ++ti;
+                    const int i0 = ti * RT, j0 = (tile - ti * (ti + 1) / 2) * RT;
+                    float acc[RT][RT];
+#pragma unroll
+                    for (int i = 0; i < RT; ++i)
+#pragma unroll
+                        for (int j = 0; j < RT; ++j) acc[i][j] = 0.f;
+#pragma unroll 1
+                    for (int h = 0; h < 2; ++h) {  // X_i . W_j, then W_i . X_j
+                        const float* pa = h ? Wt : X;
+                        const float* pb = h ? X : Wt;
+#pragma unroll
+                        for (int k = 0; k < S4; ++k) {
+                            float4 xr[RT], wr[RT];
+#pragma unroll
+                            for (int i = 0; i < RT; ++i) {
+                                xr[i] = reinterpret_cast<const float4*>(pa + min(i0 + i, q - 1) * LS)[k];
+                                wr[i] = reinterpret_cast<const float4*>(pb + min(j0 + i, q - 1) * LS)[k];
+                            }
+#pragma unroll
+                            for (int i = 0; i < RT; ++i)
+#pragma unroll
+                                for (int j = 0; j < RT; ++j) acc[i][j] = dot4(xr[i], wr[j], acc[i][j]);
+                        }
+                    }
+#pragma unroll
+                    for (int i = 0; i < RT; ++i)
+#pragma unroll
+                        for (int j = 0; j < RT; ++j)
+                            if (i0 + i < q && i0 + i >= j0 + j) {
+                                const float v = Sm[(i0 + i) * LQ + j0 + j] - acc[i][j];
+                                Sm[(i0 + i) * LQ + j0 + j] = v;
+                                Sm[(j0 + j) * LQ + i0 + i] = v;
+                            }
+                }
+                ref_sync<NT>();
+                // ---- S^-1, in place, S positive definite: no pivoting --------------
+                // (the pivot row carries -1 one column past its end, which puts
+                // the multiplier into the column that the rotation frees)
+                float r[QM];
+#pragma unroll
+                for (int j = 0; j < QM / 4; ++j) {
+                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (4 * j < q && t < q) {
+                        v = reinterpret_cast<const float4*>(Sm + t * LQ)[j];
+                        if (4 * j + 1 >= q) v.y = 0.f;
+                        if (4 * j + 2 >= q) v.z = 0.f;
+                        if (4 * j + 3 >= q) v.w = 0.f;
+                    }
+                    r[4 * j] = v.x;
+                    r[4 * j + 1] = v.y;
+                    r[4 * j + 2] = v.z;
+                    r[4 * j + 3] = v.w;
+                }
+                for (int k = 0; k < q; ++k) {
+                    float* pr = prow + (k & 1) * PB;
+                    const bool piv = t == k;
+                    if (piv) {
+                        const float d = r[0];
+                        r[0] = d > 0.f ? __frcp_rn(d) : 0.f;
+#pragma unroll
+                        for (int j = 0; j < QM / 4; ++j)
+                            if (4 * j <= q) {
+                                float4 v = make_float4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
+                                if (4 * j == q) v.x = -1.f;
+                                if (4 * j + 1 == q) v.y = -1.f;
+                                if (4 * j + 2 == q) v.z = -1.f;
+                                if (4 * j + 3 == q) v.w = -1.f;
+                                reinterpret_cast<float4*>(pr)[j] = v;
+                            }
+#pragma unroll
+                        for (int j = 1; j < QM; ++j) r[j] = 0.f;
+                    }
+                    ref_sync<NT>();
+                    const float inv = pr[0];
+                    ok = inv > 0.f && inv < INFINITY;
+                    if (!ok) break;
+                    const float f = piv ? inv : r[0] * inv;
+#pragma unroll
+                    for (int j = 0; j < QM / 4; ++j)
+                        if (4 * j <= q) {
+                            const float4 v = reinterpret_cast<const float4*>(pr)[j];
+                            if (j > 0) r[4 * j - 1] = fmaf(-f, v.x, r[4 * j]);
+                            r[4 * j] = fmaf(-f, v.y, r[4 * j + 1]);
+                            r[4 * j + 1] = fmaf(-f, v.z, r[4 * j + 2]);
+                            r[4 * j + 2] = fmaf(-f, v.w, r[4 * j + 3]);
+                            r[4 * j + 3] = 0.f;
+                        }
+                }
+                if (ok && t < q) {
+#pragma unroll
+                    for (int j = 0; j < QM / 4; ++j)
+                        if (4 * j < q)
+                            reinterpret_cast<float4*>(Sm + t * LQ)[j] =
+                                make_float4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
+                }
+            }
+
+            // ---- monomials in fixed point (W^T is no longer needed) ------------
+            if (ok && mine) {
+                const longlong2 me = cxy[t];
+                const Digits xd = fx_digits(me.x), yd = fx_digits(me.y);
+                int2* pr = pd + t * LP;
+                Digits up[M + 1];  // the previous degree's digits
+                up[0].hi = 1 << 24;
+                up[0].lo = 0;
+                pr[0] = make_int2(up[0].hi, up[0].lo);
+                int cur = 1;
+#pragma unroll
+                for (int d = 1; d <= M; ++d) {
+                    up[d] = fx_digits(fx_mono(yd, up[d - 1]));
+#pragma unroll
+                    for (int i = 0; i < d; ++i) up[i] = fx_digits(fx_mono(xd, up[i]));
+#pragma unroll
+                    for (int i = 0; i <= d; ++i) pr[cur + i] = make_int2(up[i].hi, up[i].lo);
+                    cur += d + 1;
+                }
+            }
+
+            // ---- solve and refine ------------------------------------------------
+            const float frhs = 9.0f * ((float)sown * 0x1p-60f);
+            const float grhs = (M >= 2 && (t == 3 || t == 5)) ? 2.0f : 0.0f;
+            float rf = frhs, rg = grhs;  // current residual, float32
+            int64_t ri = 0, rgi = 0;     // and in units of 2^(e - 64)
+            int64_t wi = 0;              // weight in units of 2^(e0 - 62)
+            int e0 = 0, eprev = 0;
+            float mprev = 0.f, mw0 = 0.f;
+            bool bad = false;
+            if (t < 4 * S4) {
+                vr1[t] = 0.f;
+                vg[t] = 0.f;
+                vd0[t] = 0.f;
+                vh[t] = 0.f;
+            }
+            if (t < 4 * q4) vr2[t] = vt[t] = 0.f;
+            ref_sync<NT>();
+            for (int it = 0; ok; ++it) {
+                // float32 correction (d, dl) of the residual (rf, rg)
+                if (mine) {
+                    if (pos < S) RB_AT(vr1, pos, S) = rf;
+                    else RB_AT(vr2, pos - S, q) = rf;
+                }
+                if (t < S) vg[t] = rg;
+                ref_sync<NT>();
+                const int i2 = NT - 1 - t;  // row of X, T^T and S^-1 (other threads than t < S where NT allows)
+                float a1 = 0.f, d0 = 0.f;
+                if (i2 < q) a1 = RB_AT(vr2, i2, q) - dotv(X + i2 * LS, vr1, S4);
+                if (t < S) {
+                    float s0 = 0.f, s1 = 0.f;
+#pragma unroll 4
+                    for (int k = 0; k + 1 < S; k += 2) {
+                        s0 = fmaf(C[k * LS + t], vg[k], s0);
+                        s1 = fmaf(C[(k + 1) * LS + t], vg[k + 1], s1);
+                    }
+                    if (S & 1) s0 = fmaf(C[(S - 1) * LS + t], vg[S - 1], s0);
+                    d0 = s0 + s1;
+                    vd0[t] = d0;
+                }
+                ref_sync<NT>();
+                if (i2 < q) vt[i2] = a1 - dotv(Tt + i2 * LS, vd0, S4);
+                ref_sync<NT>();
+                float yi = 0.f;
+                if (i2 < q) yi = dotv(Sm + i2 * LQ, vt, q4);
+                ref_sync<NT>();
+                if (i2 < q) {
+                    vy[i2] = yi;
+                    vdw[S + i2] = yi;
+                }
+                ref_sync<NT>();
+                if (t < S) {
+                    float s0 = 0.f, s1 = 0.f;
+#pragma unroll 4
+                    for (int j = 0; j < q; ++j) {
+                        const float y = vy[j];
+                        s0 = fmaf(X[j * LS + t], y, s0);
+                        s1 = fmaf(Tt[j * LS + t], y, s1);
+                    }
+                    vdw[t] = d0 - s0;
+                    vh[t] = vr1[t] - dotv(A11 + t * LS, vd0, S4) - s1;
+                }
+                ref_sync<NT>();
+                const float dj = mine ? RB_AT(vdw, pos, n) : 0.f;
+                const float dl = t < S ? dotv(C + (t < S ? t : 0) * LS, vh, S4) : 0.f;
+
+                // size of the correction, its rate of decrease
+                const unsigned inf = 0x7f800000u;
+                const unsigned uw = ref_max<NT>(bad ? inf : __float_as_uint(fabsf(dj)), red, 0);
+                const unsigned ul = ref_max<NT>(__float_as_uint(fabsf(dl)), red, 1);
+                const unsigned um = max(uw, ul);
+                if (um == 0u && it > 0) break;  // the residual is zero
+                const float m = __uint_as_float(um), mw = __uint_as_float(uw);
+                const int e = (int)(um >> 23) - 126;  // 2^e > m
+                if (um >= inf || e < -100 || e > 60) {  // not finite, a failed check, or out of scale
+                    ok = false;
+                    break;
+                }
+                if (it == 0) {
+                    e0 = e;
+                    mw0 = mw;
+                    ok = mw * 256.0f >= m;  // w must keep its bits in the common scale
+                    if (!ok) break;
+                }
+                const bool slow = it > 0 && !(m < kRefRate * mprev);
+                const bool done = it > 0 && mw * (m / mprev) <= kRefDone * mw0;
+                if (slow && !done) {
+                    ok = false;
+                    break;
+                }
+                // the correction in units of 2^(e - 25); the sum takes the same integers
+                const float sc = fx_pow2f(25 - e);
+                const int di = fx_round(dj * sc);
+                const int sh = 37 - (e0 - e);
+                wi += sh >= 0 ? (int64_t)((uint64_t)(int64_t)di << (sh & 63)) : ((int64_t)di >> min(-sh, 31));
+                if (done) break;
+                if (it + 1 >= kRefMaxSolves) {
+                    ok = false;
+                    break;
+                }
+                if (mine) {
+                    dI[t] = di;
+                    dI[t + n] = di;
+                }
+                if (t < S) lI[t] = fx_round(dl * sc);
+                ref_sync<NT>();
+
+                // residual: r -= Phi d + P dl, rg -= P^T d, exact digit sums of
+                // unit 2^(e - 49) (hi) and 2^(e - 81) (lo)
+                const int up = it ? eprev - e : 0;
+                if (mine) {
+                    int64_t H = 0, L = 0;
+                    int k = t;  // node t - u - 1 (cyclic)
+                    const int full = (n & 1) ? nh : nh - 1;
+#pragma unroll 4
+                    for (int u = 0; u < full; ++u) {
+                        k = k > 0 ? k - 1 : n - 1;
+                        const int2 a = phi[u * n + t], b = RB_AT(phi, u * n + k, nh * n);
+                        const int da = dI[t + u + 1], db = RB_AT(dI, k, n);
+                        H += fx_mul32(a.x, da) + fx_mul32(b.x, db);
+                        L += fx_mul32(a.y, da) + fx_mul32(b.y, db);
+                    }
+                    if (full < nh) {  // n even: the opposite node, once
+                        const int2 a = phi[full * n + t];
+                        const int da = dI[t + nh];
+                        H += fx_mul32(a.x, da);
+                        L += fx_mul32(a.y, da);
+                    }
+                    const int2* pr = pd + t * LP;
+#pragma unroll 7
+                    for (int kk = 0; kk < S; ++kk) {
+                        const int2 a = pr[kk];
+                        const int d = lI[kk];
+                        H += fx_mul32(a.x, d);
+                        L += fx_mul32(a.y, d);
+                    }
+                    if (it == 0) {  // 9 |xh|: 2^-60 to 2^(e - 64)
+                        const int s = e - 4;
+                        ri = (int64_t)(9ull * (s >= 0 ? (uint64_t)(sown >> min(s, 62)) : (uint64_t)sown << min(-s, 63)));
+                    } else {
+                        ri = up < 64 ? (int64_t)((uint64_t)ri << up) : 0;
+                    }
+                    ri = (int64_t)((uint64_t)ri - ((uint64_t)H << 15) - (uint64_t)(L >> 17));
+                    // the 64-bit wrap is harmless while the true residual is below 2^(e - 1)
+                    bad |= !(fabsf(rf - (float)H * fx_pow2f(e - 49)) < fx_pow2f(e - 2));
+                    rf = (float)ri * fx_pow2f(e - 64);
+                }
+                // rg: two threads per monomial where there are enough
+                constexpr int HS = NT / 2 >= S ? 2 : 1;
+                int64_t H = 0, L = 0;
+                const int kc = HS == 2 ? t % (NT / 2) : t;
+                if (kc < S) {
+                    const int j0 = HS == 2 ? t / (NT / 2) : 0;
+#pragma unroll 4
+                    for (int j = j0; j < n; j += HS) {
+                        const int2 a = pd[j * LP + kc];
+                        const int d = dI[j];
+                        H += fx_mul32(a.x, d);
+                        L += fx_mul32(a.y, d);
+                    }
+                    if (HS == 2 && t >= NT / 2) part[kc] = make_longlong2(H, L);
+                }
+                if (HS == 2) ref_sync<NT>();
+                if (t < S) {
+                    if (HS == 2) {
+                        H += part[t].x;
+                        L += part[t].y;
+                    }
+                    if (it == 0) {
+                        const int s = 65 - e;  // 2 in units of 2^(e - 64)
+                        rgi = grhs != 0.f && s < 64 ? (int64_t)(1ull << s) : 0;
+                    } else {
+                        rgi = up < 64 ? (int64_t)((uint64_t)rgi << up) : 0;
+                    }
+                    rgi = (int64_t)((uint64_t)rgi - ((uint64_t)H << 15) - (uint64_t)(L >> 17));
+                    bad |= !(fabsf(rg - (float)H * fx_pow2f(e - 49)) < fx_pow2f(e - 2));
+                    rg = (float)rgi * fx_pow2f(e - 64);
+                }
+                eprev = e;
+                mprev = m;
+                ref_sync<NT>();
+            }
+
+            // ---- scale back (FP64) and store --------------------------------------
+            if (ok) {
+                const double v = __dmul_rn((double)wi, __dmul_rn(inv_delta2, __hiloint2double((e0 - 62 + 1023) << 20, 0)));
+                ok = ref_max<NT>(mine && !finite64(v) ? 1u : 0u, red, 0) == 0u;
+                if (ok && mine) w[(int64_t)node * n + t] = v;
+                if (ok && node_status && t == 0) node_status[node] = 0;
+            }
+        }
+        if (!ok && t == 0) w[(int64_t)node * n] = __longlong_as_double((long long)kWeightsMark);
+        ref_sync<NT>();
+    }
+}
+
+template <int NT, int M>
+int launch(const double2* xy, const int32_t* idx, int64_t N, int n, double* w, int32_t* node_status,
+           cudaStream_t st) {
+    const RefGeom g = ref_geom(NT, n, (M + 1) * (M + 2) / 2);
+    auto kern = weights_refined_kernel<NT, M>;
+    // stencils per block: one where a stencil spans two warps, else enough
+    // warps (at most four) for the most resident stencils per SM
+    int spb = 1;
+    if (NT <= 32) {
+        int best = 0;
+        for (int s = 32 / NT; s <= 128 / NT; s += 32 / NT) {
+            const int blocks = std::min(32, (int)(233472 / (s * g.bytes + 1024)));
+            if (s * g.bytes <= 227 * 1024 && blocks * s >= best) {
+                best = blocks * s;
+                spb = s;
+            }
+        }
+    }
+    const size_t smem = (size_t)spb * g.bytes;
+    RBFFD_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    RBFFD_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+    int per_sm = 0;
+    RBFFD_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT * spb, smem));
+    if (per_sm < 1) return RBFFD_ERR_INVALID_ARG;
+    const int64_t need = (N + spb - 1) / spb;
+    const int blocks = (int)std::min<int64_t>(need, (int64_t)per_sm * sm_count());
+    kern<<<blocks, NT * spb, smem, st>>>(xy, idx, (int)N, g, w, node_status);
+    return RBFFD_OK;
+}
+
+template <int M>
+int launch_m(const double2* xy, const int32_t* idx, int64_t N, int n, double* w, int32_t* node_status,
+             cudaStream_t st) {
+    constexpr int S = (M + 1) * (M + 2) / 2;
+    if constexpr (S <= 16)
+        if (n <= 16) return launch<16, M>(xy, idx, N, n, w, node_status, st);
+    if (n <= 32) return launch<32, M>(xy, idx, N, n, w, node_status, st);
+    return launch<64, M>(xy, idx, N, n, w, node_status, st);
+}
+
+}  // namespace
+
+bool refined_applies(int n, int m) { return m >= 1 && m <= 6 && n <= 64 && n >= (m + 1) * (m + 2) / 2; }
+
+int refined_weights(const double* xy, const int32_t* idx, int64_t N, int32_t n, int32_t m, double* w,
+                    int32_t* node_status, cudaStream_t st) {
+    const double2* p = reinterpret_cast<const double2*>(xy);
+    switch (m) {
+        case 1: return launch_m<1>(p, idx, N, n, w, node_status, st);
+        case 2: return launch_m<2>(p, idx, N, n, w, node_status, st);
+        case 3: return launch_m<3>(p, idx, N, n, w, node_status, st);
+        case 4: return launch_m<4>(p, idx, N, n, w, node_status, st);
+        case 5: return launch_m<5>(p, idx, N, n, w, node_status, st);
+        case 6: return launch_m<6>(p, idx, N, n, w, node_status, st);
+        default: return RBFFD_ERR_INVALID_ARG;
+    }
+}
+
+}  // namespace rbffd

@@ -1,6 +1,8 @@
 // RBF-FD Laplacian weights: one augmented PHS+polynomial system per stencil,
 // held in shared memory and solved by one, two or four warps (sm_103a), in
-// FP64 (the default) or in double-float arithmetic (opt-in).
+// FP64 or in double-float arithmetic (opt-in).  The FP64 null-space
+// configurations run the refined solve of refined.cu first where it applies
+// (n <= 64, 1 <= m <= 6) and the elimination here for the stencils it leaves.
 //
 // Sec. II, Eq. 1: (L u)(x_c) ~ sum_j w_j u(x_j) over the stencil of x_c.
 // Sec. V: Phi(r) = r^3 augmented with the monomials of degree <= m, L = lap.
@@ -539,7 +541,10 @@ struct NsDF {
 // next diagonal entry's reciprocal, the scale) are computed by one thread
 // and handed to the others through shared memory: computed by every thread
 // of the group they cost as many FP64 lane-operations as a full row update.
-template <int NT, class R>
+//
+// MARKED (NT = 32 only): solves just the stencils whose first weight is
+// kWeightsMark; a warp looks at 32 stencils at a time.
+template <int NT, class R, bool MARKED = false>
 __global__ void __launch_bounds__(128) weights_ns_kernel(const double2* __restrict__ xy, const int* __restrict__ idx,
                                                          int N, int n, int m, int s, int LDQ, int LDS,
                                                          int bytes_per_warp, double* __restrict__ w,
@@ -586,7 +591,29 @@ __global__ void __launch_bounds__(128) weights_ns_kernel(const double2* __restri
     auto ldc = [&](const S* p) -> V { return R::ld(&RB_PT(p, Phi, region)); };
     auto stc = [&](S* p, V v) { R::st(&RB_PT(p, Phi, region), v); };
 
-    for (int node = blockIdx.x * wpb + wib; node < N; node += total_warps) {
+    static_assert(!MARKED || NT == 32, "marked stencils are found by whole warps");
+    int64_t ahead = (int64_t)(blockIdx.x * wpb + wib) * (MARKED ? 32 : 1);  // next stencil, or group of 32
+    unsigned found = 0;  // marked stencils not yet solved of the 32 from `from` on
+    int from = 0;
+    auto next = [&](int& node) -> bool {
+        if constexpr (!MARKED) {
+            node = (int)ahead;
+            ahead += total_warps;
+            return node < N && node >= 0;
+        } else {
+            while (found == 0) {
+                if (ahead >= N) return false;
+                from = (int)ahead;
+                found = __ballot_sync(0xffffffffu, ahead + lane < N && (unsigned long long)__double_as_longlong(
+                                                                           w[(ahead + lane) * n]) == kWeightsMark);
+                ahead += (int64_t)total_warps * 32;
+            }
+            node = from + __ffs(found) - 1;
+            found &= found - 1;
+            return true;
+        }
+    };
+    for (int node; next(node);) {
         const int* sten = idx + (int64_t)node * n;
         const double2 c = cxy[node];
 
@@ -1005,6 +1032,7 @@ struct WCfg {
                  // 7 / 8: null-space elimination with half a warp per stencil,
                  // FP64 / double-float; 9 / 10: the same with a quarter warp
     int wpb;     // warps per block (kernels 2, 3: 2 or 4, one stencil)
+    int direct = 0;  // FP64 null-space kernels: 1 skips the refined solve
 };
 
 std::mutex g_wcfg_mu;
@@ -1029,6 +1057,10 @@ int stencils_per_block(const WCfg& c) {
     return (c.kernel == 2 || c.kernel == 3 || c.kernel == 5 || c.kernel == 6) ? 1 : c.wpb;
 }
 
+bool cfg_is_ns64(const WCfg& c) {
+    return c.kernel == 0 || c.kernel == 2 || c.kernel == 3 || c.kernel == 7 || c.kernel == 9;
+}
+
 bool cfg_is_df(const WCfg& c) { return (c.kernel >= 4 && c.kernel <= 6) || c.kernel == 8 || c.kernel == 10; }
 
 // The double-float null-space kernels: 1 <= m <= 6 (accuracy, see NsDF).
@@ -1046,6 +1078,8 @@ bool cfg_valid(const WCfg& c, int n, int m) {
     return block_smem(c, n, m) <= 227 * 1024;
 }
 
+// (The figures are of the elimination alone: it solves every stencil for
+// n > 64 or m > 6, and under RBFFD_WEIGHTS=ns64.)
 WCfg default_cfg(int n, int m) {
     WCfg c;
     // FP64 by default: null-space elimination (m >= 1: the form needs r^3
@@ -1087,7 +1121,8 @@ WCfg small_df_cfg(int n, int m) {
 
 WCfg chosen_cfg(int n, int m) {
     // RBFFD_WEIGHTS=lu forces the full Gaussian elimination (comparisons)
-    // RBFFD_WEIGHTS=ns64 forces the FP64 null-space elimination, one warp
+    // RBFFD_WEIGHTS=ns64 forces the FP64 null-space elimination, one warp,
+    // for every stencil (no refined solve)
     // RBFFD_WEIGHTS=df forces its double-float form, one warp (1 <= m <= 6)
     const char* sel = std::getenv("RBFFD_WEIGHTS");
     if (sel && std::strcmp(sel, "df") == 0 && m >= 1 && m <= kDfMaxM) {
@@ -1101,6 +1136,7 @@ WCfg chosen_cfg(int n, int m) {
         size_t smem = 0;
         c.kernel = std::strcmp(sel, "lu") == 0 ? 1 : 0;
         c.wpb = warps_per_block_for(smem_per_stencil(c.kernel, n, m), &smem);
+        c.direct = 1;
         return c;
     }
     std::lock_guard<std::mutex> lk(g_wcfg_mu);
@@ -1109,7 +1145,7 @@ WCfg chosen_cfg(int n, int m) {
     return default_cfg(n, m);
 }
 
-template <int NT, class R>
+template <int NT, class R, bool MARKED = false>
 int launch_ns(const WCfg& c, const double2* xy, const int32_t* idx, int64_t N, int n, int m, double* w,
               int32_t* node_status, cudaStream_t st, const double2* cxy = nullptr, int64_t Nd = 0, int op = 0) {
     if (!cxy) {
@@ -1119,13 +1155,14 @@ int launch_ns(const WCfg& c, const double2* xy, const int32_t* idx, int64_t N, i
     NsGeom g = ns_geom(n, m);
     const int spb = stencils_per_block(c);
     const size_t smem = block_smem(c, n, m);
-    auto kern = weights_ns_kernel<NT, R>;
+    auto kern = weights_ns_kernel<NT, R, MARKED>;
     RBFFD_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     RBFFD_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
     int per_sm = 0;
     RBFFD_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT * spb, smem));
     if (per_sm < 1) return RBFFD_ERR_INVALID_ARG;
-    const int64_t need = (N + spb - 1) / spb;
+    const int64_t per_block = (int64_t)spb * (MARKED ? 32 : 1);
+    const int64_t need = (N + per_block - 1) / per_block;
     const int blocks = (int)std::min<int64_t>(need, (int64_t)per_sm * sm_count());
     kern<<<blocks, NT * spb, smem, st>>>(xy, idx, (int)N, n, m, g.s, g.LDQ, g.LDS, g.bytes, w, node_status, cxy,
                                          (int)Nd, op);
@@ -1137,7 +1174,17 @@ int launch_weights(const WCfg& c, const double* xy, const int32_t* idx, int64_t 
     if (!cfg_valid(c, n, m)) return RBFFD_ERR_INVALID_ARG;
     const double2* p = reinterpret_cast<const double2*>(xy);
     int rc = RBFFD_OK;
-    if (c.kernel == 1) {
+    if (cfg_is_ns64(c) && !c.direct && refined_applies(n, m)) {
+        // every FP64 null-space configuration: the refined solve, then the
+        // elimination (one warp per stencil) of the stencils it left
+        rc = refined_weights(xy, idx, N, n, m, w, node_status, st);
+        if (rc != RBFFD_OK) return rc;
+        note_launches(1);
+        WCfg left{0, 1};
+        size_t smem = 0;
+        left.wpb = warps_per_block_for(smem_per_stencil(0, n, m), &smem);
+        rc = launch_ns<32, NsF64, true>(left, p, idx, N, n, m, w, node_status, st);
+    } else if (c.kernel == 1) {
         WeightsGeom g = weights_geom(n, m);
         const int wpb = c.wpb;
         const size_t smem = block_smem(c, n, m);
@@ -1222,8 +1269,12 @@ extern "C" int rbffd_weights_autotune(const double* xy, const int32_t* idx, int6
         all.push_back(WCfg{10, wpb});
     }
     std::vector<WCfg> cands;
+    const WCfg def = default_cfg(n, m);
     for (const WCfg& c : all) {
         if (!cfg_valid(c, n, m)) continue;
+        // the FP64 null-space configurations share the refined solve where it
+        // applies: the default one stands for them
+        if (cfg_is_ns64(c) && refined_applies(n, m) && (c.kernel != def.kernel || c.wpb != def.wpb)) continue;
         if (precision == RBFFD_WEIGHTS_FP64 && cfg_is_df(c)) continue;
         if (precision == RBFFD_WEIGHTS_DF && !cfg_is_df(c)) continue;
         cands.push_back(c);
