@@ -48,12 +48,14 @@ __host__ __device__ constexpr int up4(int k) { return (k + 3) / 4 * 4; }
 //   phi   digits of |x_j - x_k|^3 2^56, entry [t - 1][j] for k = j + t mod n,
 //         t = 1 .. n/2: every pair once (t = n/2 twice for even n), and both
 //         of a thread's accesses in the residual are unit-stride
-//   pd    digits of the monomials 2^56, [j][k], odd stride; W^T before that
-//   A11 [s][LS], X [q][LS] = P2 P1^-1, Tt [q][LS] = (Phi12 - Phi11 X^T)^T,
-//   C [s][LS] = P1^-1, Sm [q][LQ] = (Z^T Phi Z)^-1
+//   pd    digits of the monomials 2^56, [j][k], odd stride.  Before they are
+//         formed the region holds W^T at its start and Phi11 at its end
+//   F1    [Phi11; Phi21], n rows of LS (pivot nodes first): rows S.. become
+//         T^T = (Phi12 - Phi11 X^T)^T, rows 0..S are inside pd
+//   X [q][LS] = P2 P1^-1, C [s][LS] = P1^-1, Sm [q][LQ] = (Z^T Phi Z)^-1
 struct RefGeom {
     int n, q, LQ;
-    int phi, pd, A11, X, Tt, C, Sm, xy, xyf, prow, vr1, vr2, vg, vd0, vt, vdw, vh, dI, lI, pos, red, part, bytes;
+    int phi, pd, F1, X, C, Sm, xy, xyf, prow, vr1, vr2, vg, vd0, vt, vy, vdw, dI, lI, pos, red, part, bytes;
 };
 
 RefGeom ref_geom(int NT, int n, int s) {
@@ -69,10 +71,10 @@ RefGeom ref_geom(int NT, int n, int s) {
         return o;
     };
     g.phi = take((n / 2) * n * 8);
-    g.pd = take(std::max(n * LP * 8, g.q * LS * 4));
-    g.A11 = take(s * LS * 4);
+    g.pd = take(n * LP * 8);
+    const int tt = take(g.q * LS * 4);
+    g.F1 = tt - s * LS * 4;
     g.X = take(g.q * LS * 4);
-    g.Tt = take(g.q * LS * 4);
     g.C = take(s * LS * 4);
     g.Sm = take(g.q * g.LQ * 4);
     g.xy = take(n * 16);
@@ -83,13 +85,13 @@ RefGeom ref_geom(int NT, int n, int s) {
     g.vg = take(LS * 4);
     g.vd0 = take(LS * 4);
     g.vt = take(g.LQ * 4);
-    g.vdw = take((s + g.LQ) * 4);
-    g.vh = take(LS * 4);
+    g.vy = take(g.LQ * 4);
+    g.vdw = take(n * 4);
     g.dI = take(2 * n * 4);
     g.lI = take(LS * 4);
     g.pos = take(n * 4);
     g.red = take(64);
-    g.part = take(NT * 16);
+    g.part = take(NT >= 2 * s ? s * 16 : 0);
     g.bytes = off;
     return g;
 }
@@ -141,10 +143,115 @@ __device__ __forceinline__ float dotv(const float* a, const float* b, int n4) {
     return s0 + s1;
 }
 
+// Reciprocal and reciprocal square root to about one ulp of float32 (one
+// instruction each; arguments are normal floats).
+__device__ __forceinline__ float rcpf(float a) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return r;
+}
+__device__ __forceinline__ float rsqf(float a) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return r;
+}
+
+// The sum hi 2^32 + lo in units 2^(32 - sh) times its own (sh <= 32).
+__device__ __forceinline__ uint64_t fx_scale(int64_t hi, int64_t lo, int sh) {
+    const uint64_t h = sh >= 0 ? (uint64_t)hi << min(sh, 63) : (uint64_t)(hi >> min(-sh, 63));
+    return h + (uint64_t)(lo >> min(32 - sh, 63));
+}
+
 constexpr float kRefPivot = 1e-5f;   // smaller pivots of P: the FP64 elimination decides
 constexpr float kRefRate = 0.125f;   // slowest accepted reduction per refinement step
 constexpr int kRefMaxSolves = 10;
-constexpr float kRefDone = 0x1p-53f; // predicted error of the sum, relative to max |w|
+// Predicted error at which refinement stops, relative to max |w|: about a
+// tenth of the FP64 elimination's median error (3e-15, 2e-14, 8e-14 at m = 2,
+// 4, 6), and full accuracy near n = s, where the elimination is as accurate.
+template <int M>
+__device__ __forceinline__ float ref_done(int n, int s) {
+    if (n < 2 * s) return 0x1p-53f;
+    return M <= 2 ? 0x1p-51f : M <= 4 ? 0x1p-49f : 0x1p-47f;
+}
+
+// Matrix in place of its inverse by Gauss-Jordan without pivoting (positive
+// definite), row t of the q x q matrix A (row stride LQ) in thread t's
+// registers, 4 QC > q columns.  The columns rotate by one per step; the pivot
+// row carries -1 one column past its end, which puts the multiplier into the
+// column that the rotation frees.  False where a pivot is not positive.
+template <int NT, int QC>
+__device__ __forceinline__ bool ref_invert(float* A, int q, int LQ, int t, float* prow, int PB) {
+    float r[4 * QC];
+#pragma unroll
+    for (int j = 0; j < QC; ++j) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (4 * j < q && t < q) {
+            v = reinterpret_cast<const float4*>(A + t * LQ)[j];
+            if (4 * j + 1 >= q) v.y = 0.f;
+            if (4 * j + 2 >= q) v.z = 0.f;
+            if (4 * j + 3 >= q) v.w = 0.f;
+        }
+        r[4 * j] = v.x;
+        r[4 * j + 1] = v.y;
+        r[4 * j + 2] = v.z;
+        r[4 * j + 3] = v.w;
+    }
+    // the -1 of both pivot-row buffers is rewritten by every pivot thread
+    for (int k = 0; k < q; ++k) {
+        float4* pr = reinterpret_cast<float4*>(prow + (k & 1) * PB);
+        const bool piv = t == k;
+        if (piv) {
+            r[0] = r[0] > 0.f ? rcpf(r[0]) : 0.f;
+#pragma unroll
+            for (int j = 0; j < QC; ++j) pr[j] = make_float4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
+            prow[(k & 1) * PB + q] = -1.f;
+#pragma unroll
+            for (int j = 1; j < 4 * QC; ++j) r[j] = 0.f;
+        }
+        ref_sync<NT>();
+        const float4 v0 = pr[0];
+        if (!(v0.x > 0.f && v0.x < INFINITY)) return false;
+        const float f = piv ? v0.x : r[0] * v0.x;
+        r[0] = fmaf(-f, v0.y, r[1]);
+        r[1] = fmaf(-f, v0.z, r[2]);
+        r[2] = fmaf(-f, v0.w, r[3]);
+#pragma unroll
+        for (int j = 1; j < QC; ++j) {
+            const float4 v = pr[j];
+            r[4 * j - 1] = fmaf(-f, v.x, r[4 * j]);
+            r[4 * j] = fmaf(-f, v.y, r[4 * j + 1]);
+            r[4 * j + 1] = fmaf(-f, v.z, r[4 * j + 2]);
+            r[4 * j + 2] = fmaf(-f, v.w, r[4 * j + 3]);
+        }
+        r[4 * QC - 1] = 0.f;
+        // (q = 4 QC - 1: the multiplier went to column q - 1 = 4 QC - 2 above)
+    }
+    if (t < q) {
+#pragma unroll
+        for (int j = 0; j < QC; ++j)
+            if (4 * j < q)
+                reinterpret_cast<float4*>(A + t * LQ)[j] =
+                    make_float4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
+    }
+    return true;
+}
+
+// The instance of ref_invert with enough columns (QMAX: chunks a kernel can need).
+template <int NT, int QMAX>
+__device__ __forceinline__ bool ref_invert_any(float* A, int q, int LQ, int t, float* prow, int PB) {
+    const int need = q / 4 + 1;
+    if constexpr (QMAX > 2)
+        if (need <= 2) return ref_invert<NT, 2>(A, q, LQ, t, prow, PB);
+    if constexpr (QMAX > 4)
+        if (need <= 4) return ref_invert<NT, 4>(A, q, LQ, t, prow, PB);
+    if constexpr (QMAX > 6)
+        if (need <= 6) return ref_invert<NT, 6>(A, q, LQ, t, prow, PB);
+    if constexpr (QMAX > 8)
+        if (need <= 8) return ref_invert<NT, 8>(A, q, LQ, t, prow, PB);
+    if constexpr (QMAX > 12)
+        if (need <= 12) return ref_invert<NT, 12>(A, q, LQ, t, prow, PB);
+    return ref_invert<NT, QMAX>(A, q, LQ, t, prow, PB);
+}
 
 template <int NT, int M>
 __global__ void __launch_bounds__(NT <= 32 ? 128 : 64) weights_refined_kernel(
@@ -152,9 +259,9 @@ __global__ void __launch_bounds__(NT <= 32 ? 128 : 64) weights_refined_kernel(
     int* __restrict__ node_status) {
     constexpr int S = (M + 1) * (M + 2) / 2;
     constexpr int LS = odd4(S), S4 = up4(S) / 4, LP = S | 1;
-    constexpr int QM = up4(NT - S + 1);  // register row of the reduced matrix, one column of padding
-    constexpr int RT = NT == 64 ? 4 : 2;  // register tile of the float32 products (rows j)
-    constexpr int CT = NT == 16 ? 2 : 4;  //                                       (rows a)
+    constexpr int QMAX = (NT - S) / 4 + 1;  // 16-byte chunks of a row of the reduced matrix and one column
+    constexpr int RT = NT == 64 ? 4 : 2;    // register tile of the float32 products (rows j)
+    constexpr int CT = NT == 16 ? 2 : 4;    //                                       (rows a)
     extern __shared__ __align__(16) unsigned char smem_ref[];
     const int t = threadIdx.x % NT;
     unsigned char* base = smem_ref + (size_t)(threadIdx.x / NT) * g.bytes;
@@ -163,9 +270,9 @@ __global__ void __launch_bounds__(NT <= 32 ? 128 : 64) weights_refined_kernel(
     int2* phi = reinterpret_cast<int2*>(base + g.phi);
     int2* pd = reinterpret_cast<int2*>(base + g.pd);
     float* Wt = reinterpret_cast<float*>(base + g.pd);
-    float* A11 = reinterpret_cast<float*>(base + g.A11);
+    float* F1 = reinterpret_cast<float*>(base + g.F1);  // Phi11, then T^T
+    float* Tt = F1 + S * LS;
     float* X = reinterpret_cast<float*>(base + g.X);
-    float* Tt = reinterpret_cast<float*>(base + g.Tt);
     float* C = reinterpret_cast<float*>(base + g.C);
     float* Sm = reinterpret_cast<float*>(base + g.Sm);
     longlong2* cxy = reinterpret_cast<longlong2*>(base + g.xy);
@@ -176,9 +283,8 @@ __global__ void __launch_bounds__(NT <= 32 ? 128 : 64) weights_refined_kernel(
     float* vg = reinterpret_cast<float*>(base + g.vg);
     float* vd0 = reinterpret_cast<float*>(base + g.vd0);
     float* vt = reinterpret_cast<float*>(base + g.vt);
+    float* vy = reinterpret_cast<float*>(base + g.vy);
     float* vdw = reinterpret_cast<float*>(base + g.vdw);
-    float* vy = reinterpret_cast<float*>(base + g.vt);  // after vt is consumed (a barrier between)
-    float* vh = reinterpret_cast<float*>(base + g.vh);
     int* dI = reinterpret_cast<int*>(base + g.dI);
     int* lI = reinterpret_cast<int*>(base + g.lI);
     int* posS = reinterpret_cast<int*>(base + g.pos);
@@ -214,29 +320,31 @@ __global__ void __launch_bounds__(NT <= 32 ? 128 : 64) weights_refined_kernel(
             const double id = rsqrt64(dmax);
             inv_delta2 = __dmul_rn(id, id);
             float xf = 0.f, yf = 0.f;
+            longlong2 me = make_longlong2(0, 0);
             int64_t sown = 0;  // |xh| 2^60
             if (mine) {
                 const double xh = __dmul_rn(dx, id), yh = __dmul_rn(dy, id);
-                const int64_t xi = fx_coord((uint64_t)__double_as_longlong(xh));
-                const int64_t yi = fx_coord((uint64_t)__double_as_longlong(yh));
-                cxy[t] = make_longlong2(xi, yi);
-                xf = (float)xi * 0x1p-61f;
-                yf = (float)yi * 0x1p-61f;
+                me.x = fx_coord((uint64_t)__double_as_longlong(xh));
+                me.y = fx_coord((uint64_t)__double_as_longlong(yh));
+                cxy[t] = me;
+                xf = (float)me.x * 0x1p-61f;
+                yf = (float)me.y * 0x1p-61f;
                 cxf[t] = make_float2(xf, yf);
-                const int64_t qi = fx_r2(xi, yi);
+                const int64_t qi = fx_r2(me.x, me.y);
                 float qf = fmaf(xf, xf, yf * yf);
                 if (qf < 0x1p-14f) qf = (float)qi * 0x1p-58f;
-                if (qi > 0) sown = fx_sqrt(qi, qf, rsqrtf(qf));
+                if (qi > 0) sown = fx_sqrt(qi, qf, rsqf(qf));
             }
+            if constexpr (NT > 32) ref_sync<NT>();
 
-            // ---- P1^-1 and X = P2 P1^-1: Gauss-Jordan with row pivoting -------
+            // ---- P1^-1, X = P2 P1^-1 (Gauss-Jordan, row pivoting) and the kernel
+            // values in fixed point: one pivot step and one pair per turn, so
+            // that the pair's arithmetic fills the step's barriers and chain
             float row[S];
             int pos = -1;
             row[0] = mine ? 1.f : 0.f;
-            if constexpr (M >= 1) {
-                row[1] = xf;
-                row[2] = yf;
-            }
+            row[1] = xf;
+            row[2] = yf;
 #pragma unroll
             for (int d = 2; d <= M; ++d) {
                 const int cur = d * (d + 1) / 2, prev = (d - 1) * d / 2;
@@ -244,41 +352,89 @@ __global__ void __launch_bounds__(NT <= 32 ? 128 : 64) weights_refined_kernel(
                 for (int i = 0; i < d; ++i) row[cur + i] = xf * row[prev + i];
                 row[cur + d] = yf * row[prev + d - 1];
             }
-            for (int k = 0; k < S; ++k) {
-                // largest |entry| of the column (ties and the last six bits: lower thread)
-                const unsigned key =
-                    mine && pos < 0 ? ((__float_as_uint(row[0]) & 0x7fffffc0u) | (unsigned)(63 - t)) : 0u;
-                const unsigned best = ref_max<NT>(key, red, 2 + (k & 1));
-                ok = best >= __float_as_uint(kRefPivot) && best < 0x7f800000u;
-                if (!ok) break;
-                const bool piv = t == 63 - (int)(best & 63u);
+            float qmin = 4.f;  // smallest r^2 seen
+            int other = mine ? t : 0;  // pair u: nodes t and t + u + 1 (cyclic)
+            if constexpr (NT <= 32) ref_sync<NT>();
+            for (int k = 0; k < max(S, nh); ++k) {
+                const bool step = k < S, pair = k < nh && mine;
+                unsigned best = 0;
                 float* pr = prow + (k & 1) * PB;
-                if (piv) {
-                    pos = k;
-                    row[0] = __frcp_rn(row[0]);
+                // largest |entry| of the column (ties and the last six bits: lower thread)
+                if (step) {
+                    const unsigned key =
+                        mine && pos < 0 ? ((__float_as_uint(row[0]) & 0x7fffffc0u) | (unsigned)(63 - t)) : 0u;
+                    best = __reduce_max_sync(ref_mask<NT>(), key);
+                    if constexpr (NT > 32)
+                        if ((t & 31) == 0) red[4 + (k & 1) * 2 + (t >> 5)] = best;
+                }
+                int64_t qi = 0;
+                float qf = 1.f, ry = 1.f;
+                if (pair) {
+                    other = other + 1 < n ? other + 1 : 0;
+                    const longlong2 o = RB_AT(cxy, other, n);
+                    const float2 of = RB_AT(cxf, other, n);
+                    qi = fx_r2(me.x - o.x, me.y - o.y);
+                    const float fx = xf - of.x, fy = yf - of.y;
+                    qf = fmaf(fx, fx, fy * fy);
+                    qmin = fminf(qmin, qf);
+                    ry = rsqf(qf);
+                }
+                bool piv = false;
+                if (step) {
+                    if constexpr (NT > 32) {
+                        __syncthreads();
+                        best = max(red[4 + (k & 1) * 2], red[5 + (k & 1) * 2]);
+                    }
+                    ok = best >= __float_as_uint(kRefPivot) && best < 0x7f800000u;
+                    if (!ok) break;
+                    piv = t == 63 - (int)(best & 63u);
+                    if (piv) {
+                        pos = k;
+                        row[0] = rcpf(row[0]);
+#pragma unroll
+                        for (int j = 0; j < S4; ++j) {
+                            float4 v;
+                            v.x = row[4 * j];
+                            v.y = 4 * j + 1 < S ? row[4 * j + 1 < S ? 4 * j + 1 : 0] : 0.f;
+                            v.z = 4 * j + 2 < S ? row[4 * j + 2 < S ? 4 * j + 2 : 0] : 0.f;
+                            v.w = 4 * j + 3 < S ? row[4 * j + 3 < S ? 4 * j + 3 : 0] : 0.f;
+                            reinterpret_cast<float4*>(pr)[j] = v;
+                        }
+#pragma unroll
+                        for (int j = 1; j < S; ++j) row[j] = 0.f;
+                    }
+                }
+                if (pair) {
+                    const Digits v = fx_digits(fx_cube(qi, fx_sqrt(qi, qf, ry)));
+                    RB_AT(phi, k * n + t, nh * n) = make_int2(v.hi, v.lo);
+                }
+                if (step) {
+                    ref_sync<NT>();
+                    const float4 v0 = reinterpret_cast<const float4*>(pr)[0];
+                    const float f = piv ? v0.x : row[0] * v0.x;
 #pragma unroll
                     for (int j = 0; j < S4; ++j) {
-                        float4 v;
-                        v.x = row[4 * j];
-                        v.y = 4 * j + 1 < S ? row[4 * j + 1 < S ? 4 * j + 1 : 0] : 0.f;
-                        v.z = 4 * j + 2 < S ? row[4 * j + 2 < S ? 4 * j + 2 : 0] : 0.f;
-                        v.w = 4 * j + 3 < S ? row[4 * j + 3 < S ? 4 * j + 3 : 0] : 0.f;
-                        reinterpret_cast<float4*>(pr)[j] = v;
+                        const float4 v = j ? reinterpret_cast<const float4*>(pr)[j] : v0;
+                        if (j > 0) row[4 * j - 1] = fmaf(-f, v.x, row[4 * j]);
+                        if (4 * j + 1 < S) row[4 * j] = fmaf(-f, v.y, row[4 * j + 1 < S ? 4 * j + 1 : 0]);
+                        if (4 * j + 2 < S) row[4 * j + 1 < S ? 4 * j + 1 : 0] = fmaf(-f, v.z, row[4 * j + 2 < S ? 4 * j + 2 : 0]);
+                        if (4 * j + 3 < S) row[4 * j + 2 < S ? 4 * j + 2 : 0] = fmaf(-f, v.w, row[4 * j + 3 < S ? 4 * j + 3 : 0]);
                     }
-#pragma unroll
-                    for (int j = 1; j < S; ++j) row[j] = 0.f;
+                    row[S - 1] = f;
                 }
-                ref_sync<NT>();
-                const float f = piv ? row[0] : row[0] * pr[0];
-#pragma unroll
-                for (int j = 0; j < S4; ++j) {
-                    const float4 v = reinterpret_cast<const float4*>(pr)[j];
-                    if (j > 0) row[4 * j - 1] = fmaf(-f, v.x, row[4 * j]);
-                    if (4 * j + 1 < S) row[4 * j] = fmaf(-f, v.y, row[4 * j + 1 < S ? 4 * j + 1 : 0]);
-                    if (4 * j + 2 < S) row[4 * j + 1 < S ? 4 * j + 1 : 0] = fmaf(-f, v.z, row[4 * j + 2 < S ? 4 * j + 2 : 0]);
-                    if (4 * j + 3 < S) row[4 * j + 2 < S ? 4 * j + 2 : 0] = fmaf(-f, v.w, row[4 * j + 3 < S ? 4 * j + 3 : 0]);
+            }
+            // pairs closer than 2^-7 of the radius: again, from an exact r^2
+            bool close = false;
+            if (ok && mine && qmin < 0x1p-14f) {
+                for (int u = 0; u < nh; ++u) {
+                    const int k = t + u + 1 < n ? t + u + 1 : t + u + 1 - n;
+                    const longlong2 o = RB_AT(cxy, k, n);
+                    const int64_t qi = fx_r2(me.x - o.x, me.y - o.y);
+                    close |= qi < 16;
+                    const float qf = fmaxf((float)qi * 0x1p-58f, 0x1p-58f);
+                    const Digits v = fx_digits(fx_cube(qi, fx_sqrt(qi, qf, rsqf(qf))));
+                    phi[u * n + t] = make_int2(v.hi, v.lo);
                 }
-                row[S - 1] = f;
             }
             if (ok) {
                 // permuted position: pivots in pivot order, then the others in node order
@@ -291,7 +447,7 @@ __global__ void __launch_bounds__(NT <= 32 ? 128 : 64) weights_refined_kernel(
                 }
                 if (mine) {
                     if (pos < 0) pos = S + rank;
-                    RB_AT(posS, t, n) = pos;
+                    posS[t] = pos;
                     float* dst = pos < S ? &RB_AT(C, pos * LS, S * LS) : &RB_AT(X, (pos - S) * LS, q * LS);
 #pragma unroll
                     for (int j = 0; j < S4; ++j) {
@@ -302,54 +458,35 @@ __global__ void __launch_bounds__(NT <= 32 ? 128 : 64) weights_refined_kernel(
                         v.w = 4 * j + 3 < S ? row[4 * j + 3 < S ? 4 * j + 3 : 0] : 0.f;
                         reinterpret_cast<float4*>(dst)[j] = v;
                     }
-                    // zero diagonal and padding of this row's block
-                    if (pos < S) {
-                        A11[pos * LS + pos] = 0.f;
-                        for (int j = S; j < 4 * S4; ++j) A11[pos * LS + j] = 0.f;
-                    } else {
-                        Sm[(pos - S) * LQ + pos - S] = 0.f;
-                        for (int j = S; j < 4 * S4; ++j) Tt[(pos - S) * LS + j] = Wt[(pos - S) * LS + j] = 0.f;
+                    // zero diagonal and padding of this row's blocks
+                    if (pos < S) F1[pos * LS + pos] = 0.f;
+                    else Sm[(pos - S) * LQ + pos - S] = 0.f;
+                    for (int j = S; j < 4 * S4; ++j) {
+                        F1[pos * LS + j] = 0.f;
+                        if (pos >= S) Wt[(pos - S) * LS + j] = 0.f;
                     }
+                }
+            }
+            ok = ref_max<NT>(close || !ok ? 1u : 0u, red, 0) == 0u;
+            if constexpr (NT <= 32) ref_sync<NT>();
+
+            // ---- the float32 blocks of Phi from the leading digits ------------------
+            if (ok && mine) {
+                const int smo = (int)(Sm - F1);
+#pragma unroll 4
+                for (int u = 0; u < nh; ++u) {
+                    const int k = t + u + 1 < n ? t + u + 1 : t + u + 1 - n;
+                    const float pf = (float)phi[u * n + t].x * 0x1p-24f;
+                    const int b = RB_AT(posS, k, n);
+                    const int lo = min(pos, b), hi = max(pos, b);
+                    // (hi, lo), and its mirror in Phi11 and Phi22
+                    const int o1 = lo < S ? hi * LS + lo : smo + (hi - S) * LQ + lo - S;
+                    const int o2 = hi < S ? lo * LS + hi : (lo < S ? o1 : smo + (lo - S) * LQ + hi - S);
+                    RB_AT(F1, o1, smo + q * LQ) = pf;
+                    RB_AT(F1, o2, smo + q * LQ) = pf;
                 }
             }
             ref_sync<NT>();
-
-            // ---- kernel values: fixed point for the residual, float32 blocks ----
-            bool close = false;  // two nodes closer than 2^-27 of the radius
-            if (ok && mine) {
-                const longlong2 me = cxy[t];
-                int k = t;
-#pragma unroll 2
-                for (int u = 0; u < nh; ++u) {
-                    k = k + 1 < n ? k + 1 : 0;
-                    const longlong2 o = RB_AT(cxy, k, n);
-                    const float2 of = RB_AT(cxf, k, n);
-                    const int64_t qi = fx_r2(me.x - o.x, me.y - o.y);
-                    const float fx = xf - of.x, fy = yf - of.y;
-                    float qf = fmaf(fx, fx, fy * fy);
-                    if (qf < 0x1p-14f) {
-                        close |= qi < 16;
-                        qf = fmaxf((float)qi * 0x1p-58f, 0x1p-58f);
-                    }
-                    const float ry = rsqrtf(qf);
-                    const Digits v = fx_digits(fx_cube(qi, fx_sqrt(qi, qf, ry)));
-                    phi[u * n + t] = make_int2(v.hi, v.lo);
-                    const float pf = qf * (qf * ry);
-                    const int b = RB_AT(posS, k, n);
-                    const int lo = min(pos, b), hi = max(pos, b);
-                    if (hi < S) {
-                        RB_AT(A11, hi * LS + lo, S * LS) = pf;
-                        RB_AT(A11, lo * LS + hi, S * LS) = pf;
-                    } else if (lo < S) {
-                        RB_AT(Tt, (hi - S) * LS + lo, q * LS) = pf;
-                    } else {
-                        RB_AT(Sm, (hi - S) * LQ + lo - S, q * LQ) = pf;
-                        RB_AT(Sm, (lo - S) * LQ + hi - S, q * LQ) = pf;
-                    }
-                }
-            }
-            ok = ok && ref_max<NT>(close ? 1u : 0u, red, 0) == 0u;  // (a barrier for NT = 64)
-            if constexpr (NT <= 32) ref_sync<NT>();
 
             if (ok && q > 0) {
                 // ---- U^T = X Phi11; T^T = Phi21 - U^T, W^T = Phi21 - U^T / 2 ------
@@ -370,7 +507,7 @@ __global__ void __launch_bounds__(NT <= 32 ? 128 : 64) weights_refined_kernel(
                             xr[i] = reinterpret_cast<const float4*>(X + min(j0 + i, q - 1) * LS)[k];
 #pragma unroll
                         for (int a = 0; a < CT; ++a)
-                            ar[a] = reinterpret_cast<const float4*>(A11 + min(a0 + a, S - 1) * LS)[k];
+                            ar[a] = reinterpret_cast<const float4*>(F1 + min(a0 + a, S - 1) * LS)[k];
 #pragma unroll
                         for (int i = 0; i < RT; ++i)
 #pragma unroll
@@ -429,71 +566,21 @@ __global__ void __launch_bounds__(NT <= 32 ? 128 : 64) weights_refined_kernel(
                             }
                 }
                 ref_sync<NT>();
-                // ---- S^-1, in place, S positive definite: no pivoting --------------
-                // (the pivot row carries -1 one column past its end, which puts
-                // the multiplier into the column that the rotation frees)
-                float r[QM];
-#pragma unroll
-                for (int j = 0; j < QM / 4; ++j) {
-                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (4 * j < q && t < q) {
-                        v = reinterpret_cast<const float4*>(Sm + t * LQ)[j];
-                        if (4 * j + 1 >= q) v.y = 0.f;
-                        if (4 * j + 2 >= q) v.z = 0.f;
-                        if (4 * j + 3 >= q) v.w = 0.f;
-                    }
-                    r[4 * j] = v.x;
-                    r[4 * j + 1] = v.y;
-                    r[4 * j + 2] = v.z;
-                    r[4 * j + 3] = v.w;
+                // ---- S^-1, by one warp where its rows fit one ------------------------
+                if constexpr (NT > 32) {
+                    bool pos_def = true;
+                    if (q > 32) pos_def = ref_invert_any<NT, QMAX>(Sm, q, LQ, t, prow, PB);
+                    else if (t < 32) pos_def = ref_invert_any<32, (QMAX < 9 ? QMAX : 9)>(Sm, q, LQ, t, prow, PB);
+                    if (t == 0) red[9] = pos_def ? 1u : 0u;
+                } else {
+                    ok = ref_invert_any<NT, QMAX>(Sm, q, LQ, t, prow, PB);
                 }
-                for (int k = 0; k < q; ++k) {
-                    float* pr = prow + (k & 1) * PB;
-                    const bool piv = t == k;
-                    if (piv) {
-                        const float d = r[0];
-                        r[0] = d > 0.f ? __frcp_rn(d) : 0.f;
-#pragma unroll
-                        for (int j = 0; j < QM / 4; ++j)
-                            if (4 * j <= q) {
-                                float4 v = make_float4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
-                                if (4 * j == q) v.x = -1.f;
-                                if (4 * j + 1 == q) v.y = -1.f;
-                                if (4 * j + 2 == q) v.z = -1.f;
-                                if (4 * j + 3 == q) v.w = -1.f;
-                                reinterpret_cast<float4*>(pr)[j] = v;
-                            }
-#pragma unroll
-                        for (int j = 1; j < QM; ++j) r[j] = 0.f;
-                    }
-                    ref_sync<NT>();
-                    const float inv = pr[0];
-                    ok = inv > 0.f && inv < INFINITY;
-                    if (!ok) break;
-                    const float f = piv ? inv : r[0] * inv;
-#pragma unroll
-                    for (int j = 0; j < QM / 4; ++j)
-                        if (4 * j <= q) {
-                            const float4 v = reinterpret_cast<const float4*>(pr)[j];
-                            if (j > 0) r[4 * j - 1] = fmaf(-f, v.x, r[4 * j]);
-                            r[4 * j] = fmaf(-f, v.y, r[4 * j + 1]);
-                            r[4 * j + 1] = fmaf(-f, v.z, r[4 * j + 2]);
-                            r[4 * j + 2] = fmaf(-f, v.w, r[4 * j + 3]);
-                            r[4 * j + 3] = 0.f;
-                        }
-                }
-                if (ok && t < q) {
-#pragma unroll
-                    for (int j = 0; j < QM / 4; ++j)
-                        if (4 * j < q)
-                            reinterpret_cast<float4*>(Sm + t * LQ)[j] =
-                                make_float4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
-                }
+            } else if (NT > 32 && t == 0) {
+                red[9] = 1u;
             }
 
-            // ---- monomials in fixed point (W^T is no longer needed) ------------
+            // ---- monomials in fixed point (Phi11 and W^T are no longer needed) ---
             if (ok && mine) {
-                const longlong2 me = cxy[t];
                 const Digits xd = fx_digits(me.x), yd = fx_digits(me.y);
                 int2* pr = pd + t * LP;
                 Digits up[M + 1];  // the previous degree's digits
@@ -513,24 +600,24 @@ __global__ void __launch_bounds__(NT <= 32 ? 128 : 64) weights_refined_kernel(
             }
 
             // ---- solve and refine ------------------------------------------------
-            const float frhs = 9.0f * ((float)sown * 0x1p-60f);
             const float grhs = (M >= 2 && (t == 3 || t == 5)) ? 2.0f : 0.0f;
-            float rf = frhs, rg = grhs;  // current residual, float32
-            int64_t ri = 0, rgi = 0;     // and in units of 2^(e - 64)
-            int64_t wi = 0;              // weight in units of 2^(e0 - 62)
-            int e0 = 0, eprev = 0;
+            float rf = 9.0f * ((float)sown * 0x1p-60f);  // current residual, float32
+            float rg = grhs;
+            int64_t ri = 0, rgi = 0;                     // and in units of 2^(e0 - 60)
+            int64_t wi = 0;                              // weight in units of 2^(e0 - 62)
+            int e0 = 0;
             float mprev = 0.f, mw0 = 0.f;
             bool bad = false;
             if (t < 4 * S4) {
                 vr1[t] = 0.f;
                 vg[t] = 0.f;
                 vd0[t] = 0.f;
-                vh[t] = 0.f;
             }
             if (t < 4 * q4) vr2[t] = vt[t] = 0.f;
             ref_sync<NT>();
+            if constexpr (NT > 32) ok = ok && red[9] != 0u;
             for (int it = 0; ok; ++it) {
-                // float32 correction (d, dl) of the residual (rf, rg)
+                // float32 correction d of the residual (rf, rg)
                 if (mine) {
                     if (pos < S) RB_AT(vr1, pos, S) = rf;
                     else RB_AT(vr2, pos - S, q) = rf;
@@ -539,10 +626,10 @@ __global__ void __launch_bounds__(NT <= 32 ? 128 : 64) weights_refined_kernel(
                 ref_sync<NT>();
                 const int i2 = NT - 1 - t;  // row of X, T^T and S^-1 (other threads than t < S where NT allows)
                 float a1 = 0.f, d0 = 0.f;
-                if (i2 < q) a1 = RB_AT(vr2, i2, q) - dotv(X + i2 * LS, vr1, S4);
+                if (i2 < q) a1 = vr2[i2] - dotv(X + i2 * LS, vr1, S4);
                 if (t < S) {
                     float s0 = 0.f, s1 = 0.f;
-#pragma unroll 4
+#pragma unroll
                     for (int k = 0; k + 1 < S; k += 2) {
                         s0 = fmaf(C[k * LS + t], vg[k], s0);
                         s1 = fmaf(C[(k + 1) * LS + t], vg[k + 1], s1);
@@ -554,150 +641,149 @@ __global__ void __launch_bounds__(NT <= 32 ? 128 : 64) weights_refined_kernel(
                 ref_sync<NT>();
                 if (i2 < q) vt[i2] = a1 - dotv(Tt + i2 * LS, vd0, S4);
                 ref_sync<NT>();
-                float yi = 0.f;
-                if (i2 < q) yi = dotv(Sm + i2 * LQ, vt, q4);
-                ref_sync<NT>();
                 if (i2 < q) {
-                    vy[i2] = yi;
-                    vdw[S + i2] = yi;
+                    const float y = dotv(Sm + i2 * LQ, vt, q4);
+                    vy[i2] = y;
+                    vdw[S + i2] = y;
                 }
                 ref_sync<NT>();
                 if (t < S) {
                     float s0 = 0.f, s1 = 0.f;
+                    int j = 0;
 #pragma unroll 4
-                    for (int j = 0; j < q; ++j) {
-                        const float y = vy[j];
-                        s0 = fmaf(X[j * LS + t], y, s0);
-                        s1 = fmaf(Tt[j * LS + t], y, s1);
+                    for (; j + 1 < q; j += 2) {
+                        s0 = fmaf(X[j * LS + t], vy[j], s0);
+                        s1 = fmaf(X[(j + 1) * LS + t], vy[j + 1], s1);
                     }
-                    vdw[t] = d0 - s0;
-                    vh[t] = vr1[t] - dotv(A11 + t * LS, vd0, S4) - s1;
+                    if (j < q) s0 = fmaf(X[j * LS + t], vy[j], s0);
+                    vdw[t] = d0 - (s0 + s1);
                 }
                 ref_sync<NT>();
                 const float dj = mine ? RB_AT(vdw, pos, n) : 0.f;
-                const float dl = t < S ? dotv(C + (t < S ? t : 0) * LS, vh, S4) : 0.f;
 
                 // size of the correction, its rate of decrease
-                const unsigned inf = 0x7f800000u;
-                const unsigned uw = ref_max<NT>(bad ? inf : __float_as_uint(fabsf(dj)), red, 0);
-                const unsigned ul = ref_max<NT>(__float_as_uint(fabsf(dl)), red, 1);
-                const unsigned um = max(uw, ul);
+                const unsigned um = ref_max<NT>(bad ? 0x7f800000u : __float_as_uint(fabsf(dj)), red, it & 1);
                 if (um == 0u && it > 0) break;  // the residual is zero
-                const float m = __uint_as_float(um), mw = __uint_as_float(uw);
+                const float m = __uint_as_float(um);
                 const int e = (int)(um >> 23) - 126;  // 2^e > m
-                if (um >= inf || e < -100 || e > 60) {  // not finite, a failed check, or out of scale
+                if (um >= 0x7f800000u || e < -100 || e > 60) {  // not finite, a failed check, or out of scale
                     ok = false;
                     break;
                 }
                 if (it == 0) {
                     e0 = e;
-                    mw0 = mw;
-                    ok = mw * 256.0f >= m;  // w must keep its bits in the common scale
-                    if (!ok) break;
+                    mw0 = m;
                 }
                 const bool slow = it > 0 && !(m < kRefRate * mprev);
-                const bool done = it > 0 && mw * (m / mprev) <= kRefDone * mw0;
-                if (slow && !done) {
+                const bool done = it > 0 && m * (m / mprev) <= ref_done<M>(n, S) * mw0;
+                if ((slow && !done) || (!done && it + 1 >= kRefMaxSolves)) {
                     ok = false;
                     break;
                 }
+                mprev = m;
                 // the correction in units of 2^(e - 25); the sum takes the same integers
-                const float sc = fx_pow2f(25 - e);
-                const int di = fx_round(dj * sc);
+                const int di = fx_round(dj * fx_pow2f(25 - e));
                 const int sh = 37 - (e0 - e);
                 wi += sh >= 0 ? (int64_t)((uint64_t)(int64_t)di << (sh & 63)) : ((int64_t)di >> min(-sh, 31));
                 if (done) break;
-                if (it + 1 >= kRefMaxSolves) {
-                    ok = false;
-                    break;
-                }
                 if (mine) {
                     dI[t] = di;
                     dI[t + n] = di;
                 }
-                if (t < S) lI[t] = fx_round(dl * sc);
                 ref_sync<NT>();
 
-                // residual: r -= Phi d + P dl, rg -= P^T d, exact digit sums of
-                // unit 2^(e - 49) (hi) and 2^(e - 81) (lo)
-                const int up = it ? eprev - e : 0;
+                // residual: r -= Phi d, rg -= P^T d, exact sums of the digits'
+                // products, of unit 2^(e - 49) (H) and 2^(e - 81) (L).  The 64-bit
+                // wrap of r is harmless while the true residual is below 2^(e0 + 2)
+                const float hs = fx_pow2f(e - 49);
+                float check = rf;
                 if (mine) {
                     int64_t H = 0, L = 0;
-                    int k = t;  // node t - u - 1 (cyclic)
                     const int full = (n & 1) ? nh : nh - 1;
+                    const int2* pa = phi + t;                   // pair (t, t + u + 1)
+                    const int2* pb = phi + t - 1;               // pair (t - u - 1, t)
+                    const int* da = dI + t + 1;
+                    const int* db = dI + t + n - 1;
 #pragma unroll 4
                     for (int u = 0; u < full; ++u) {
-                        k = k > 0 ? k - 1 : n - 1;
-                        const int2 a = phi[u * n + t], b = RB_AT(phi, u * n + k, nh * n);
-                        const int da = dI[t + u + 1], db = RB_AT(dI, k, n);
-                        H += fx_mul32(a.x, da) + fx_mul32(b.x, db);
-                        L += fx_mul32(a.y, da) + fx_mul32(b.y, db);
+                        const int2 a = *pa, b = RB_PT(pb + (t <= u ? n : 0), phi, nh * n);
+                        const int va = RB_PT(da, dI, 2 * n), vb = RB_PT(db, dI, 2 * n);
+                        H += fx_mul32(a.x, va) + fx_mul32(b.x, vb);
+                        L += fx_mul32(a.y, va) + fx_mul32(b.y, vb);
+                        pa += n;
+                        pb += n - 1;
+                        ++da;
+                        --db;
                     }
                     if (full < nh) {  // n even: the opposite node, once
-                        const int2 a = phi[full * n + t];
-                        const int da = dI[t + nh];
-                        H += fx_mul32(a.x, da);
-                        L += fx_mul32(a.y, da);
+                        const int2 a = *pa;
+                        H += fx_mul32(a.x, *da);
+                        L += fx_mul32(a.y, *da);
                     }
+                    if (it == 0)  // 9 |xh|: 2^-60 to 2^(e0 - 60)
+                        ri = (int64_t)(e0 >= 0 ? 9ull * (uint64_t)sown >> min(e0, 63) : 9ull * (uint64_t)sown << min(-e0, 63));
+                    ri = (int64_t)((uint64_t)ri - fx_scale(H, L, 11 - (e0 - e)));
+                    check -= (float)H * hs;
+                    // (rounded through the check's magnitude until P l is subtracted)
+                    if (pos < S) RB_AT(vr1, pos, S) = it == 0 ? check : (float)ri * fx_pow2f(e0 - 60);
+                }
+                // rg: two threads per monomial where there are enough
+                constexpr int HS = NT / 2 >= S ? 2 : 1;
+                int64_t GH = 0, GL = 0;
+                const int kc = HS == 2 ? t % (NT / 2) : t;
+                if (kc < S) {
+#pragma unroll 4
+                    for (int j = HS == 2 ? t / (NT / 2) : 0; j < n; j += HS) {
+                        const int2 a = pd[j * LP + kc];
+                        const int d = dI[j];
+                        GH += fx_mul32(a.x, d);
+                        GL += fx_mul32(a.y, d);
+                    }
+                    if (HS == 2 && t >= NT / 2) part[kc] = make_longlong2(GH, GL);
+                }
+                ref_sync<NT>();
+                // correction of l from the residual of the pivot rows, and its scale
+                float dl = 0.f;
+                if (t < S) {
+                    dl = dotv(C + t * LS, vr1, S4);
+                    if (HS == 2) {
+                        GH += part[t].x;
+                        GL += part[t].y;
+                    }
+                    if (it == 0) rgi = grhs != 0.f && 61 - e0 < 64 ? (int64_t)(1ull << (61 - e0)) : 0;
+                    rgi = (int64_t)((uint64_t)rgi - fx_scale(GH, GL, 11 - (e0 - e)));
+                    bad |= !(fabsf(rg - (float)GH * hs) < fx_pow2f(e0));
+                    rg = (float)rgi * fx_pow2f(e0 - 60);
+                }
+                const unsigned ul = ref_max<NT>(__float_as_uint(fabsf(dl)), red, 2 + (it & 1));
+                const int el = max((int)(ul >> 23) - 126, -100);
+                if (ul >= 0x7f800000u || el > e0 + 12) {  // (e0 + 12: l in the range of the sums)
+                    ok = false;
+                    break;
+                }
+                if (t < S) lI[t] = fx_round(dl * fx_pow2f(25 - el));
+                ref_sync<NT>();
+                if (mine) {
+                    int64_t H = 0, L = 0;
                     const int2* pr = pd + t * LP;
-#pragma unroll 7
+#pragma unroll
                     for (int kk = 0; kk < S; ++kk) {
                         const int2 a = pr[kk];
                         const int d = lI[kk];
                         H += fx_mul32(a.x, d);
                         L += fx_mul32(a.y, d);
                     }
-                    if (it == 0) {  // 9 |xh|: 2^-60 to 2^(e - 64)
-                        const int s = e - 4;
-                        ri = (int64_t)(9ull * (s >= 0 ? (uint64_t)(sown >> min(s, 62)) : (uint64_t)sown << min(-s, 63)));
-                    } else {
-                        ri = up < 64 ? (int64_t)((uint64_t)ri << up) : 0;
-                    }
-                    ri = (int64_t)((uint64_t)ri - ((uint64_t)H << 15) - (uint64_t)(L >> 17));
-                    // the 64-bit wrap is harmless while the true residual is below 2^(e - 1)
-                    bad |= !(fabsf(rf - (float)H * fx_pow2f(e - 49)) < fx_pow2f(e - 2));
-                    rf = (float)ri * fx_pow2f(e - 64);
+                    ri = (int64_t)((uint64_t)ri - fx_scale(H, L, 11 - (e0 - el)));
+                    check -= (float)H * fx_pow2f(el - 49);
+                    bad |= !(fabsf(check) < fx_pow2f(e0));
+                    rf = (float)ri * fx_pow2f(e0 - 60);
                 }
-                // rg: two threads per monomial where there are enough
-                constexpr int HS = NT / 2 >= S ? 2 : 1;
-                int64_t H = 0, L = 0;
-                const int kc = HS == 2 ? t % (NT / 2) : t;
-                if (kc < S) {
-                    const int j0 = HS == 2 ? t / (NT / 2) : 0;
-#pragma unroll 4
-                    for (int j = j0; j < n; j += HS) {
-                        const int2 a = pd[j * LP + kc];
-                        const int d = dI[j];
-                        H += fx_mul32(a.x, d);
-                        L += fx_mul32(a.y, d);
-                    }
-                    if (HS == 2 && t >= NT / 2) part[kc] = make_longlong2(H, L);
-                }
-                if (HS == 2) ref_sync<NT>();
-                if (t < S) {
-                    if (HS == 2) {
-                        H += part[t].x;
-                        L += part[t].y;
-                    }
-                    if (it == 0) {
-                        const int s = 65 - e;  // 2 in units of 2^(e - 64)
-                        rgi = grhs != 0.f && s < 64 ? (int64_t)(1ull << s) : 0;
-                    } else {
-                        rgi = up < 64 ? (int64_t)((uint64_t)rgi << up) : 0;
-                    }
-                    rgi = (int64_t)((uint64_t)rgi - ((uint64_t)H << 15) - (uint64_t)(L >> 17));
-                    bad |= !(fabsf(rg - (float)H * fx_pow2f(e - 49)) < fx_pow2f(e - 2));
-                    rg = (float)rgi * fx_pow2f(e - 64);
-                }
-                eprev = e;
-                mprev = m;
-                ref_sync<NT>();
             }
 
             // ---- scale back (FP64) and store --------------------------------------
             if (ok) {
                 const double v = __dmul_rn((double)wi, __dmul_rn(inv_delta2, __hiloint2double((e0 - 62 + 1023) << 20, 0)));
-                ok = ref_max<NT>(mine && !finite64(v) ? 1u : 0u, red, 0) == 0u;
+                ok = ref_max<NT>(mine && !finite64(v) ? 1u : 0u, red, 4) == 0u;
                 if (ok && mine) w[(int64_t)node * n + t] = v;
                 if (ok && node_status && t == 0) node_status[node] = 0;
             }
