@@ -97,30 +97,55 @@ __device__ __forceinline__ double* part_at(double* part, int slot, int q) {
     return part + ((size_t)slot * kQ + q) * kMaxBlocks;
 }
 
+// Sums of NQ values over the block, in thread 0; two barriers in all (one
+// reduction at a time cost three each, most of a small launch's time).
+template <int NQ>
+__device__ __forceinline__ void block_sums(double (&v)[NQ], double (*sh)[kThreads / 32]) {
+    constexpr int W = kThreads / 32;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+    __syncthreads();
+    if (lane == 0)
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) RB_AT(sh[q], wid, W) = v[q];
+    __syncthreads();
+    if (wid == 0) {
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) v[q] = lane < W ? RB_AT(sh[q], lane, W) : 0.0;
+#pragma unroll
+        for (int o = W / 2; o > 0; o >>= 1)
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+    }
+}
+
 // Block-reduce NQ values, store block partials, and let the last block to
-// arrive sum all partials in block order (returned in tot[]).  True there.
+// arrive sum all partials in block order (tot[], in its thread 0).  True in
+// that block.
 template <int NQ>
 __device__ bool reduce_last(double (&v)[NQ], double* part, int slot, unsigned int* counter, double (&tot)[NQ]) {
-    __shared__ double sh[32];
+    __shared__ double sh[NQ][kThreads / 32];
     __shared__ unsigned int is_last;
+    block_sums<NQ>(v, sh);
+    if (threadIdx.x == 0) {
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        const double bs = block_sum<kThreads>(v[q], sh);
-        if (threadIdx.x == 0) RB_AT(part_at(part, slot, q), blockIdx.x, kMaxBlocks) = bs;
+        for (int q = 0; q < NQ; ++q) RB_AT(part_at(part, slot, q), blockIdx.x, kMaxBlocks) = v[q];
+        __threadfence();
+        is_last = (atomicAdd(counter, 1u) == gridDim.x - 1) ? 1u : 0u;
     }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) is_last = (atomicAdd(counter, 1u) == gridDim.x - 1) ? 1u : 0u;
     __syncthreads();
     if (!is_last) return false;
     __threadfence();
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        double acc = 0.0;
-        const double* pq = part_at(part, slot, q);
-        for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) acc += __ldcg(pq + b);
-        tot[q] = block_sum<kThreads>(acc, sh);
+    for (int q = 0; q < NQ; ++q) tot[q] = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) tot[q] += __ldcg(part_at(part, slot, q) + b);
     }
+    block_sums<NQ>(tot, sh);
     if (threadIdx.x == 0) *counter = 0u;
     return true;
 }
@@ -788,26 +813,34 @@ int tpr32_for(int64_t N, int64_t nnz) {
     return 2;
 }
 
-// Grid of a persistent-style launch: every block resident at once (blocks
-// per SM from the occupancy calculator, cached per kernel), capped at the
-// partial-sum capacity.  Reductions finish in the last block of the grid, so
-// each launch may use its own grid size.
+// Grid of a persistent-style launch over `work` threads of work: every block
+// resident at once (blocks per SM from the occupancy calculator, cached per
+// kernel), capped at the partial-sum capacity and at the blocks the work
+// fills: each block costs an atomic and a partial sum that the last block
+// adds up (10k rows: 16 us per reduction with the full grid of ~1,200 blocks
+// and 4 us with the 40 to 80 that have work).  Reductions finish in the last
+// block of the grid, so each launch may use its own grid size.
 template <class K>
-int grid_of(K kernel) {
+int grid_of(K kernel, int64_t work) {
     static std::mutex mu;
     static std::unordered_map<const void*, int> cache;
     const void* key = reinterpret_cast<const void*>(kernel);
-    std::lock_guard<std::mutex> lk(mu);
-    auto it = cache.find(key);
-    if (it != cache.end()) return it->second;
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, 0) != cudaSuccess || per_sm < 1)
-        per_sm = 4;
-    const int g = std::min(kMaxBlocks, per_sm * sm_count());
-    cache[key] = g;
-    return g;
+    int g = 0;
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        auto it = cache.find(key);
+        if (it != cache.end()) g = it->second;
+    }
+    if (g == 0) {
+        int per_sm = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, 0) != cudaSuccess || per_sm < 1)
+            per_sm = 4;
+        g = std::min(kMaxBlocks, per_sm * sm_count());
+        std::lock_guard<std::mutex> lk(mu);
+        cache[key] = g;
+    }
+    return (int)std::max<int64_t>(1, std::min<int64_t>(g, (work + kThreads - 1) / kThreads));
 }
-
 
 int64_t spmv_bytes(const rbffd_csr& A, int val_bytes) {
     return A.nnz * (int64_t)(val_bytes + 4) + 8 * (A.n_rows + 1) + 4 * 8 * A.n_rows;
@@ -819,10 +852,10 @@ struct Ops64 {
                       double tol, int max_iter, double repl, unsigned long long seed, cudaStream_t st) {
         const double* val = static_cast<const double*>(A.val);
         if (mode == kInit)
-            resid64_kernel<TPR, kInit><<<grid_of(resid64_kernel<TPR, kInit>), kThreads, 0, st>>>(
+            resid64_kernel<TPR, kInit><<<grid_of(resid64_kernel<TPR, kInit>, A.n_rows * TPR), kThreads, 0, st>>>(
                 A.row_ptr, A.col, val, A.n_rows, b, x, w.dinv, r, w.rh, w.p, w.v, tol, max_iter, repl, seed, w.st, w.part);
         else
-            resid64_kernel<TPR, kCheck><<<grid_of(resid64_kernel<TPR, kCheck>), kThreads, 0, st>>>(
+            resid64_kernel<TPR, kCheck><<<grid_of(resid64_kernel<TPR, kCheck>, A.n_rows * TPR), kThreads, 0, st>>>(
                 A.row_ptr, A.col, val, A.n_rows, b, x, w.dinv, r, w.rh, w.p, w.v, tol, max_iter, repl, seed, w.st, w.part);
         note_launches(1);
     }
@@ -834,23 +867,23 @@ struct Ops64 {
         const double* val = static_cast<const double*>(A.val);
         const int64_t bytes = spmv_bytes(A, 8);
         const int* flag = reinterpret_cast<const int*>(reinterpret_cast<const char*>(w.st) + offsetof(KState, flag));
-        update_p64_kernel<<<grid_of(update_p64_kernel), kThreads, 0, st>>>(N, w.r, w.v, w.p, w.st);
+        update_p64_kernel<<<grid_of(update_p64_kernel, N), kThreads, 0, st>>>(N, w.r, w.v, w.p, w.st);
         int e = prof_begin(st);
-        spmv64_kernel<TPR, 2><<<grid_of(spmv64_kernel<TPR, 2>), kThreads, 0, st>>>(
+        spmv64_kernel<TPR, 2><<<grid_of(spmv64_kernel<TPR, 2>, N * TPR), kThreads, 0, st>>>(
             A.row_ptr, A.col, val, N, w.p, w.dinv, w.ph, nullptr, w.st, w.part, nullptr);
         prof_end(e, st, kProfSpmv64, bytes);
         ev.push_back(e);
         mg_apply_interior(w.mg, w.mg32, w.ph, w.v, flag, st, &ev);
-        dot64_kernel<0><<<grid_of(dot64_kernel<0>), kThreads, 0, st>>>(N, w.rh, w.v, w.st, w.part);
-        update_s64_kernel<<<grid_of(update_s64_kernel), kThreads, 0, st>>>(N, w.r, w.v, w.s, w.st);
+        dot64_kernel<0><<<grid_of(dot64_kernel<0>, N), kThreads, 0, st>>>(N, w.rh, w.v, w.st, w.part);
+        update_s64_kernel<<<grid_of(update_s64_kernel, N), kThreads, 0, st>>>(N, w.r, w.v, w.s, w.st);
         e = prof_begin(st);
-        spmv64_kernel<TPR, 2><<<grid_of(spmv64_kernel<TPR, 2>), kThreads, 0, st>>>(
+        spmv64_kernel<TPR, 2><<<grid_of(spmv64_kernel<TPR, 2>, N * TPR), kThreads, 0, st>>>(
             A.row_ptr, A.col, val, N, w.s, w.dinv, w.sh, nullptr, w.st, w.part, nullptr);
         prof_end(e, st, kProfSpmv64, bytes);
         ev.push_back(e);
         mg_apply_interior(w.mg, w.mg32, w.sh, w.t, flag, st, &ev);
-        dot64_kernel<1><<<grid_of(dot64_kernel<1>), kThreads, 0, st>>>(N, w.t, w.s, w.st, w.part);
-        update_xr64_kernel<<<grid_of(update_xr64_kernel), kThreads, 0, st>>>(N, x, w.p, w.s, w.t, w.r, w.rh, w.d,
+        dot64_kernel<1><<<grid_of(dot64_kernel<1>, N), kThreads, 0, st>>>(N, w.t, w.s, w.st, w.part);
+        update_xr64_kernel<<<grid_of(update_xr64_kernel, N), kThreads, 0, st>>>(N, x, w.p, w.s, w.t, w.r, w.rh, w.d,
                                                                              w.st, w.part, nullptr);
         note_launches(7);
     }
@@ -863,21 +896,21 @@ struct Ops64 {
         const int* flag = reinterpret_cast<const int*>(reinterpret_cast<const char*>(w.st) + offsetof(KState, flag));
         const double* pin = w.mg ? w.ph : w.p;
         const double* sin_ = w.mg ? w.sh : w.s;
-        update_p64_kernel<<<grid_of(update_p64_kernel), kThreads, 0, st>>>(N, w.r, w.v, w.p, w.st);
+        update_p64_kernel<<<grid_of(update_p64_kernel, N), kThreads, 0, st>>>(N, w.r, w.v, w.p, w.st);
         if (w.mg) mg_apply(w.mg, w.mg32, w.p, w.ph, flag, st, &ev);
         int e = prof_begin(st);
-        spmv64_kernel<TPR, 0><<<grid_of(spmv64_kernel<TPR, 0>), kThreads, 0, st>>>(
+        spmv64_kernel<TPR, 0><<<grid_of(spmv64_kernel<TPR, 0>, N * TPR), kThreads, 0, st>>>(
             A.row_ptr, A.col, val, N, pin, w.dinv, w.v, w.rh, w.st, w.part, nullptr);
         prof_end(e, st, kProfSpmv64, bytes);
         ev.push_back(e);
-        update_s64_kernel<<<grid_of(update_s64_kernel), kThreads, 0, st>>>(N, w.r, w.v, w.s, w.st);
+        update_s64_kernel<<<grid_of(update_s64_kernel, N), kThreads, 0, st>>>(N, w.r, w.v, w.s, w.st);
         if (w.mg) mg_apply(w.mg, w.mg32, w.s, w.sh, flag, st, &ev);
         e = prof_begin(st);
-        spmv64_kernel<TPR, 1><<<grid_of(spmv64_kernel<TPR, 1>), kThreads, 0, st>>>(
+        spmv64_kernel<TPR, 1><<<grid_of(spmv64_kernel<TPR, 1>, N * TPR), kThreads, 0, st>>>(
             A.row_ptr, A.col, val, N, sin_, w.dinv, w.t, nullptr, w.st, w.part, w.mg ? w.s : nullptr);
         prof_end(e, st, kProfSpmv64, bytes);
         ev.push_back(e);
-        update_xr64_kernel<<<grid_of(update_xr64_kernel), kThreads, 0, st>>>(N, x, pin, w.s, w.t, w.r, w.rh, w.d,
+        update_xr64_kernel<<<grid_of(update_xr64_kernel, N), kThreads, 0, st>>>(N, x, pin, w.s, w.t, w.r, w.rh, w.d,
                                                                              w.st, w.part, w.mg ? w.sh : nullptr);
         note_launches(5);
     }
@@ -891,19 +924,19 @@ struct OpsDf {
         // algorithmic bytes: nnz (4 + 4) + row_ptr + 8-byte df32 vectors
         // (gathered once, result, dot partner) + 4-byte sigma and scale
         const int64_t bytes = spmv_bytes(A32, 4);
-        update_p_df_kernel<<<grid_of(update_p_df_kernel), kThreads, 0, st>>>(N, w.rd, w.vd, w.pd, w.st);
+        update_p_df_kernel<<<grid_of(update_p_df_kernel, N), kThreads, 0, st>>>(N, w.rd, w.vd, w.pd, w.st);
         int e = prof_begin(st);
-        spmv_df_kernel<TPR, 0><<<grid_of(spmv_df_kernel<TPR, 0>), kThreads, 0, st>>>(
+        spmv_df_kernel<TPR, 0><<<grid_of(spmv_df_kernel<TPR, 0>, N * TPR), kThreads, 0, st>>>(
             A32.row_ptr, A32.col, val, N, w.pd, w.sigma32, w.dinv32, w.vd, w.rhd, w.st, w.part);
         prof_end(e, st, kProfSpmv32, bytes);
         ev.push_back(e);
-        update_s_df_kernel<<<grid_of(update_s_df_kernel), kThreads, 0, st>>>(N, w.rd, w.vd, w.sd, w.st);
+        update_s_df_kernel<<<grid_of(update_s_df_kernel, N), kThreads, 0, st>>>(N, w.rd, w.vd, w.sd, w.st);
         e = prof_begin(st);
-        spmv_df_kernel<TPR, 1><<<grid_of(spmv_df_kernel<TPR, 1>), kThreads, 0, st>>>(
+        spmv_df_kernel<TPR, 1><<<grid_of(spmv_df_kernel<TPR, 1>, N * TPR), kThreads, 0, st>>>(
             A32.row_ptr, A32.col, val, N, w.sd, w.sigma32, w.dinv32, w.td, nullptr, w.st, w.part);
         prof_end(e, st, kProfSpmv32, bytes);
         ev.push_back(e);
-        update_xr_df_kernel<<<grid_of(update_xr_df_kernel), kThreads, 0, st>>>(N, w.xd, w.pd, w.sd, w.td, w.rd,
+        update_xr_df_kernel<<<grid_of(update_xr_df_kernel, N), kThreads, 0, st>>>(N, w.xd, w.pd, w.sd, w.td, w.rd,
                                                                                w.rhd, w.d32, w.st, w.part);
         note_launches(5);
     }
@@ -1195,7 +1228,7 @@ int solve_fp64(const rbffd_csr& A, const double* b, double* x, const rbffd_solve
             const int* flag =
                 reinterpret_cast<const int*>(reinterpret_cast<const char*>(w.st) + offsetof(KState, flag));
             if ((rc = mg_apply_interior(w.mg, w.mg32, w.r, w.ph, flag, st)) != RBFFD_OK) return rc;
-            left_init_kernel<<<grid_of(left_init_kernel), kThreads, 0, st>>>(N, w.ph, w.r, w.rh,
+            left_init_kernel<<<grid_of(left_init_kernel, N), kThreads, 0, st>>>(N, w.ph, w.r, w.rh,
                                                                              shadow_seed(rnd, passes), w.st, w.part);
             note_launches(1);
             RBFFD_LAUNCH_CHECK();
@@ -1294,7 +1327,7 @@ int solve_mixed(const rbffd_csr& A, const rbffd_csr& A32, const double* b, doubl
         const double inner = std::min(std::max(o.inner_tol, 0.5 * o.tol / rel), 0.5);
         const int budget = std::min(o.max_iter - total, g.cap);
         const unsigned long long seed = shadow_seed(rnd, outer);
-        load_df_kernel<<<grid_of(load_df_kernel), kThreads, 0, st>>>(N, w.r64, w.dinv32, w.rd, w.rhd, w.pd, w.vd,
+        load_df_kernel<<<grid_of(load_df_kernel, N), kThreads, 0, st>>>(N, w.r64, w.dinv32, w.rd, w.rhd, w.pd, w.vd,
                                                                      w.xd, inner, budget, seed, w.st, w.part);
         note_launches(1);
         RBFFD_LAUNCH_CHECK();
@@ -1309,7 +1342,7 @@ int solve_mixed(const rbffd_csr& A, const rbffd_csr& A32, const double* b, doubl
                     hs.iter, hs.flag, std::sqrt(hs.rnorm2 / start2), rel);
         g.last_iters = hs.iter;
         RBFFD_CUDA_TRY(cudaMemcpyAsync(w.x_save, x, sizeof(double) * N, cudaMemcpyDeviceToDevice, st));
-        refine_kernel<<<grid_of(refine_kernel), kThreads, 0, st>>>(N, x, w.xd);
+        refine_kernel<<<grid_of(refine_kernel, N), kThreads, 0, st>>>(N, x, w.xd);
         note_launches(1);
         RBFFD_LAUNCH_CHECK();
         if (hs.flag == kBreakdown) {
