@@ -40,6 +40,7 @@
 // accuracy, the outer FP64 BiCGSTAB keeps the residual exact).
 #include "common.cuh"
 #include "internal.cuh"
+#include "mg_cluster.cuh"
 #include "scan.cuh"
 
 #include <cooperative_groups.h>
@@ -47,6 +48,8 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <map>
+#include <mutex>
 #include <vector>
 
 namespace rbffd {
@@ -1085,6 +1088,53 @@ void restrict_to(const MgLevel& L, int64_t nc, const T* r, T* bc, const int* fla
     }
 }
 
+// The levels [first, n_levels) by one cluster.  TOP: level 0 is among them,
+// its right-hand side and result are the caller's FP64 vectors.
+template <typename T, bool TOP>
+__global__ void __launch_bounds__(kClThreads) mg_cluster_kernel(const __grid_constant__ ClCycle<T> c,
+                                                                const double* __restrict__ b, double* __restrict__ x) {
+    if (stopped(c.flag)) return;
+    auto cluster = cooperative_groups::this_cluster();
+    const ClLevel<T>& L = c.lv[0];
+    if constexpr (TOP)
+        cl_cycle<T>(c, [&](int i) { return (T)__ldg(&RB_AT(b, i, L.n)); }, [&](int i, T v) { x[i] = (double)v; },
+                    [&] { cluster.sync(); });
+    else
+        cl_cycle<T>(c, [&](int i) { return __ldg(&RB_AT(L.b, i, L.n)); },
+                    [&](int i, T v) { (c.levels == 1 ? L.x : L.t)[i] = v; }, [&] { cluster.sync(); });
+}
+
+// Rows up to which a level belongs to the cluster: its operations cost the
+// cluster's 16 SMs about as long as a launch over the whole GPU.  (FP64: the
+// units' rate on 16 SMs is the limit, 12 multiply-adds per row.)
+template <typename T>
+constexpr int64_t cl_rows() {
+    return sizeof(T) == 8 ? 8192 : 32768;
+}
+
+// Launches the cluster V-cycle; false where it does not apply.
+template <typename T, bool TOP>
+bool cluster_cycle(const MgHierarchy& h, int first, const double* b, double* x, const int* flag, cudaStream_t st) {
+    const void* kern = reinterpret_cast<const void*>(mg_cluster_kernel<T, TOP>);
+    const int size = cl_cluster_size(kern);
+    ClCycle<T> c;
+    if (size == 0 || !cl_make<T>(h, first, flag, &c)) return false;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)size);
+    cfg.blockDim = dim3(kClThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)size;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, mg_cluster_kernel<T, TOP>, c, b, x) == cudaSuccess) return true;
+    (void)cudaGetLastError();  // the per-operation kernels run instead
+    return false;
+}
+
 // One level of the cycle: b (BT) in, result in x (OT) for level 0, in the
 // level's own current-iterate buffer otherwise (returned).
 template <typename T>
@@ -1095,6 +1145,16 @@ T* cycle_level(const MgHierarchy& h, int l, const void* bin, bool b_is_double, d
     const bool top = (l == 0);
     T* cur = Sel<T>::x(L);
     T* oth = Sel<T>::t(L);
+    // small levels: the rest of the cycle in one launch (not the top level
+    // while its sweeps are being timed)
+    if (L.N <= cl_rows<T>() && !(top && ev && profiling())) {
+        const bool done = top ? b_is_double && cluster_cycle<T, true>(h, l, static_cast<const double*>(bin), out, flag, st)
+                              : cluster_cycle<T, false>(h, l, nullptr, nullptr, flag, st);
+        if (done) {
+            ++*launches;
+            return last_level ? cur : oth;
+        }
+    }
     auto launch_first = [&](T* x) {
         const int g = blocks_for(L.N);
         if (b_is_double)
@@ -1161,6 +1221,71 @@ T* cycle_level(const MgHierarchy& h, int l, const void* bin, bool b_is_double, d
 }
 
 }  // namespace
+
+template <typename T>
+bool cl_make(const MgHierarchy& h, int first, const int* flag, ClCycle<T>* out) {
+    out->levels = h.n_levels - first;
+    if (first < 0 || out->levels < 1 || out->levels > kClMaxLevels) return false;
+    out->nu = h.nu;
+    out->flag = flag;
+    out->minv = Sel<T>::minv(h.lv[h.n_levels - 1]);
+    for (int l = first; l < h.n_levels; ++l) {
+        const MgLevel& L = h.lv[l];
+        if (L.N > 0x3fffffff) return false;
+        ClLevel<T>& c = out->lv[l - first];
+        const bool last = l == h.n_levels - 1;
+        c.n = (int)L.N;
+        c.tpr = L.tpr;
+        c.rtpr = last ? 1 : L.rtpr;
+        c.row_ptr = L.row_ptr;
+        c.col = L.col;
+        c.val = Sel<T>::val(L);
+        c.w = Sel<T>::dinv(L);
+        c.pidx = last ? nullptr : L.pidx;
+        c.pval = last ? nullptr : Sel<T>::pval(L);
+        c.rrow = last ? nullptr : L.rrow;
+        c.rcol = last ? nullptr : L.rcol;
+        c.rval = last ? nullptr : Sel<T>::rval(L);
+        c.x = Sel<T>::x(L);
+        c.t = Sel<T>::t(L);
+        c.r = Sel<T>::r(L);
+        c.b = Sel<T>::b(L);
+    }
+    return true;
+}
+template bool cl_make<float>(const MgHierarchy&, int, const int*, ClCycle<float>*);
+template bool cl_make<double>(const MgHierarchy&, int, const int*, ClCycle<double>*);
+
+int cl_cluster_size(const void* kernel) {
+    static std::mutex mu;
+    static std::map<std::pair<int, const void*>, int> cache;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    const auto key = std::make_pair(dev, kernel);
+    std::lock_guard<std::mutex> lk(mu);
+    auto it = cache.find(key);
+    if (it != cache.end()) return it->second;
+    int size = 0;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+        for (int s = 16; s >= 8 && size == 0; s /= 2) {
+            cudaLaunchConfig_t cfg{};
+            cfg.gridDim = dim3((unsigned)s);
+            cfg.blockDim = dim3(kClThreads);
+            cudaLaunchAttribute attr{};
+            attr.id = cudaLaunchAttributeClusterDimension;
+            attr.val.clusterDim.x = (unsigned)s;
+            attr.val.clusterDim.y = 1;
+            attr.val.clusterDim.z = 1;
+            cfg.attrs = &attr;
+            cfg.numAttrs = 1;
+            int clusters = 0;
+            if (cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess && clusters > 0) size = s;
+        }
+    }
+    (void)cudaGetLastError();  // a refused size is not the caller's error
+    cache[key] = size;
+    return size;
+}
 
 size_t mg_multi_coarse_floats(const MgHierarchy* h, int R) {
     if (!h) return 0;
