@@ -61,6 +61,32 @@ struct Carver {
 
 inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 
+// Programmatic dependent launch: with `chained`, the kernel may start while the
+// one before it in the stream still runs, and its pdl_wait() returns once that
+// one has completed.  Used in chains of short kernels (V-cycles, Krylov
+// iterations, explicit steps), where the launch and the loads that do not
+// depend on the chain (matrix rows, read before pdl_wait) otherwise cost more
+// than the work.  Rules, for the chain to stay ordered: every kernel of a
+// chain calls pdl_wait() in every thread before it touches anything the chain
+// writes and before it may return, and pdl_next() only after that (so at most
+// two kernels overlap); the first kernel of a chain is not `chained`, so what
+// is read before the wait was written by kernels that had completed.
+template <class... P, class... A>
+inline cudaError_t launch_chained(bool chained, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem,
+                                  cudaStream_t st, A&&... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = chained ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Number of SMs of the current device (cached per device).
 int sm_count();
 
@@ -83,6 +109,10 @@ void prof_commit(const int* slots, int count, int keep);
 void prof_commit_as(int slot, int count, int64_t bytes);
 
 // ---------------------------------------------------------------- device --
+// See launch_chained.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

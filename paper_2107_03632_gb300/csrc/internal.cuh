@@ -104,16 +104,18 @@ bool mg_is_galerkin(const MgHierarchy* h);
 // B on the residuals a forward solve started by mg_dirichlet_fix produces.
 // With A = [I 0; L_ib L_ii] (Dirichlet rows first) M A = diag(I, B_ii L_ii),
 // so the adjoint's preconditioned operator is block diagonal.
+// chained: the first kernel continues a chain of launch_chained kernels.
 int mg_apply(const MgHierarchy* h, bool fp32, const double* b, double* x, const int* flag, cudaStream_t st,
-             std::vector<int>* ev = nullptr);
+             std::vector<int>* ev = nullptr, bool chained = false);
 // x = Pi B b: the V-cycle alone, Dirichlet entries of the result zeroed
 // (Pi); with the adjoint hierarchy, on boundary-free b, B_ii^T b_i (the left
 // preconditioner of the adjoint's interior system).
 int mg_apply_interior(const MgHierarchy* h, bool fp32, const double* b, double* x, const int* flag, cudaStream_t st,
-                      std::vector<int>* ev = nullptr);
+                      std::vector<int>* ev = nullptr, bool chained = false);
 // y_b += W_b (r_b - (A y)_b) on the Dirichlet rows of level 0 (see
 // mg_bfix_kernel); one launch on st.
-int mg_dirichlet_fix(const MgHierarchy* h, const double* r, double* y, const int* flag, cudaStream_t st);
+int mg_dirichlet_fix(const MgHierarchy* h, const double* r, double* y, const int* flag, cudaStream_t st,
+                     bool chained = false);
 
 // rbffd_mg_setup for a fine operator given by arrays: row_ptr points at the
 // fine rows' first entry (values are offsets into col/val), and column

@@ -364,6 +364,8 @@ __global__ void __launch_bounds__(kThreads) resid64_kernel(const int64_t* __rest
 __global__ void __launch_bounds__(kThreads) update_p64_kernel(int64_t N, const double* __restrict__ r,
                                                               const double* __restrict__ v, double* __restrict__ p,
                                                               const KState* st) {
+    pdl_wait();
+    pdl_next();
     if (st->flag != kRunning) return;
     const double beta = (st->rho_new / st->rho) * (st->alpha / st->omega);
     const double omega = st->omega;
@@ -382,6 +384,8 @@ __global__ void __launch_bounds__(kThreads) spmv64_kernel(const int64_t* __restr
                                                           const double* __restrict__ dinv, double* __restrict__ y,
                                                           const double* __restrict__ rh, KState* st, double* part,
                                                           const double* __restrict__ dotv) {
+    pdl_wait();
+    pdl_next();
     if (st->flag != kRunning) return;
     const int sub = threadIdx.x & (TPR - 1);
     double acc[3] = {0.0, 0.0, 0.0};
@@ -417,6 +421,8 @@ __global__ void __launch_bounds__(kThreads) spmv64_kernel(const int64_t* __restr
 template <int MODE>
 __global__ void __launch_bounds__(kThreads) dot64_kernel(int64_t N, const double* __restrict__ a,
                                                          const double* __restrict__ b, KState* st, double* part) {
+    pdl_wait();
+    pdl_next();
     if (st->flag != kRunning) return;
     double acc[3] = {0.0, 0.0, 0.0};
     RBFFD_ELEM_LOOP(N, i) {
@@ -444,6 +450,8 @@ __global__ void __launch_bounds__(kThreads) dot64_kernel(int64_t N, const double
 __global__ void __launch_bounds__(kThreads) left_init_kernel(int64_t N, const double* __restrict__ mr,
                                                              double* __restrict__ r, double* __restrict__ rh,
                                                              unsigned long long seed, KState* st, double* part) {
+    pdl_wait();
+    pdl_next();
     if (st->flag != kRunning) return;
     double acc[2] = {0.0, 0.0};
     RBFFD_ELEM_LOOP(N, i) {
@@ -468,6 +476,8 @@ __global__ void __launch_bounds__(kThreads) left_init_kernel(int64_t N, const do
 __global__ void __launch_bounds__(kThreads) update_s64_kernel(int64_t N, const double* __restrict__ r,
                                                               const double* __restrict__ v, double* __restrict__ s,
                                                               const KState* st) {
+    pdl_wait();
+    pdl_next();
     if (st->flag != kRunning) return;
     const double alpha = st->alpha;
     RBFFD_ELEM_LOOP(N, i) s[i] = fma(-alpha, v[i], r[i]);
@@ -500,6 +510,8 @@ __global__ void __launch_bounds__(kThreads) update_xr64_kernel(int64_t N, double
                                                                const double* __restrict__ rh,
                                                                const double* __restrict__ d, KState* st,
                                                                double* part, const double* __restrict__ sx) {
+    pdl_wait();
+    pdl_next();
     if (st->flag != kRunning) return;
     const double alpha = st->alpha, omega = st->omega;
     double acc[3] = {0.0, 0.0, 0.0};
@@ -599,6 +611,8 @@ __global__ void __launch_bounds__(kThreads) load_df_kernel(int64_t N, const doub
 __global__ void __launch_bounds__(kThreads) update_p_df_kernel(int64_t N, const float2* __restrict__ r,
                                                                const float2* __restrict__ v,
                                                                float2* __restrict__ p, const KState* st) {
+    pdl_wait();
+    pdl_next();
     if (st->flag != kRunning) return;
     const df beta = df_from_double((st->rho_new / st->rho) * (st->alpha / st->omega));
     const df nomega = df_from_double(-st->omega);
@@ -619,6 +633,8 @@ __global__ void __launch_bounds__(kThreads) spmv_df_kernel(const int64_t* __rest
                                                            const float* __restrict__ dinv,
                                                            float2* __restrict__ y, const float2* __restrict__ rh,
                                                            KState* st, double* part) {
+    pdl_wait();
+    pdl_next();
     if (st->flag != kRunning) return;
     const int sub = threadIdx.x & (TPR - 1);
     DfAcc a0, a1, a2;
@@ -659,6 +675,8 @@ __global__ void __launch_bounds__(kThreads) spmv_df_kernel(const int64_t* __rest
 __global__ void __launch_bounds__(kThreads) update_s_df_kernel(int64_t N, const float2* __restrict__ r,
                                                                const float2* __restrict__ v,
                                                                float2* __restrict__ s, const KState* st) {
+    pdl_wait();
+    pdl_next();
     if (st->flag != kRunning) return;
     const df nalpha = df_from_double(-st->alpha);
     RBFFD_ELEM_LOOP(N, i) df_store(s + i, df_fma(nalpha, df_load(v + i), df_load(r + i)));
@@ -672,6 +690,8 @@ __global__ void __launch_bounds__(kThreads) update_xr_df_kernel(int64_t N, float
                                                                 const float2* __restrict__ rh,
                                                                 const float* __restrict__ d, KState* st,
                                                                 double* part) {
+    pdl_wait();
+    pdl_next();
     if (st->flag != kRunning) return;
     const df alpha = df_from_double(st->alpha), omega = df_from_double(st->omega);
     const df nomega = df_from_double(-st->omega);
@@ -862,33 +882,38 @@ struct Ops64 {
     // Left-preconditioned iteration on the interior unknowns (see
     // solve_fp64): v = Pi B^T (A p), t = Pi B^T (A s), x += alpha p + omega s.
     static void iteration_left(const rbffd_csr& A, double* x, const Work& w, cudaStream_t st,
-                               std::vector<int>& ev) {
+                               std::vector<int>& ev, bool chained) {
         const int64_t N = A.n_rows;
         const double* val = static_cast<const double*>(A.val);
         const int64_t bytes = spmv_bytes(A, 8);
         const int* flag = reinterpret_cast<const int*>(reinterpret_cast<const char*>(w.st) + offsetof(KState, flag));
-        update_p64_kernel<<<grid_of(update_p64_kernel, N), kThreads, 0, st>>>(N, w.r, w.v, w.p, w.st);
+        launch_chained(chained, update_p64_kernel, grid_of(update_p64_kernel, N), kThreads, 0, st, N, w.r, w.v, w.p,
+                       w.st);
         int e = prof_begin(st);
-        spmv64_kernel<TPR, 2><<<grid_of(spmv64_kernel<TPR, 2>, N * TPR), kThreads, 0, st>>>(
-            A.row_ptr, A.col, val, N, w.p, w.dinv, w.ph, nullptr, w.st, w.part, nullptr);
+        launch_chained(true, spmv64_kernel<TPR, 2>, grid_of(spmv64_kernel<TPR, 2>, N * TPR), kThreads, 0, st,
+                       A.row_ptr, A.col, val, N, w.p, w.dinv, w.ph, nullptr, w.st, w.part, nullptr);
         prof_end(e, st, kProfSpmv64, bytes);
         ev.push_back(e);
-        mg_apply_interior(w.mg, w.mg32, w.ph, w.v, flag, st, &ev);
-        dot64_kernel<0><<<grid_of(dot64_kernel<0>, N), kThreads, 0, st>>>(N, w.rh, w.v, w.st, w.part);
-        update_s64_kernel<<<grid_of(update_s64_kernel, N), kThreads, 0, st>>>(N, w.r, w.v, w.s, w.st);
+        mg_apply_interior(w.mg, w.mg32, w.ph, w.v, flag, st, &ev, true);
+        launch_chained(true, dot64_kernel<0>, grid_of(dot64_kernel<0>, N), kThreads, 0, st, N, w.rh, w.v, w.st,
+                       w.part);
+        launch_chained(true, update_s64_kernel, grid_of(update_s64_kernel, N), kThreads, 0, st, N, w.r, w.v, w.s,
+                       w.st);
         e = prof_begin(st);
-        spmv64_kernel<TPR, 2><<<grid_of(spmv64_kernel<TPR, 2>, N * TPR), kThreads, 0, st>>>(
-            A.row_ptr, A.col, val, N, w.s, w.dinv, w.sh, nullptr, w.st, w.part, nullptr);
+        launch_chained(true, spmv64_kernel<TPR, 2>, grid_of(spmv64_kernel<TPR, 2>, N * TPR), kThreads, 0, st,
+                       A.row_ptr, A.col, val, N, w.s, w.dinv, w.sh, nullptr, w.st, w.part, nullptr);
         prof_end(e, st, kProfSpmv64, bytes);
         ev.push_back(e);
-        mg_apply_interior(w.mg, w.mg32, w.sh, w.t, flag, st, &ev);
-        dot64_kernel<1><<<grid_of(dot64_kernel<1>, N), kThreads, 0, st>>>(N, w.t, w.s, w.st, w.part);
-        update_xr64_kernel<<<grid_of(update_xr64_kernel, N), kThreads, 0, st>>>(N, x, w.p, w.s, w.t, w.r, w.rh, w.d,
-                                                                             w.st, w.part, nullptr);
+        mg_apply_interior(w.mg, w.mg32, w.sh, w.t, flag, st, &ev, true);
+        launch_chained(true, dot64_kernel<1>, grid_of(dot64_kernel<1>, N), kThreads, 0, st, N, w.t, w.s, w.st,
+                       w.part);
+        launch_chained(true, update_xr64_kernel, grid_of(update_xr64_kernel, N), kThreads, 0, st, N, x, w.p, w.s,
+                       w.t, w.r, w.rh, w.d, w.st, w.part, nullptr);
         note_launches(7);
     }
-    static void iteration(const rbffd_csr& A, double* x, const Work& w, cudaStream_t st, std::vector<int>& ev) {
-        if (w.left) return iteration_left(A, x, w, st, ev);
+    static void iteration(const rbffd_csr& A, double* x, const Work& w, cudaStream_t st, std::vector<int>& ev,
+                          bool chained) {
+        if (w.left) return iteration_left(A, x, w, st, ev, chained);
         const int64_t N = A.n_rows;
         const double* val = static_cast<const double*>(A.val);
         const int64_t bytes = spmv_bytes(A, 8);
@@ -896,48 +921,52 @@ struct Ops64 {
         const int* flag = reinterpret_cast<const int*>(reinterpret_cast<const char*>(w.st) + offsetof(KState, flag));
         const double* pin = w.mg ? w.ph : w.p;
         const double* sin_ = w.mg ? w.sh : w.s;
-        update_p64_kernel<<<grid_of(update_p64_kernel, N), kThreads, 0, st>>>(N, w.r, w.v, w.p, w.st);
-        if (w.mg) mg_apply(w.mg, w.mg32, w.p, w.ph, flag, st, &ev);
+        launch_chained(chained, update_p64_kernel, grid_of(update_p64_kernel, N), kThreads, 0, st, N, w.r, w.v, w.p,
+                       w.st);
+        if (w.mg) mg_apply(w.mg, w.mg32, w.p, w.ph, flag, st, &ev, true);
         int e = prof_begin(st);
-        spmv64_kernel<TPR, 0><<<grid_of(spmv64_kernel<TPR, 0>, N * TPR), kThreads, 0, st>>>(
-            A.row_ptr, A.col, val, N, pin, w.dinv, w.v, w.rh, w.st, w.part, nullptr);
+        launch_chained(true, spmv64_kernel<TPR, 0>, grid_of(spmv64_kernel<TPR, 0>, N * TPR), kThreads, 0, st,
+                       A.row_ptr, A.col, val, N, pin, w.dinv, w.v, w.rh, w.st, w.part, nullptr);
         prof_end(e, st, kProfSpmv64, bytes);
         ev.push_back(e);
-        update_s64_kernel<<<grid_of(update_s64_kernel, N), kThreads, 0, st>>>(N, w.r, w.v, w.s, w.st);
-        if (w.mg) mg_apply(w.mg, w.mg32, w.s, w.sh, flag, st, &ev);
+        launch_chained(true, update_s64_kernel, grid_of(update_s64_kernel, N), kThreads, 0, st, N, w.r, w.v, w.s,
+                       w.st);
+        if (w.mg) mg_apply(w.mg, w.mg32, w.s, w.sh, flag, st, &ev, true);
         e = prof_begin(st);
-        spmv64_kernel<TPR, 1><<<grid_of(spmv64_kernel<TPR, 1>, N * TPR), kThreads, 0, st>>>(
-            A.row_ptr, A.col, val, N, sin_, w.dinv, w.t, nullptr, w.st, w.part, w.mg ? w.s : nullptr);
+        launch_chained(true, spmv64_kernel<TPR, 1>, grid_of(spmv64_kernel<TPR, 1>, N * TPR), kThreads, 0, st,
+                       A.row_ptr, A.col, val, N, sin_, w.dinv, w.t, nullptr, w.st, w.part, w.mg ? w.s : nullptr);
         prof_end(e, st, kProfSpmv64, bytes);
         ev.push_back(e);
-        update_xr64_kernel<<<grid_of(update_xr64_kernel, N), kThreads, 0, st>>>(N, x, pin, w.s, w.t, w.r, w.rh, w.d,
-                                                                             w.st, w.part, w.mg ? w.sh : nullptr);
+        launch_chained(true, update_xr64_kernel, grid_of(update_xr64_kernel, N), kThreads, 0, st, N, x, pin, w.s,
+                       w.t, w.r, w.rh, w.d, w.st, w.part, w.mg ? w.sh : nullptr);
         note_launches(5);
     }
 };
 
 template <int TPR>
 struct OpsDf {
-    static void iteration(const rbffd_csr& A32, const Work& w, cudaStream_t st, std::vector<int>& ev) {
+    static void iteration(const rbffd_csr& A32, const Work& w, cudaStream_t st, std::vector<int>& ev, bool chained) {
         const int64_t N = A32.n_rows;
         const float* val = static_cast<const float*>(A32.val);
         // algorithmic bytes: nnz (4 + 4) + row_ptr + 8-byte df32 vectors
         // (gathered once, result, dot partner) + 4-byte sigma and scale
         const int64_t bytes = spmv_bytes(A32, 4);
-        update_p_df_kernel<<<grid_of(update_p_df_kernel, N), kThreads, 0, st>>>(N, w.rd, w.vd, w.pd, w.st);
+        launch_chained(chained, update_p_df_kernel, grid_of(update_p_df_kernel, N), kThreads, 0, st, N, w.rd, w.vd,
+                       w.pd, w.st);
         int e = prof_begin(st);
-        spmv_df_kernel<TPR, 0><<<grid_of(spmv_df_kernel<TPR, 0>, N * TPR), kThreads, 0, st>>>(
-            A32.row_ptr, A32.col, val, N, w.pd, w.sigma32, w.dinv32, w.vd, w.rhd, w.st, w.part);
+        launch_chained(true, spmv_df_kernel<TPR, 0>, grid_of(spmv_df_kernel<TPR, 0>, N * TPR), kThreads, 0, st,
+                       A32.row_ptr, A32.col, val, N, w.pd, w.sigma32, w.dinv32, w.vd, w.rhd, w.st, w.part);
         prof_end(e, st, kProfSpmv32, bytes);
         ev.push_back(e);
-        update_s_df_kernel<<<grid_of(update_s_df_kernel, N), kThreads, 0, st>>>(N, w.rd, w.vd, w.sd, w.st);
+        launch_chained(true, update_s_df_kernel, grid_of(update_s_df_kernel, N), kThreads, 0, st, N, w.rd, w.vd,
+                       w.sd, w.st);
         e = prof_begin(st);
-        spmv_df_kernel<TPR, 1><<<grid_of(spmv_df_kernel<TPR, 1>, N * TPR), kThreads, 0, st>>>(
-            A32.row_ptr, A32.col, val, N, w.sd, w.sigma32, w.dinv32, w.td, nullptr, w.st, w.part);
+        launch_chained(true, spmv_df_kernel<TPR, 1>, grid_of(spmv_df_kernel<TPR, 1>, N * TPR), kThreads, 0, st,
+                       A32.row_ptr, A32.col, val, N, w.sd, w.sigma32, w.dinv32, w.td, nullptr, w.st, w.part);
         prof_end(e, st, kProfSpmv32, bytes);
         ev.push_back(e);
-        update_xr_df_kernel<<<grid_of(update_xr_df_kernel, N), kThreads, 0, st>>>(N, w.xd, w.pd, w.sd, w.td, w.rd,
-                                                                               w.rhd, w.d32, w.st, w.part);
+        launch_chained(true, update_xr_df_kernel, grid_of(update_xr_df_kernel, N), kThreads, 0, st, N, w.xd, w.pd,
+                       w.sd, w.td, w.rd, w.rhd, w.d32, w.st, w.part);
         note_launches(5);
     }
 };
@@ -952,21 +981,23 @@ void resid64(int tpr, int mode, const rbffd_csr& A, const double* b, const doubl
     }
 }
 
-void iter64(int tpr, const rbffd_csr& A, double* x, const Work& w, cudaStream_t st, std::vector<int>& ev) {
+// One iteration; chained: it follows another one of the same chunk.
+void iter64(int tpr, const rbffd_csr& A, double* x, const Work& w, cudaStream_t st, std::vector<int>& ev,
+            bool chained) {
     switch (tpr) {
-        case 1: Ops64<1>::iteration(A, x, w, st, ev); break;
-        case 2: Ops64<2>::iteration(A, x, w, st, ev); break;
-        case 8: Ops64<8>::iteration(A, x, w, st, ev); break;
-        default: Ops64<4>::iteration(A, x, w, st, ev); break;
+        case 1: Ops64<1>::iteration(A, x, w, st, ev, chained); break;
+        case 2: Ops64<2>::iteration(A, x, w, st, ev, chained); break;
+        case 8: Ops64<8>::iteration(A, x, w, st, ev, chained); break;
+        default: Ops64<4>::iteration(A, x, w, st, ev, chained); break;
     }
 }
 
-void iter_df(int tpr, const rbffd_csr& A32, const Work& w, cudaStream_t st, std::vector<int>& ev) {
+void iter_df(int tpr, const rbffd_csr& A32, const Work& w, cudaStream_t st, std::vector<int>& ev, bool chained) {
     switch (tpr) {
-        case 2: OpsDf<2>::iteration(A32, w, st, ev); break;
-        case 8: OpsDf<8>::iteration(A32, w, st, ev); break;
-        case 16: OpsDf<16>::iteration(A32, w, st, ev); break;
-        default: OpsDf<4>::iteration(A32, w, st, ev); break;
+        case 2: OpsDf<2>::iteration(A32, w, st, ev, chained); break;
+        case 8: OpsDf<8>::iteration(A32, w, st, ev, chained); break;
+        case 16: OpsDf<16>::iteration(A32, w, st, ev, chained); break;
+        default: OpsDf<4>::iteration(A32, w, st, ev, chained); break;
     }
 }
 
@@ -1072,7 +1103,7 @@ int run_chunks(const Work& w, KState* hs, cudaStream_t st, ChunkPlan& plan, Iter
         const int chunk = plan.chunk;
         const auto t0 = std::chrono::steady_clock::now();
         ev.clear();
-        for (int c = 0; c < chunk; ++c) iter(ev);
+        for (int c = 0; c < chunk; ++c) iter(ev, c > 0);
         RBFFD_LAUNCH_CHECK();
         const int rc = read_state(w, hs, st);
         if (rc != RBFFD_OK) return -rc;
@@ -1234,8 +1265,9 @@ int solve_fp64(const rbffd_csr& A, const double* b, double* x, const rbffd_solve
             RBFFD_LAUNCH_CHECK();
             if ((rc = read_state(w, &hs, st)) != RBFFD_OK) return rc;
         }
-        const int f = run_chunks(w, &hs, st, chunk, [&](std::vector<int>& ev) { iter64(tpr, A, x, w, st, ev); },
-                                 &mon, rel, total);
+        const int f = run_chunks(
+            w, &hs, st, chunk, [&](std::vector<int>& ev, bool chained) { iter64(tpr, A, x, w, st, ev, chained); }, &mon,
+            rel, total);
         if (f < 0) return -f;
         if (w.left && (rc = mg_dirichlet_fix(w.mg, b, x, nullptr, st)) != RBFFD_OK) return rc;
         total += hs.iter;
@@ -1333,8 +1365,9 @@ int solve_mixed(const rbffd_csr& A, const rbffd_csr& A32, const double* b, doubl
         RBFFD_LAUNCH_CHECK();
         if ((rc = read_state(w, &hs, st)) != RBFFD_OK) return rc;
         const double start2 = hs.rmax2;
-        const int f = run_chunks(w, &hs, st, chunk, [&](std::vector<int>& ev) { iter_df(tpr32, A32, w, st, ev); },
-                                 &mon, rel, total);
+        const int f = run_chunks(
+            w, &hs, st, chunk, [&](std::vector<int>& ev, bool chained) { iter_df(tpr32, A32, w, st, ev, chained); },
+            &mon, rel, total);
         if (f < 0) return -f;
         total += hs.iter;
         if (trace_on())

@@ -40,7 +40,6 @@
 // accuracy, the outer FP64 BiCGSTAB keeps the residual exact).
 #include "common.cuh"
 #include "internal.cuh"
-#include "mg_cluster.cuh"
 #include "scan.cuh"
 
 #include <cooperative_groups.h>
@@ -48,8 +47,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <map>
-#include <mutex>
+#include <type_traits>
 #include <vector>
 
 namespace rbffd {
@@ -108,53 +106,111 @@ __device__ __forceinline__ T row_sum(const int64_t* __restrict__ row_ptr, const 
 
 __device__ __forceinline__ bool stopped(const int* flag) { return flag && *(volatile const int*)flag != 0; }
 
+// The start of a lane's share of a row (its first U entries), loaded before
+// the chain's previous kernel has completed; sum() is row_sum with them.
+template <typename T, int TPR>
+struct RowHead {
+    static constexpr int U = TPR >= 4 ? 4 : 6;
+    int64_t a, e;
+    int c[U];
+    T v[U];
+    __device__ __forceinline__ void load(const int64_t* __restrict__ row_ptr, const int* __restrict__ col,
+                                         const T* __restrict__ val, int64_t row, int sub, bool valid) {
+        a = e = 0;
+        if (valid) {
+            a = __ldg(row_ptr + row);
+            e = __ldg(row_ptr + row + 1);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t k = a + sub + u * TPR;
+            c[u] = k < e ? __ldg(col + k) : 0;
+            v[u] = k < e ? __ldg(val + k) : T(0);
+        }
+    }
+    __device__ __forceinline__ T sum(const int* __restrict__ col, const T* __restrict__ val,
+                                     const T* __restrict__ x, int64_t nx, int sub) const {
+        (void)nx;  // length of x: bound of the checked build's tests
+        T xv[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) xv[u] = a + sub + u * TPR < e ? __ldg(&RB_AT(x, c[u], nx)) : T(0);
+        T s = T(0);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (a + sub + u * TPR < e) s = fmaT<T>(v[u], xv[u], s);
+#pragma unroll 4
+        for (int64_t k = a + sub + U * TPR; k < e; k += TPR)
+            s = fmaT<T>(__ldg(val + k), __ldg(&RB_AT(x, __ldg(col + k), nx)), s);
+#pragma unroll
+        for (int o = TPR / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, TPR);
+        return s;
+    }
+};
+
+// A chained kernel over the rows of a CSR matrix: f(i, sum) in one lane per
+// row, sum = (A x)_i.  HEAD: the first row's entries are loaded before the
+// wait (for launches whose lanes have one row each; it costs the registers
+// that hold 64 warps per SM in the large ones).
+template <typename T, int TPR, bool HEAD, class F>
+__device__ __forceinline__ void chained_rows(const int64_t* __restrict__ row_ptr, const int* __restrict__ col,
+                                             const T* __restrict__ val, int64_t N, const T* __restrict__ x,
+                                             int64_t nx, const int* flag, F&& f) {
+    const int sub = threadIdx.x & (TPR - 1);
+    if constexpr (HEAD) {
+        const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / TPR;  // one row per group of lanes
+        RowHead<T, TPR> head;
+        head.load(row_ptr, col, val, i, sub, i < N);
+        pdl_wait();
+        pdl_next();
+        if (stopped(flag)) return;
+        const T s = head.sum(col, val, x, nx, sub);
+        if (i < N && sub == 0) f(i, s);
+    } else {
+        pdl_wait();
+        pdl_next();
+        if (stopped(flag)) return;
+        MG_ROWS(TPR, N, i, valid, {
+            const T s = row_sum<T, TPR>(row_ptr, col, val, x, nx, i, sub, valid);
+            if (valid && sub == 0) f(i, s);
+        })
+    }
+}
+
 // x = W b (the first sweep from x = 0); dinv holds W = Omega D^-1
 template <typename T, typename BT>
 __global__ void __launch_bounds__(kT) mg_first_kernel(int64_t N, const BT* __restrict__ b, const T* __restrict__ dinv,
                                                       T* __restrict__ x, const int* flag) {
+    pdl_wait();
+    pdl_next();
     if (stopped(flag)) return;
     MG_ELEMS(N, i) x[i] = dinv[i] * (T)b[i];
 }
 
 // xo = xi + W (b - A xi)
-template <typename T, typename BT, typename OT, int TPR>
+template <typename T, typename BT, typename OT, int TPR, bool HEAD>
 __global__ void __launch_bounds__(kT) mg_jacobi_kernel(const int64_t* __restrict__ row_ptr, const int* __restrict__ col,
                                                        const T* __restrict__ val, int64_t N, const T* __restrict__ xi,
                                                        const BT* __restrict__ b, const T* __restrict__ dinv,
                                                        OT* __restrict__ xo, const int* flag) {
-    if (stopped(flag)) return;
-    const int sub = threadIdx.x & (TPR - 1);
-    MG_ROWS(TPR, N, i, valid, {
-        const T ax = row_sum<T, TPR>(row_ptr, col, val, xi, N, i, sub, valid);
-        if (valid && sub == 0) xo[i] = (OT)fmaT<T>(dinv[i], (T)b[i] - ax, xi[i]);
-    })
+    chained_rows<T, TPR, HEAD>(row_ptr, col, val, N, xi, N, flag,
+                         [&](int64_t i, T ax) { xo[i] = (OT)fmaT<T>(dinv[i], (T)b[i] - ax, xi[i]); });
 }
 
 // r = b - A x
-template <typename T, typename BT, int TPR>
+template <typename T, typename BT, int TPR, bool HEAD>
 __global__ void __launch_bounds__(kT) mg_resid_kernel(const int64_t* __restrict__ row_ptr, const int* __restrict__ col,
                                                       const T* __restrict__ val, int64_t N, const T* __restrict__ x,
                                                       const BT* __restrict__ b, T* __restrict__ r, const int* flag) {
-    if (stopped(flag)) return;
-    const int sub = threadIdx.x & (TPR - 1);
-    MG_ROWS(TPR, N, i, valid, {
-        const T ax = row_sum<T, TPR>(row_ptr, col, val, x, N, i, sub, valid);
-        if (valid && sub == 0) r[i] = (T)b[i] - ax;
-    })
+    chained_rows<T, TPR, HEAD>(row_ptr, col, val, N, x, N, flag, [&](int64_t i, T ax) { r[i] = (T)b[i] - ax; });
 }
 
 // y = R r (restriction, CSR with n rows)
-template <typename T, int TPR>
+template <typename T, int TPR, bool HEAD>
 __global__ void __launch_bounds__(kT) mg_restrict_kernel(const int64_t* __restrict__ row_ptr,
                                                          const int* __restrict__ col, const T* __restrict__ val,
                                                          int64_t n, const T* __restrict__ r, int64_t nr,
                                                          T* __restrict__ y, const int* flag) {
-    if (stopped(flag)) return;
-    const int sub = threadIdx.x & (TPR - 1);
-    MG_ROWS(TPR, n, i, valid, {
-        const T v = row_sum<T, TPR>(row_ptr, col, val, r, nr, i, sub, valid);
-        if (valid && sub == 0) y[i] = v;
-    })
+    chained_rows<T, TPR, HEAD>(row_ptr, col, val, n, r, nr, flag, [&](int64_t i, T v) { y[i] = v; });
 }
 
 // x += P e (ELL, kMgK entries per row)
@@ -163,13 +219,34 @@ __global__ void __launch_bounds__(kT) mg_prolong_kernel(int64_t N, const int32_t
                                                         const T* __restrict__ pval, const T* __restrict__ e,
                                                         int64_t ne, T* __restrict__ x, const int* flag) {
     (void)ne;  // length of e: bound of the checked build's tests
+    // the first row's entries before the wait (three 16-byte loads of each array)
+    static_assert(kMgK % 4 == 0, "rows of whole 16-byte loads");
+    int4 c[kMgK / 4];
+    T v[kMgK];
+    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    auto load = [&](int64_t i) {
+#pragma unroll
+        for (int j = 0; j < kMgK / 4; ++j) c[j] = __ldg(reinterpret_cast<const int4*>(pidx + i * kMgK) + j);
+#pragma unroll
+        for (int j = 0; j < (int)(kMgK * sizeof(T) / 16); ++j) {
+            const float4 q = __ldg(reinterpret_cast<const float4*>(pval + i * kMgK) + j);
+            memcpy(reinterpret_cast<char*>(v) + 16 * j, &q, 16);
+        }
+    };
+    if (i0 < N) load(i0);
+    pdl_wait();
+    pdl_next();
     if (stopped(flag)) return;
     MG_ELEMS(N, i) {
-        const int32_t* ip = pidx + i * kMgK;
-        const T* vp = pval + i * kMgK;
+        if (i != i0) load(i);
         T acc = x[i];
 #pragma unroll
-        for (int j = 0; j < kMgK; ++j) acc = fmaT<T>(__ldg(vp + j), __ldg(&RB_AT(e, __ldg(ip + j), ne)), acc);
+        for (int j = 0; j < kMgK / 4; ++j) {
+            acc = fmaT<T>(v[4 * j], __ldg(&RB_AT(e, c[j].x, ne)), acc);
+            acc = fmaT<T>(v[4 * j + 1], __ldg(&RB_AT(e, c[j].y, ne)), acc);
+            acc = fmaT<T>(v[4 * j + 2], __ldg(&RB_AT(e, c[j].z, ne)), acc);
+            acc = fmaT<T>(v[4 * j + 3], __ldg(&RB_AT(e, c[j].w, ne)), acc);
+        }
         x[i] = acc;
     }
 }
@@ -178,6 +255,8 @@ __global__ void __launch_bounds__(kT) mg_prolong_kernel(int64_t N, const int32_t
 template <typename T, typename BT, typename OT>
 __global__ void __launch_bounds__(kT) mg_dense_kernel(int n, const T* __restrict__ minv, const BT* __restrict__ b,
                                                       OT* __restrict__ x, const int* flag) {
+    pdl_wait();
+    pdl_next();
     if (stopped(flag)) return;
     const int lane = threadIdx.x & 31;
     const int warps = (gridDim.x * blockDim.x) >> 5;
@@ -300,6 +379,8 @@ __global__ void __launch_bounds__(kT) mg_bfix_kernel(const int64_t* __restrict__
                                                      const double* __restrict__ val, int64_t N,
                                                      const uint8_t* __restrict__ mask, const double* __restrict__ w,
                                                      const double* __restrict__ r, double* y, const int* flag) {
+    pdl_wait();
+    pdl_next();
     if (stopped(flag)) return;
     MG_ELEMS(N, i) {
         if (!mask[i]) continue;
@@ -1051,95 +1132,275 @@ struct Sel<float> {
     static float* b(const MgLevel& L) { return L.b32; }
 };
 
+// Launches whose rows are at most this many groups' lanes load the rows
+// before the wait for the previous kernel (all lanes resident at once).
+bool head_rows(int64_t rows, int tpr) { return rows * tpr <= (int64_t)sm_count() * 4 * kT; }
+
+// f(lanes per row, rows loaded ahead) with both as compile-time constants.
+template <class F>
+void row_launch(int64_t rows, int tpr, F&& f) {
+    const bool head = head_rows(rows, tpr);
+    auto go = [&](auto tc) {
+        if (head) f(tc, std::true_type());
+        else f(tc, std::false_type());
+    };
+    switch (tpr) {
+        case 8: go(std::integral_constant<int, 8>()); break;
+        case 4: go(std::integral_constant<int, 4>()); break;
+        case 2: go(std::integral_constant<int, 2>()); break;
+        default: go(std::integral_constant<int, 1>()); break;
+    }
+}
+
 template <typename T, typename BT, typename OT>
 void jacobi(const MgLevel& L, const T* xi, const BT* b, OT* xo, const int* flag, cudaStream_t st) {
-    const int g = blocks_for(L.N * L.tpr);
-    const T* val = Sel<T>::val(L);
-    const T* dinv = Sel<T>::dinv(L);
-    switch (L.tpr) {
-        case 8: mg_jacobi_kernel<T, BT, OT, 8><<<g, kT, 0, st>>>(L.row_ptr, L.col, val, L.N, xi, b, dinv, xo, flag); break;
-        case 4: mg_jacobi_kernel<T, BT, OT, 4><<<g, kT, 0, st>>>(L.row_ptr, L.col, val, L.N, xi, b, dinv, xo, flag); break;
-        case 2: mg_jacobi_kernel<T, BT, OT, 2><<<g, kT, 0, st>>>(L.row_ptr, L.col, val, L.N, xi, b, dinv, xo, flag); break;
-        default: mg_jacobi_kernel<T, BT, OT, 1><<<g, kT, 0, st>>>(L.row_ptr, L.col, val, L.N, xi, b, dinv, xo, flag); break;
-    }
+    row_launch(L.N, L.tpr, [&](auto tc, auto hc) {
+        launch_chained(true, mg_jacobi_kernel<T, BT, OT, decltype(tc)::value, decltype(hc)::value>,
+                       blocks_for(L.N * L.tpr), kT, 0, st, L.row_ptr, L.col, Sel<T>::val(L), L.N, xi, b,
+                       Sel<T>::dinv(L), xo, flag);
+    });
 }
 
 template <typename T, typename BT>
 void resid(const MgLevel& L, const T* x, const BT* b, T* r, const int* flag, cudaStream_t st) {
-    const int g = blocks_for(L.N * L.tpr);
-    const T* val = Sel<T>::val(L);
-    switch (L.tpr) {
-        case 8: mg_resid_kernel<T, BT, 8><<<g, kT, 0, st>>>(L.row_ptr, L.col, val, L.N, x, b, r, flag); break;
-        case 4: mg_resid_kernel<T, BT, 4><<<g, kT, 0, st>>>(L.row_ptr, L.col, val, L.N, x, b, r, flag); break;
-        case 2: mg_resid_kernel<T, BT, 2><<<g, kT, 0, st>>>(L.row_ptr, L.col, val, L.N, x, b, r, flag); break;
-        default: mg_resid_kernel<T, BT, 1><<<g, kT, 0, st>>>(L.row_ptr, L.col, val, L.N, x, b, r, flag); break;
-    }
+    row_launch(L.N, L.tpr, [&](auto tc, auto hc) {
+        launch_chained(true, mg_resid_kernel<T, BT, decltype(tc)::value, decltype(hc)::value>,
+                       blocks_for(L.N * L.tpr), kT, 0, st, L.row_ptr, L.col, Sel<T>::val(L), L.N, x, b, r, flag);
+    });
 }
 
 template <typename T>
 void restrict_to(const MgLevel& L, int64_t nc, const T* r, T* bc, const int* flag, cudaStream_t st) {
-    const int g = blocks_for(nc * L.rtpr);
-    const T* val = Sel<T>::rval(L);
-    switch (L.rtpr) {
-        case 8: mg_restrict_kernel<T, 8><<<g, kT, 0, st>>>(L.rrow, L.rcol, val, nc, r, L.N, bc, flag); break;
-        case 4: mg_restrict_kernel<T, 4><<<g, kT, 0, st>>>(L.rrow, L.rcol, val, nc, r, L.N, bc, flag); break;
-        case 2: mg_restrict_kernel<T, 2><<<g, kT, 0, st>>>(L.rrow, L.rcol, val, nc, r, L.N, bc, flag); break;
-        default: mg_restrict_kernel<T, 1><<<g, kT, 0, st>>>(L.rrow, L.rcol, val, nc, r, L.N, bc, flag); break;
+    row_launch(nc, L.rtpr, [&](auto tc, auto hc) {
+        launch_chained(true, mg_restrict_kernel<T, decltype(tc)::value, decltype(hc)::value>,
+                       blocks_for(nc * L.rtpr), kT, 0, st, L.rrow, L.rcol, Sel<T>::rval(L), nc, r, L.N, bc, flag);
+    });
+}
+
+// The small levels' part of the cycle by one block, its vectors in shared
+// memory: a level of some hundred nodes is a few microseconds of launch
+// latency per operation (six per level) and a fraction of one of work.  Every
+// row is summed by the same lanes in the same order as in the kernels above,
+// so the result has the same bits.
+// 845 + 190 + 45 rows: 23 us, 14 launches before.  (A cluster of 16 blocks, up
+// to 20k rows, took 88 us for five levels: its barrier costs 600 to 1,700
+// cycles and a neighbour in another block's shared memory or in L2 500 to
+// 700, once per operation and entry.)
+constexpr int kTailT = 1024;
+constexpr int kTailLevels = 16;
+constexpr int kTailSmem = 64 * 1024;  // leaves the rest of L1 to the matrices
+
+template <typename T>
+struct TailLevel {
+    int n, tpr, rtpr;  // rows; lanes per row of A and of the restriction into the next level
+    int nnz;
+    const int64_t* row_ptr;
+    const int* col;
+    const T* val;
+    const T* w;
+    const int32_t* pidx;
+    const T* pval;
+    const int64_t* rrow;
+    const int32_t* rcol;
+    const T* rval;
+};
+
+template <typename T>
+struct TailCycle {
+    int levels, nu;
+    const T* minv;
+    const T* b;  // right-hand side and result of the first level (not TOP)
+    T* x;
+    TailLevel<T> lv[kTailLevels];
+};
+
+// Rows of a CSR matrix by one block, TPR lanes per row: f(i, sum) in one lane.
+template <typename T, int TPR, class F>
+__device__ __forceinline__ void tail_rows(const int64_t* __restrict__ row_ptr, const int* __restrict__ col,
+                                          const T* __restrict__ val, const T* x, int nx, int n, F&& f) {
+    (void)nx;  // length of x: bound of the checked build's tests
+    const int sub = threadIdx.x & (TPR - 1), off = (threadIdx.x & 31) / TPR;
+    for (int base = (int)threadIdx.x / TPR - off; base < n; base += kTailT / TPR) {
+        const int i = base + off;
+        int64_t a = 0, e = 0;
+        if (i < n) {
+            a = __ldg(row_ptr + i);
+            e = __ldg(row_ptr + i + 1);
+        }
+        T sum = T(0);
+#pragma unroll 4
+        for (int64_t k = a + sub; k < e; k += TPR) sum = fmaT<T>(__ldg(val + k), RB_AT(x, __ldg(col + k), nx), sum);
+#pragma unroll
+        for (int o = TPR / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o, TPR);
+        if (i < n && sub == 0) f(i, sum);
     }
 }
 
-// The levels [first, n_levels) by one cluster.  TOP: level 0 is among them,
-// its right-hand side and result are the caller's FP64 vectors.
-template <typename T, bool TOP>
-__global__ void __launch_bounds__(kClThreads) mg_cluster_kernel(const __grid_constant__ ClCycle<T> c,
-                                                                const double* __restrict__ b, double* __restrict__ x) {
-    if (stopped(c.flag)) return;
-    auto cluster = cooperative_groups::this_cluster();
-    const ClLevel<T>& L = c.lv[0];
-    if constexpr (TOP)
-        cl_cycle<T>(c, [&](int i) { return (T)__ldg(&RB_AT(b, i, L.n)); }, [&](int i, T v) { x[i] = (double)v; },
-                    [&] { cluster.sync(); });
-    else
-        cl_cycle<T>(c, [&](int i) { return __ldg(&RB_AT(L.b, i, L.n)); },
-                    [&](int i, T v) { (c.levels == 1 ? L.x : L.t)[i] = v; }, [&] { cluster.sync(); });
+template <typename T, class F>
+__device__ __forceinline__ void tail_csr(int tpr, const int64_t* row_ptr, const int* col, const T* val, const T* x,
+                                         int nx, int n, F&& f) {
+    if (tpr == 8) tail_rows<T, 8>(row_ptr, col, val, x, nx, n, f);
+    else if (tpr == 4) tail_rows<T, 4>(row_ptr, col, val, x, nx, n, f);
+    else if (tpr == 2) tail_rows<T, 2>(row_ptr, col, val, x, nx, n, f);
+    else tail_rows<T, 1>(row_ptr, col, val, x, nx, n, f);
 }
 
-// Rows up to which a level belongs to the cluster: its operations cost the
-// cluster's 16 SMs about as long as a launch over the whole GPU.  (FP64: the
-// units' rate on 16 SMs is the limit, 12 multiply-adds per row.)
+__device__ __forceinline__ void tail_prefetch(const void* p, int64_t bytes) {
+    const char* c = static_cast<const char*>(p);
+    for (int64_t o = (int64_t)threadIdx.x * 128; o < bytes; o += (int64_t)kTailT * 128)
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(c + o));
+}
+
+// TOP: level 0 is the first one, its right-hand side and result are the
+// caller's FP64 vectors.
+template <typename T, bool TOP>
+__global__ void __launch_bounds__(kTailT) mg_tail_kernel(const __grid_constant__ TailCycle<T> c,
+                                                         const double* __restrict__ b64, double* __restrict__ x64,
+                                                         const int* flag) {
+    extern __shared__ __align__(16) unsigned char tail_smem[];
+    T* vec = reinterpret_cast<T*>(tail_smem);  // per level: two iterates, residual, right-hand side
+    const int tid = (int)threadIdx.x, last = c.levels - 1;
+    for (int l = 0; l < last; ++l) {
+        const TailLevel<T>& L = c.lv[l];
+        const int64_t rn = (int64_t)L.n * kMgK;
+        tail_prefetch(L.row_ptr, (L.n + 1) * 8);
+        tail_prefetch(L.col, L.nnz * 4);
+        tail_prefetch(L.val, L.nnz * (int64_t)sizeof(T));
+        tail_prefetch(L.rcol, rn * 4);
+        tail_prefetch(L.rval, rn * (int64_t)sizeof(T));
+    }
+    pdl_wait();
+    pdl_next();
+    if (stopped(flag)) return;
+    for (int i = tid; i < c.lv[0].n; i += kTailT) vec[3 * c.lv[0].n + i] = TOP ? (T)b64[i] : c.b[i];
+    __syncthreads();
+    T* v = vec;  // the level's vectors
+    for (int l = 0; l < last; ++l) {
+        const TailLevel<T>& L = c.lv[l];
+        const int n = L.n;
+        T *cur = v, *oth = v + n, *r = v + 2 * n, *b = v + 3 * n, *bc = v + 4 * n + 3 * c.lv[l + 1].n;
+        for (int i = tid; i < n; i += kTailT) cur[i] = __ldg(L.w + i) * b[i];
+        __syncthreads();
+        for (int k = 1; k < c.nu; ++k) {
+            tail_csr<T>(L.tpr, L.row_ptr, L.col, L.val, cur, n, n,
+                        [&](int i, T ax) { oth[i] = fmaT<T>(__ldg(L.w + i), b[i] - ax, cur[i]); });
+            T* s = cur;
+            cur = oth;
+            oth = s;
+            __syncthreads();
+        }
+        tail_csr<T>(L.tpr, L.row_ptr, L.col, L.val, cur, n, n, [&](int i, T ax) { r[i] = b[i] - ax; });
+        __syncthreads();
+        tail_csr<T>(L.rtpr, L.rrow, L.rcol, L.rval, r, n, c.lv[l + 1].n, [&](int i, T s) { bc[i] = s; });
+        __syncthreads();
+        v += 4 * n;
+    }
+    {  // coarsest: one warp per row
+        const int n = c.lv[last].n, lane = tid & 31;
+        for (int i = tid >> 5; i < n; i += kTailT / 32) {
+            T acc = T(0);
+            for (int j = lane; j < n; j += 32) acc = fmaT<T>(__ldg(c.minv + (int64_t)i * n + j), v[3 * n + j], acc);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (lane == 0) v[i] = acc;
+        }
+    }
+    for (int l = last - 1; l >= 0; --l) {
+        __syncthreads();
+        const TailLevel<T>& L = c.lv[l];
+        const int n = L.n, nc = c.lv[l + 1].n;
+        // the coarse result: in the second iterate (an odd number of swaps),
+        // in the first at the coarsest level
+        const T* e = v + (l + 1 == last ? 0 : nc);
+        (void)nc;
+        v -= 4 * n;
+        T* cur = v + ((c.nu & 1) ? 0 : n);
+        T* oth = v + ((c.nu & 1) ? n : 0);
+        const T* b = v + 3 * n;
+        for (int i = tid; i < n; i += kTailT) {
+            const int32_t* ip = L.pidx + (int64_t)i * kMgK;
+            const T* vp = L.pval + (int64_t)i * kMgK;
+            T acc = cur[i];
+#pragma unroll
+            for (int j = 0; j < kMgK; ++j) acc = fmaT<T>(__ldg(vp + j), RB_AT(e, __ldg(ip + j), nc), acc);
+            cur[i] = acc;
+        }
+        for (int k = 0; k < c.nu; ++k) {
+            __syncthreads();
+            tail_csr<T>(L.tpr, L.row_ptr, L.col, L.val, cur, n, n,
+                        [&](int i, T ax) { oth[i] = fmaT<T>(__ldg(L.w + i), b[i] - ax, cur[i]); });
+            T* s = cur;
+            cur = oth;
+            oth = s;
+        }
+    }
+    __syncthreads();
+    const int n = c.lv[0].n;
+    const T* res = vec + (last == 0 ? 0 : n);
+    for (int i = tid; i < n; i += kTailT) {
+        if constexpr (TOP) x64[i] = (double)res[i];
+        else c.x[i] = res[i];
+    }
+}
+
+// Matrix entries of the first level up to which one block takes it: a sweep
+// then costs about as long as a launch (the block reads ~64 bytes per clock
+// from L2; FP64: 2 multiply-adds per clock).
 template <typename T>
-constexpr int64_t cl_rows() {
-    return sizeof(T) == 8 ? 8192 : 32768;
+constexpr int64_t tail_entries() {
+    return sizeof(T) == 8 ? 6144 : 24576;
 }
 
-// Launches the cluster V-cycle; false where it does not apply.
+// The cycle of levels [first, n_levels) in one launch; false where it does
+// not apply.
 template <typename T, bool TOP>
-bool cluster_cycle(const MgHierarchy& h, int first, const double* b, double* x, const int* flag, cudaStream_t st) {
-    const void* kern = reinterpret_cast<const void*>(mg_cluster_kernel<T, TOP>);
-    const int size = cl_cluster_size(kern);
-    ClCycle<T> c;
-    if (size == 0 || !cl_make<T>(h, first, flag, &c)) return false;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)size);
-    cfg.blockDim = dim3(kClThreads);
-    cfg.stream = st;
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = (unsigned)size;
-    attr.val.clusterDim.y = 1;
-    attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, mg_cluster_kernel<T, TOP>, c, b, x) == cudaSuccess) return true;
-    (void)cudaGetLastError();  // the per-operation kernels run instead
-    return false;
+bool tail_cycle(const MgHierarchy& h, int first, const double* b, double* x, const int* flag, cudaStream_t st,
+                bool chained) {
+    const int levels = h.n_levels - first;
+    if (h.lv[first].nnz > tail_entries<T>() || levels > kTailLevels) return false;
+    TailCycle<T> c;
+    c.levels = levels;
+    c.nu = h.nu;
+    c.minv = Sel<T>::minv(h.lv[h.n_levels - 1]);
+    c.b = Sel<T>::b(h.lv[first]);
+    c.x = levels == 1 ? Sel<T>::x(h.lv[first]) : Sel<T>::t(h.lv[first]);
+    size_t smem = 0;
+    for (int l = 0; l < levels; ++l) {
+        const MgLevel& L = h.lv[first + l];
+        const bool last = l == levels - 1;
+        TailLevel<T>& t = c.lv[l];
+        t = TailLevel<T>{};
+        t.n = (int)L.N;
+        t.nnz = (int)L.nnz;
+        t.tpr = L.tpr;
+        t.row_ptr = L.row_ptr;
+        t.col = L.col;
+        t.val = Sel<T>::val(L);
+        t.w = Sel<T>::dinv(L);
+        if (!last) {
+            t.rtpr = L.rtpr;
+            t.pidx = L.pidx;
+            t.pval = Sel<T>::pval(L);
+            t.rrow = L.rrow;
+            t.rcol = L.rcol;
+            t.rval = Sel<T>::rval(L);
+        }
+        smem += 4 * (size_t)L.N * sizeof(T);
+    }
+    if (smem > kTailSmem) return false;
+    if (cudaFuncSetAttribute(mg_tail_kernel<T, TOP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTailSmem) !=
+        cudaSuccess)
+        return false;
+    launch_chained(chained, mg_tail_kernel<T, TOP>, 1, kTailT, smem, st, c, b, x, flag);
+    return true;
 }
 
 // One level of the cycle: b (BT) in, result in x (OT) for level 0, in the
-// level's own current-iterate buffer otherwise (returned).
+// level's own current-iterate buffer otherwise (returned).  chained: the
+// first kernel continues a chain (launch_chained); the others always do.
 template <typename T>
 T* cycle_level(const MgHierarchy& h, int l, const void* bin, bool b_is_double, double* out, const int* flag,
-               cudaStream_t st, int* launches, std::vector<int>* ev) {
+               cudaStream_t st, int* launches, std::vector<int>* ev, bool chained) {
     const MgLevel& L = h.lv[l];
     const bool last_level = (l == h.n_levels - 1);
     const bool top = (l == 0);
@@ -1147,20 +1408,20 @@ T* cycle_level(const MgHierarchy& h, int l, const void* bin, bool b_is_double, d
     T* oth = Sel<T>::t(L);
     // small levels: the rest of the cycle in one launch (not the top level
     // while its sweeps are being timed)
-    if (L.N <= cl_rows<T>() && !(top && ev && profiling())) {
-        const bool done = top ? b_is_double && cluster_cycle<T, true>(h, l, static_cast<const double*>(bin), out, flag, st)
-                              : cluster_cycle<T, false>(h, l, nullptr, nullptr, flag, st);
-        if (done) {
-            ++*launches;
-            return last_level ? cur : oth;
-        }
+    if (top ? b_is_double && !(ev && profiling()) &&
+                  tail_cycle<T, true>(h, l, static_cast<const double*>(bin), out, flag, st, chained)
+            : tail_cycle<T, false>(h, l, nullptr, nullptr, flag, st, chained)) {
+        ++*launches;
+        return last_level ? cur : oth;
     }
     auto launch_first = [&](T* x) {
         const int g = blocks_for(L.N);
         if (b_is_double)
-            mg_first_kernel<T, double><<<g, kT, 0, st>>>(L.N, static_cast<const double*>(bin), Sel<T>::dinv(L), x, flag);
+            launch_chained(chained, mg_first_kernel<T, double>, g, kT, 0, st, L.N, static_cast<const double*>(bin),
+                           Sel<T>::dinv(L), x, flag);
         else
-            mg_first_kernel<T, T><<<g, kT, 0, st>>>(L.N, static_cast<const T*>(bin), Sel<T>::dinv(L), x, flag);
+            launch_chained(chained, mg_first_kernel<T, T>, g, kT, 0, st, L.N, static_cast<const T*>(bin),
+                           Sel<T>::dinv(L), x, flag);
         ++*launches;
     };
     auto sweep = [&](T* xi, T* xo, double* xo64) {
@@ -1189,9 +1450,11 @@ T* cycle_level(const MgHierarchy& h, int l, const void* bin, bool b_is_double, d
         const int g = blocks_for((int64_t)L.N * 32);
         const T* mv = Sel<T>::minv(L);
         if (top) {
-            mg_dense_kernel<T, double, double><<<g, kT, 0, st>>>((int)L.N, mv, static_cast<const double*>(bin), out, flag);
+            launch_chained(chained, mg_dense_kernel<T, double, double>, g, kT, 0, st, (int)L.N, mv,
+                           static_cast<const double*>(bin), out, flag);
         } else {
-            mg_dense_kernel<T, T, T><<<g, kT, 0, st>>>((int)L.N, mv, static_cast<const T*>(bin), cur, flag);
+            launch_chained(chained, mg_dense_kernel<T, T, T>, g, kT, 0, st, (int)L.N, mv, static_cast<const T*>(bin),
+                           cur, flag);
         }
         ++*launches;
         return cur;
@@ -1208,8 +1471,9 @@ T* cycle_level(const MgHierarchy& h, int l, const void* bin, bool b_is_double, d
     const MgLevel& C = h.lv[l + 1];
     restrict_to<T>(L, C.N, Sel<T>::r(L), Sel<T>::b(C), flag, st);
     *launches += 2;
-    T* e = cycle_level<T>(h, l + 1, Sel<T>::b(C), false, nullptr, flag, st, launches, ev);
-    mg_prolong_kernel<T><<<blocks_for(L.N), kT, 0, st>>>(L.N, L.pidx, Sel<T>::pval(L), e, C.N, cur, flag);
+    T* e = cycle_level<T>(h, l + 1, Sel<T>::b(C), false, nullptr, flag, st, launches, ev, true);
+    launch_chained(true, mg_prolong_kernel<T>, blocks_for(L.N), kT, 0, st, L.N, L.pidx, Sel<T>::pval(L), e, C.N, cur,
+                   flag);
     ++*launches;
     // post-smoothing; the last sweep of level 0 writes the FP64 output
     for (int k = 0; k < h.nu; ++k) {
@@ -1221,71 +1485,6 @@ T* cycle_level(const MgHierarchy& h, int l, const void* bin, bool b_is_double, d
 }
 
 }  // namespace
-
-template <typename T>
-bool cl_make(const MgHierarchy& h, int first, const int* flag, ClCycle<T>* out) {
-    out->levels = h.n_levels - first;
-    if (first < 0 || out->levels < 1 || out->levels > kClMaxLevels) return false;
-    out->nu = h.nu;
-    out->flag = flag;
-    out->minv = Sel<T>::minv(h.lv[h.n_levels - 1]);
-    for (int l = first; l < h.n_levels; ++l) {
-        const MgLevel& L = h.lv[l];
-        if (L.N > 0x3fffffff) return false;
-        ClLevel<T>& c = out->lv[l - first];
-        const bool last = l == h.n_levels - 1;
-        c.n = (int)L.N;
-        c.tpr = L.tpr;
-        c.rtpr = last ? 1 : L.rtpr;
-        c.row_ptr = L.row_ptr;
-        c.col = L.col;
-        c.val = Sel<T>::val(L);
-        c.w = Sel<T>::dinv(L);
-        c.pidx = last ? nullptr : L.pidx;
-        c.pval = last ? nullptr : Sel<T>::pval(L);
-        c.rrow = last ? nullptr : L.rrow;
-        c.rcol = last ? nullptr : L.rcol;
-        c.rval = last ? nullptr : Sel<T>::rval(L);
-        c.x = Sel<T>::x(L);
-        c.t = Sel<T>::t(L);
-        c.r = Sel<T>::r(L);
-        c.b = Sel<T>::b(L);
-    }
-    return true;
-}
-template bool cl_make<float>(const MgHierarchy&, int, const int*, ClCycle<float>*);
-template bool cl_make<double>(const MgHierarchy&, int, const int*, ClCycle<double>*);
-
-int cl_cluster_size(const void* kernel) {
-    static std::mutex mu;
-    static std::map<std::pair<int, const void*>, int> cache;
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-    const auto key = std::make_pair(dev, kernel);
-    std::lock_guard<std::mutex> lk(mu);
-    auto it = cache.find(key);
-    if (it != cache.end()) return it->second;
-    int size = 0;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
-        for (int s = 16; s >= 8 && size == 0; s /= 2) {
-            cudaLaunchConfig_t cfg{};
-            cfg.gridDim = dim3((unsigned)s);
-            cfg.blockDim = dim3(kClThreads);
-            cudaLaunchAttribute attr{};
-            attr.id = cudaLaunchAttributeClusterDimension;
-            attr.val.clusterDim.x = (unsigned)s;
-            attr.val.clusterDim.y = 1;
-            attr.val.clusterDim.z = 1;
-            cfg.attrs = &attr;
-            cfg.numAttrs = 1;
-            int clusters = 0;
-            if (cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess && clusters > 0) size = s;
-        }
-    }
-    (void)cudaGetLastError();  // a refused size is not the caller's error
-    cache[key] = size;
-    return size;
-}
 
 size_t mg_multi_coarse_floats(const MgHierarchy* h, int R) {
     if (!h) return 0;
@@ -1309,10 +1508,12 @@ bool mg_is_transposed(const MgHierarchy* h) { return h && h->transposed; }
 
 bool mg_is_galerkin(const MgHierarchy* h) { return h && h->galerkin; }
 
-int mg_dirichlet_fix(const MgHierarchy* h, const double* r, double* y, const int* flag, cudaStream_t st) {
+int mg_dirichlet_fix(const MgHierarchy* h, const double* r, double* y, const int* flag, cudaStream_t st,
+                     bool chained) {
     if (!h || !r || !y || h->col_base != 0) return RBFFD_ERR_INVALID_ARG;
     const MgLevel& L = h->lv[0];
-    mg_bfix_kernel<<<blocks_for(L.N), kT, 0, st>>>(L.row_ptr, L.col, L.val, L.N, L.mask, L.dinv, r, y, flag);
+    launch_chained(chained, mg_bfix_kernel, blocks_for(L.N), kT, 0, st, L.row_ptr, L.col, L.val, L.N, L.mask, L.dinv, r,
+                   y, flag);
     note_launches(1);
     RBFFD_LAUNCH_CHECK();
     return RBFFD_OK;
@@ -1320,36 +1521,38 @@ int mg_dirichlet_fix(const MgHierarchy* h, const double* r, double* y, const int
 
 __global__ void __launch_bounds__(kT) mg_zero_dirichlet_kernel(int64_t N, const uint8_t* __restrict__ mask,
                                                                double* __restrict__ y, const int* flag) {
+    pdl_wait();
+    pdl_next();
     if (stopped(flag)) return;
     MG_ELEMS(N, i) if (mask[i]) y[i] = 0.0;
 }
 
 int mg_apply_interior(const MgHierarchy* h, bool fp32, const double* b, double* x, const int* flag, cudaStream_t st,
-                      std::vector<int>* ev) {
+                      std::vector<int>* ev, bool chained) {
     if (!h || !b || !x || h->col_base != 0) return RBFFD_ERR_INVALID_ARG;
     if (fp32 && !h->has32) return RBFFD_ERR_INVALID_ARG;
     int launches = 0;
-    if (fp32) cycle_level<float>(*h, 0, b, true, x, flag, st, &launches, ev);
-    else cycle_level<double>(*h, 0, b, true, x, flag, st, &launches, ev);
+    if (fp32) cycle_level<float>(*h, 0, b, true, x, flag, st, &launches, ev, chained);
+    else cycle_level<double>(*h, 0, b, true, x, flag, st, &launches, ev, chained);
     const MgLevel& L = h->lv[0];
-    mg_zero_dirichlet_kernel<<<blocks_for(L.N), kT, 0, st>>>(L.N, L.mask, x, flag);
+    launch_chained(true, mg_zero_dirichlet_kernel, blocks_for(L.N), kT, 0, st, L.N, L.mask, x, flag);
     note_launches(launches + 1);
     RBFFD_LAUNCH_CHECK();
     return RBFFD_OK;
 }
 
 int mg_apply(const MgHierarchy* h, bool fp32, const double* b, double* x, const int* flag, cudaStream_t st,
-             std::vector<int>* ev) {
+             std::vector<int>* ev, bool chained) {
     if (!h || !b || !x || h->col_base != 0) return RBFFD_ERR_INVALID_ARG;
     if (fp32 && !h->has32) return RBFFD_ERR_INVALID_ARG;
     int launches = 0;
-    if (fp32) cycle_level<float>(*h, 0, b, true, x, flag, st, &launches, ev);
-    else cycle_level<double>(*h, 0, b, true, x, flag, st, &launches, ev);
+    if (fp32) cycle_level<float>(*h, 0, b, true, x, flag, st, &launches, ev, chained);
+    else cycle_level<double>(*h, 0, b, true, x, flag, st, &launches, ev, chained);
     note_launches(launches);
     RBFFD_LAUNCH_CHECK();
     // adjoint: the transpose of the boundary-eliminated forward cycle
     // E_b + B (I - A E_b) is B^T followed by the Dirichlet back substitution
-    if (h->transposed) return mg_dirichlet_fix(h, b, x, flag, st);
+    if (h->transposed) return mg_dirichlet_fix(h, b, x, flag, st, true);
     return RBFFD_OK;
 }
 
