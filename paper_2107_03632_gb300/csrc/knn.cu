@@ -8,10 +8,14 @@
 //
 // Pipeline (all on the stream, no host synchronisation):
 //   1. bounding box (block partials, then one block)         -> GridParams
-//   2. cell key per node, histogram of keys (atomics)
+//   2. histogram of the nodes' cells (atomics)
 //   3. exclusive scan of the histogram                       -> cell_start
-//   4. scatter nodes into cell order (SoA double2 + original index)
-//   5. one warp per query, in cell order: scan cells ring by ring around the
+//   4. scatter nodes into cell order (double2, original index, fixed-point
+//      coordinates)
+//   5. one warp per query, in cell order: select the candidates by fixed-point
+//      distances, rank the few that remain by their exact keys, once
+//      (knn_fast_kernel, n <= 112)
+//   6. the queries left, and n > 112: scan cells ring by ring around the
 //      query's cell, keep a sorted top-n list of keys distributed over the
 //      warp's registers (entry e at lane e%32, slot e/32), prune cells whose
 //      nearest point cannot beat the current n-th key, and stop once the
@@ -37,12 +41,18 @@ struct GridParams {
     double cell;        // cell side
     double inv_cell;    // 1 / cell
     double margin;      // absolute slack for the geometric pruning tests
+    double inv_fix;     // kFix / cell
     int G;              // cells per axis (G x G cells)
-    int pad;
+    int fast;           // every coordinate is finite: the fixed-point search applies
 };
+
+// Fixed-point grid coordinates: units per cell.
+constexpr int kFixBits = 12;
+constexpr int kFix = 1 << kFixBits;
 
 struct Box {
     double mnx, mny, mxx, mxy;
+    double odd;  // 1: a coordinate is not finite
 };
 
 constexpr int kBoxBlocks = 256;
@@ -50,16 +60,18 @@ constexpr int kBoxThreads = 256;
 
 __global__ void __launch_bounds__(kBoxThreads) bbox_partial_kernel(const double2* __restrict__ xy, int64_t N,
                                                                    Box* __restrict__ part) {
-    double mnx = INFINITY, mny = INFINITY, mxx = -INFINITY, mxy = -INFINITY;
+    double mnx = INFINITY, mny = INFINITY, mxx = -INFINITY, mxy = -INFINITY, odd = 0.0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
         const double2 p = xy[i];
         mnx = fmin(mnx, p.x);
         mny = fmin(mny, p.y);
         mxx = fmax(mxx, p.x);
         mxy = fmax(mxy, p.y);
+        if (!finite64(p.x) || !finite64(p.y)) odd = 1.0;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
+        odd = fmax(odd, __shfl_xor_sync(0xffffffffu, odd, o));
         mnx = fmin(mnx, __shfl_xor_sync(0xffffffffu, mnx, o));
         mny = fmin(mny, __shfl_xor_sync(0xffffffffu, mny, o));
         mxx = fmax(mxx, __shfl_xor_sync(0xffffffffu, mxx, o));
@@ -67,7 +79,7 @@ __global__ void __launch_bounds__(kBoxThreads) bbox_partial_kernel(const double2
     }
     __shared__ Box sh[kBoxThreads / 32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) RB_AT(sh, wid, kBoxThreads / 32) = Box{mnx, mny, mxx, mxy};
+    if (lane == 0) RB_AT(sh, wid, kBoxThreads / 32) = Box{mnx, mny, mxx, mxy, odd};
     __syncthreads();
     if (threadIdx.x == 0) {
         Box r = sh[0];
@@ -76,6 +88,7 @@ __global__ void __launch_bounds__(kBoxThreads) bbox_partial_kernel(const double2
             r.mny = fmin(r.mny, sh[k].mny);
             r.mxx = fmax(r.mxx, sh[k].mxx);
             r.mxy = fmax(r.mxy, sh[k].mxy);
+            r.odd = fmax(r.odd, sh[k].odd);
         }
         part[blockIdx.x] = r;
     }
@@ -92,6 +105,7 @@ __global__ void __launch_bounds__(kBoxBlocks) grid_setup_kernel(const Box* __res
         r.mny = fmin(r.mny, __shfl_xor_sync(0xffffffffu, r.mny, o));
         r.mxx = fmax(r.mxx, __shfl_xor_sync(0xffffffffu, r.mxx, o));
         r.mxy = fmax(r.mxy, __shfl_xor_sync(0xffffffffu, r.mxy, o));
+        r.odd = fmax(r.odd, __shfl_xor_sync(0xffffffffu, r.odd, o));
     }
     __shared__ Box sh[kBoxBlocks / 32];
     if ((threadIdx.x & 31) == 0) RB_AT(sh, threadIdx.x >> 5, kBoxBlocks / 32) = r;
@@ -102,9 +116,11 @@ __global__ void __launch_bounds__(kBoxBlocks) grid_setup_kernel(const Box* __res
         r.mny = fmin(r.mny, sh[k].mny);
         r.mxx = fmax(r.mxx, sh[k].mxx);
         r.mxy = fmax(r.mxy, sh[k].mxy);
+        r.odd = fmax(r.odd, sh[k].odd);
     }
     double x0 = r.mnx, y0 = r.mny;
     double span = fmax(r.mxx - r.mnx, r.mxy - r.mny);
+    const bool finite_box = r.odd == 0.0 && x0 <= r.mxx && y0 <= r.mxy;
     if (!(x0 > -INFINITY && x0 < INFINITY)) x0 = 0.0;  // no finite point
     if (!(y0 > -INFINITY && y0 < INFINITY)) y0 = 0.0;
     if (!(span > 0.0 && span < INFINITY)) span = 1.0;    // single point / degenerate
@@ -114,10 +130,20 @@ __global__ void __launch_bounds__(kBoxBlocks) grid_setup_kernel(const Box* __res
     p.cell = span / G;
     p.inv_cell = G / span;
     p.margin = 1e-12 * (span + fabs(x0) + fabs(y0));
+    p.inv_fix = p.inv_cell * kFix;
     p.G = G;
-    p.pad = 0;
+    p.fast = finite_box && p.cell > 0.0 && p.inv_fix < INFINITY ? 1 : 0;
     *gp = p;
 }
+
+// Coordinate in units of cell / kFix, rounded down (NaN: 0; saturating).
+__device__ __forceinline__ int fix_coord(double v, double v0, double inv_fix) {
+    return __double2int_rd((v - v0) * inv_fix);
+}
+// Cell of a fixed-point coordinate, clamped to the grid: floor of the exact
+// product, since rounding down to kFix units and then to cells is rounding
+// down to cells.
+__device__ __forceinline__ int fix_cell(int u, int G) { return min(max(u >> kFixBits, 0), G - 1); }
 
 __device__ __forceinline__ int cell_coord(double v, double v0, double inv, int G) {
     const double t = floor((v - v0) * inv);
@@ -127,30 +153,40 @@ __device__ __forceinline__ int cell_coord(double v, double v0, double inv, int G
 }
 
 __global__ void cell_count_kernel(const double2* __restrict__ xy, int64_t N, const GridParams* __restrict__ gp,
-                                  int* __restrict__ keys, int* __restrict__ counts) {
+                                  int* __restrict__ counts) {
     const GridParams p = *gp;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
         const double2 q = xy[i];
-        const int cx = cell_coord(q.x, p.x0, p.inv_cell, p.G);
-        const int cy = cell_coord(q.y, p.y0, p.inv_cell, p.G);
-        const int key = cy * p.G + cx;
-        keys[i] = key;
-        atomicAdd(&RB_AT(counts, key, p.G * p.G), 1);
+        const int cx = fix_cell(fix_coord(q.x, p.x0, p.inv_fix), p.G);
+        const int cy = fix_cell(fix_coord(q.y, p.y0, p.inv_fix), p.G);
+        atomicAdd(&RB_AT(counts, cy * p.G + cx, p.G * p.G), 1);
     }
 }
 
 // counts[key] runs from the cell size down to 1, so positions fill
 // [start[key], start[key+1]) exactly once.  Order inside a cell is arbitrary;
 // stencils do not depend on it because the ranking key is a total order.
-__global__ void cell_scatter_kernel(const double2* __restrict__ xy, int64_t N, const int* __restrict__ keys,
-                                    const int* __restrict__ cell_start, int* __restrict__ counts, int64_t cells,
-                                    double2* __restrict__ sxy, int* __restrict__ sorig) {
+// su: the low 16 bits of both fixed-point coordinates (position modulo 16
+// cells).  cells_of (may be NULL): the cell (cy << 16 | cx) of point i goes
+// to cells_of[i * stride] (the first entry of its output row, which its query
+// overwrites).
+__global__ void cell_scatter_kernel(const double2* __restrict__ xy, int64_t N, const GridParams* __restrict__ gp,
+                                    const int* __restrict__ cell_start, int* __restrict__ counts,
+                                    double2* __restrict__ sxy, int* __restrict__ sorig, unsigned* __restrict__ su,
+                                    int* __restrict__ cells_of, int stride) {
+    const GridParams p = *gp;
+    const int64_t cells = (int64_t)p.G * p.G;
     (void)cells;  // bound of the checked build's tests
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-        const int key = keys[i];
+        const double2 q = xy[i];
+        const int ux = fix_coord(q.x, p.x0, p.inv_fix), uy = fix_coord(q.y, p.y0, p.inv_fix);
+        const int cx = fix_cell(ux, p.G), cy = fix_cell(uy, p.G);
+        const int key = cy * p.G + cx;
         const int pos = RB_AT(cell_start, key + 1, cells + 1) - atomicSub(&RB_AT(counts, key, cells), 1);
-        RB_AT(sxy, pos, N) = xy[i];
+        RB_AT(sxy, pos, N) = q;
         RB_AT(sorig, pos, N) = (int)i;
+        RB_AT(su, pos, N) = ((unsigned)uy << 16) | ((unsigned)ux & 0xffffu);
+        if (cells_of) cells_of[i * stride] = cy << 16 | cx;
     }
 }
 
@@ -317,16 +353,41 @@ constexpr int kMergeBatch = 16;
 // that an exact bound would have skipped.  (On this chip the FP64 units issue
 // 2 lanes per clock per SM: per-cell FP64 bounds and one-cell candidate
 // batches made the search FP64-bound.)
+//
+// chunk > 0: only the queries that knn_fast_kernel left (first entry kLeft),
+// a warp looks at `chunk` consecutive queries; chunk = 0: every query, one
+// per warp.
+constexpr int kLeft = -1;
+template <int SLOTS>
+__device__ __forceinline__ void knn_query(const double2* __restrict__ sxy, const int* __restrict__ sorig,
+                                          const int* __restrict__ cell_start, int Np, const GridParams& p, int Nq,
+                                          const double2* __restrict__ qxy, const int* __restrict__ qorig, int n,
+                                          int R0, int* __restrict__ idx, int q, int lane);
 template <int SLOTS>
 __global__ void __launch_bounds__(256) knn_kernel(const double2* __restrict__ sxy, const int* __restrict__ sorig,
                                                   const int* __restrict__ cell_start, int Np,
                                                   const GridParams* __restrict__ gp, int Nq,
                                                   const double2* __restrict__ qxy, const int* __restrict__ qorig,
-                                                  int n, int R0, int* __restrict__ idx) {
+                                                  int n, int R0, int* __restrict__ idx, int chunk) {
     const int lane = threadIdx.x & 31;
-    const int q = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (q >= Nq) return;
+    const int warp = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const GridParams p = *gp;
+    if (chunk == 0) {
+        if (warp < Nq) knn_query<SLOTS>(sxy, sorig, cell_start, Np, p, Nq, qxy, qorig, n, R0, idx, warp, lane);
+        return;
+    }
+    const int64_t q = (int64_t)warp * chunk + lane;
+    bool left = false;
+    if (lane < chunk && q < Nq) left = idx[(int64_t)(qorig ? qorig[q] : (int)q) * n] == kLeft;
+    for (unsigned m = __ballot_sync(0xffffffffu, left); m; m &= m - 1)
+        knn_query<SLOTS>(sxy, sorig, cell_start, Np, p, Nq, qxy, qorig, n, R0, idx, warp * chunk + __ffs(m) - 1, lane);
+}
+
+template <int SLOTS>
+__device__ __forceinline__ void knn_query(const double2* __restrict__ sxy, const int* __restrict__ sorig,
+                                          const int* __restrict__ cell_start, int Np, const GridParams& p, int Nq,
+                                          const double2* __restrict__ qxy, const int* __restrict__ qorig, int n,
+                                          int R0, int* __restrict__ idx, int q, int lane) {
     const double2 Q = qxy[q];
     const int qo = qorig ? qorig[q] : q;
     const int G = p.G;
@@ -462,6 +523,300 @@ __global__ void __launch_bounds__(256) knn_kernel(const double2* __restrict__ sx
     }
 }
 
+// ---------------------------------------------------------------------------
+// The search of most queries (n <= 112): select first, sort once.
+//
+// A warp reads the cells that meet a disk around the query, its radius from
+// the point count of the 3 x 3 cells there, and keeps the candidates' integer
+// squared distances (fixed-point coordinates modulo 16 cells, 4 bytes per
+// point) in registers, one row of cells per slot.  A threshold with n to
+// 32 SLOTS candidates below it is found by counting (ballots); the fixed-point
+// distances are within kErr units of the exact ones, so the candidates below
+// the threshold plus 2 kErr contain the n nearest.  Only those are ranked:
+// exact FP64 keys, one bitonic sort of 64-bit words (the leading bits of d^2
+// and the candidate's number; equal leading bits: the full keys are sorted).
+// A query whose candidates do not fit (strongly graded points, fewer than n
+// points in reach) is left to knn_kernel.
+// The block-first search above executes 5k to 9k warp instructions per query,
+// most of them sorting and merging batches into the list; this one about 900.
+// 300k nodes, n = 45: 1,603 -> 383 us; 1M nodes, n = 30: 4.9 -> 1.26 ms; the
+// multigrid's coarse and interpolation searches there 5.5 -> 1.3 ms.
+constexpr float kErr = 1.5f;     // > sqrt(2): each coordinate is rounded down by less than a unit
+constexpr float kReach = 6.5f;   // cells: differences stay inside the 16-cell wrap
+
+template <int SLOTS>
+__device__ __forceinline__ void sort_words(unsigned long long (&key)[SLOTS], int lane) {
+#pragma unroll
+    for (int k = 2; k <= 32 * SLOTS; k <<= 1) {
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            if (j >= 32) {
+                const int js = j / 32;
+#pragma unroll
+                for (int s = 0; s < SLOTS; ++s)
+                    if ((s & js) == 0) {
+                        const bool up = ((s * 32) & k) == 0;
+                        const unsigned long long a = key[s], b = key[s ^ js];
+                        const bool swap = (a > b) == up;
+                        key[s] = swap ? b : a;
+                        key[s ^ js] = swap ? a : b;
+                    }
+            } else {
+#pragma unroll
+                for (int s = 0; s < SLOTS; ++s) {
+                    const unsigned long long o = __shfl_xor_sync(0xffffffffu, key[s], j);
+                    const bool low = ((lane & j) == 0) == (((s * 32 + lane) & k) == 0);  // this lane keeps the smaller
+                    key[s] = (o < key[s]) == low ? o : key[s];
+                }
+            }
+        }
+    }
+}
+
+// The same network on full keys (d, j).
+template <int SLOTS>
+__device__ __noinline__ void sort_keys(unsigned long long* kd, unsigned* kj, int lane) {
+    unsigned long long d[SLOTS];
+    unsigned jj[SLOTS];
+#pragma unroll
+    for (int s = 0; s < SLOTS; ++s) {
+        d[s] = kd[s * 32 + lane];
+        jj[s] = kj[s * 32 + lane];
+    }
+    for (int k = 2; k <= 32 * SLOTS; k <<= 1)
+        for (int j = k >> 1; j > 0; j >>= 1) {
+#pragma unroll
+            for (int s = 0; s < SLOTS; ++s) {
+                kd[s * 32 + lane] = d[s];
+                kj[s * 32 + lane] = jj[s];
+            }
+            __syncwarp();
+#pragma unroll
+            for (int s = 0; s < SLOTS; ++s) {
+                const int e = s * 32 + lane, o = e ^ j;
+                const unsigned long long od = kd[o];
+                const unsigned oj = kj[o];
+                const bool low = ((e & j) == 0) == ((e & k) == 0);
+                if (key_less(od, oj, d[s], jj[s]) == low && !(od == d[s] && oj == jj[s])) {
+                    d[s] = od;
+                    jj[s] = oj;
+                }
+            }
+            __syncwarp();
+        }
+#pragma unroll
+    for (int s = 0; s < SLOTS; ++s) {
+        kd[s * 32 + lane] = d[s];
+        kj[s * 32 + lane] = jj[s];
+    }
+    __syncwarp();
+}
+
+// qxy NULL: the queries are the indexed points in cell order (row sorig[q],
+// whose first entry holds the point's cell); else Nq separate points.
+template <int SLOTS>
+__global__ void __launch_bounds__(256) knn_fast_kernel(const double2* __restrict__ sxy,
+                                                       const int* __restrict__ sorig,
+                                                       const unsigned* __restrict__ su,
+                                                       const int* __restrict__ cell_start, int Np,
+                                                       const GridParams* __restrict__ gp, int Nq,
+                                                       const double2* __restrict__ qxy, int n,
+                                                       int* __restrict__ idx) {
+    constexpr int CAP = 32 * SLOTS;          // candidates that are ranked
+    constexpr int K = SLOTS == 4 ? 12 : SLOTS == 2 ? 10 : 8;  // register slots of candidates (rows of cells)
+    constexpr int IB = SLOTS == 4 ? 7 : 6;   // bits of a candidate's number
+    __shared__ unsigned long long sh_d[8][CAP];
+    __shared__ unsigned sh_j[8][CAP];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int q = blockIdx.x * 8 + wid;
+    if (q >= Nq) return;
+    (void)Np;  // bound of the checked build's tests
+    const GridParams p = *gp;
+    const int G = p.G;
+    const int qo = qxy ? q : sorig[q];
+    int* out = idx + (int64_t)qo * n;
+    RB_SPAN((int64_t)qo * n, n, (int64_t)Nq * n);
+    int ux, uy;  // the query's fixed-point coordinates
+    double2 Q;
+    bool ok = p.fast != 0;
+    if (qxy) {
+        Q = qxy[q];
+        ux = fix_coord(Q.x, p.x0, p.inv_fix);
+        uy = fix_coord(Q.y, p.y0, p.inv_fix);
+        // (far outside the grid, or not a number: the other search)
+        ok = ok && ux > -8 * kFix && uy > -8 * kFix && ux < (G + 8) * kFix && uy < (G + 8) * kFix && finite64(Q.x) &&
+             finite64(Q.y);
+    } else {
+        Q = sxy[q];
+        const int cell = out[0], cx = cell & 0xffff, cy = cell >> 16;
+        const unsigned s = su[q];
+        ux = (cx << kFixBits) + (short)(unsigned short)(s - ((unsigned)cx << kFixBits));
+        uy = (cy << kFixBits) + (short)(unsigned short)((s >> 16) - ((unsigned)cy << kFixBits));
+    }
+    const int* cs = cell_start;
+    const int ncell = G * G + 1;
+    (void)ncell;
+    int cnt2 = 0;
+    if (ok) {
+        // density of the 3 x 3 cells around the query (cells outside the grid count as empty)
+        int near = 0;
+        {
+            const int yy = (uy >> kFixBits) - 1 + lane, x0 = max((ux >> kFixBits) - 1, 0),
+                      x1 = min((ux >> kFixBits) + 1, G - 1);
+            if (lane < 3 && yy >= 0 && yy < G && x0 <= x1)
+                near = RB_AT(cs, yy * G + x1 + 1, ncell) - RB_AT(cs, yy * G + x0, ncell);
+            near = __reduce_add_sync(0xffffffffu, near);
+        }
+        const float area = 9.0f / (3.14159265f * (float)max(near, 1));  // cells per point, over pi
+        float reach = sqrtf((float)n * area) * 1.08f + 0.12f;
+        ok = false;
+        for (int attempt = 0; attempt < 6 && reach <= kReach; ++attempt, reach *= 1.3f) {
+            const float rf = reach * (float)kFix;
+            const int ri = (int)rf + 2;
+            const int y0 = (uy - ri) >> kFixBits, nr = ((uy + ri) >> kFixBits) - y0 + 1;
+            // lane r: the columns of row y0 + r that the disk meets
+            int beg = 0, len = 0;
+            {
+                const int yy = y0 + lane;
+                if (lane < nr && yy >= 0 && yy < G) {
+                    const int lo = yy << kFixBits;
+                    const float dy = (float)max(0, max(lo - uy - 1, uy - lo - kFix));
+                    const int half = (int)sqrtf(fmaxf(rf * rf - dy * dy, 0.f)) + 3;
+                    const int xl = max((ux - half) >> kFixBits, 0), xh = min((ux + half) >> kFixBits, G - 1);
+                    if (xl <= xh) {
+                        beg = RB_AT(cs, yy * G + xl, ncell);
+                        len = RB_AT(cs, yy * G + xh + 1, ncell) - beg;
+                    }
+                }
+            }
+            // candidates: one row (or 32 points of it) per slot
+            unsigned d[K];
+            int pos[K];
+            int r = 0, off = 0;
+#pragma unroll
+            for (int s = 0; s < K; ++s) {
+                pos[s] = -1;
+                d[s] = 0xffffffffu;
+                if (r < nr) {
+                    const int b = __shfl_sync(0xffffffffu, beg, r) + off, l = __shfl_sync(0xffffffffu, len, r) - off;
+                    if (lane < l) {
+                        pos[s] = b + lane;
+                        const unsigned v = RB_AT(su, b + lane, Np);
+                        const int ex = (int)(short)(unsigned short)(v - (unsigned)ux);
+                        const int ey = (int)(short)(unsigned short)((v >> 16) - (unsigned)uy);
+                        d[s] = (unsigned)(ex * ex) + (unsigned)(ey * ey);
+                    }
+                    off += 32;
+                    if (l <= 32) {
+                        ++r;
+                        off = 0;
+                    }
+                }
+            }
+            if (r < nr) break;  // more candidates than slots
+            auto count = [&](unsigned T) -> int {
+                int c = 0;
+#pragma unroll
+                for (int s = 0; s < K; ++s) c += __popc(__ballot_sync(0xffffffffu, d[s] <= T));
+                return c;
+            };
+            const float tmax = (rf - 2.0f * kErr) * (rf - 2.0f * kErr);
+            const float target = (float)n + fminf(5.0f, 0.4f * (float)(CAP - n));
+            float lo = 0.f, hi = tmax, T = fminf(target * area * (float)kFix * (float)kFix, tmax);
+            bool grow = false;
+            for (int step = 0; step < 12; ++step) {
+                const int c = count((unsigned)T);
+                if (c < n) {
+                    if (T >= tmax) {
+                        grow = true;
+                        break;
+                    }
+                    lo = T;
+                } else {
+                    // everything nearer than the n-th may be: sqrt(T) + 2 kErr
+                    const float root = sqrtf(T) * 1.000001f + 2.0f * kErr + 0.5f;
+                    const unsigned T2 = (unsigned)(root * root * 1.000001f) + 1u;
+                    cnt2 = count(T2);
+                    if (cnt2 <= CAP) {
+                        int base = 0;
+#pragma unroll
+                        for (int s = 0; s < K; ++s) {
+                            const bool in = d[s] <= T2;
+                            const unsigned m = __ballot_sync(0xffffffffu, in);
+                            if (in) RB_AT(sh_j[wid], base + __popc(m & ((1u << lane) - 1u)), CAP) = (unsigned)pos[s];
+                            base += __popc(m);
+                        }
+                        ok = true;
+                        break;
+                    }
+                    hi = T;
+                }
+                const float next = T * target / (float)max(c, 1);
+                T = next > lo && next < hi ? next : (c < n && hi == tmax && next >= hi ? tmax : 0.5f * (lo + hi));
+            }
+            if (ok || !grow) break;
+        }
+    }
+    if (!ok) {
+        __syncwarp();
+        if (lane == 0) out[0] = kLeft;
+        return;
+    }
+    __syncwarp();
+    // rank the candidates by their exact keys
+    unsigned long long key[SLOTS];
+    unsigned long long kd[SLOTS];
+    unsigned kj[SLOTS];
+#pragma unroll
+    for (int s = 0; s < SLOTS; ++s) {
+        const int e = s * 32 + lane;
+        kd[s] = ~0ull;
+        kj[s] = ~0u;
+        if (e < cnt2) {
+            const int at = (int)sh_j[wid][e];
+            const double2 P = RB_AT(sxy, at, Np);
+            const double dx = __dadd_rn(P.x, -Q.x);
+            const double dy = __dadd_rn(P.y, -Q.y);
+            const double d2 = __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
+            kd[s] = (unsigned long long)__double_as_longlong(d2) & 0x7fffffffffffffffull;
+            kj[s] = (unsigned)RB_AT(sorig, at, Np);
+        }
+        // ((d^2 bits << 1) without its last IB bits, number)
+        key[s] = e < cnt2 ? (((kd[s] << 1) >> IB) << IB) | (unsigned long long)e : ~0ull;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int s = 0; s < SLOTS; ++s) sh_j[wid][s * 32 + lane] = kj[s];
+    sort_words<SLOTS>(key, lane);
+    // equal leading bits among the first n (or across its end): the full keys decide
+    bool tie = false;
+#pragma unroll
+    for (int s = 0; s < SLOTS; ++s) {
+        unsigned long long nx = __shfl_down_sync(0xffffffffu, key[s], 1);
+        if (s + 1 < SLOTS) {
+            const unsigned long long first = __shfl_sync(0xffffffffu, key[s + 1 < SLOTS ? s + 1 : 0], 0);
+            if (lane == 31) nx = first;
+        } else if (lane == 31) {
+            nx = ~0ull;
+        }
+        tie |= s * 32 + lane < n && s * 32 + lane + 1 < cnt2 && (key[s] >> IB) == (nx >> IB);
+    }
+    __syncwarp();
+    if (__any_sync(0xffffffffu, tie)) {
+#pragma unroll
+        for (int s = 0; s < SLOTS; ++s) sh_d[wid][s * 32 + lane] = kd[s];
+        __syncwarp();
+        sort_keys<SLOTS>(sh_d[wid], sh_j[wid], lane);
+        for (int e = lane; e < n; e += 32) out[e] = (int)sh_j[wid][e];
+        return;
+    }
+#pragma unroll
+    for (int s = 0; s < SLOTS; ++s) {
+        const int e = s * 32 + lane;
+        if (e < n) out[e] = (int)RB_AT(sh_j[wid], (int)(key[s] & ((1u << IB) - 1u)), CAP);
+    }
+}
+
 // Block radius of the first search phase: about n points in (2 R0 + 1)^2
 // cells at ~3 points per cell, plus half a cell.
 int block_radius(int n) { return std::max(1, (int)std::ceil(std::sqrt((double)n / (3.0 * 3.14159265358979)) + 0.5)); }
@@ -479,7 +834,7 @@ int grid_side(int64_t N, int n) {
 struct KnnLayout {
     GridParams* gp;
     Box* part;
-    int* keys;
+    unsigned* su;
     int* counts;
     int* cell_start;
     int* sums;
@@ -495,7 +850,7 @@ KnnLayout knn_layout(void* ws, int64_t N, int n) {
     KnnLayout L;
     L.gp = c.take<GridParams>(1);
     L.part = c.take<Box>(kBoxBlocks);
-    L.keys = c.take<int>(N);
+    L.su = c.take<unsigned>(N);
     L.counts = c.take<int>(cells);
     L.cell_start = c.take<int>(cells + 1);
     L.sums = c.take<int>(scan_tiles(cells) + 1);
@@ -543,20 +898,36 @@ int rbffd::knn_search(const double* xy, int64_t N, const double* qxy, int64_t Nq
     bbox_partial_kernel<<<kBoxBlocks, kBoxThreads, 0, st>>>(p, N, L.part);
     grid_setup_kernel<<<1, kBoxBlocks, 0, st>>>(L.part, G, L.gp);
     RBFFD_CUDA_TRY(cudaMemsetAsync(L.counts, 0, sizeof(int) * cells, st));
-    cell_count_kernel<<<grid_pts, 256, 0, st>>>(p, N, L.gp, L.keys, L.counts);
+    cell_count_kernel<<<grid_pts, 256, 0, st>>>(p, N, L.gp, L.counts);
     RBFFD_CUDA_TRY(exclusive_scan<int>(CountLoad{L.counts}, cells, L.cell_start, L.sums, L.cell_start + cells, st));
-    cell_scatter_kernel<<<grid_pts, 256, 0, st>>>(p, N, L.keys, L.cell_start, L.counts, cells, L.sxy, L.sorig);
-    const int warps_per_block = 8;
-    const int blocks = (int)((Nq + warps_per_block - 1) / warps_per_block);
+    cell_scatter_kernel<<<grid_pts, 256, 0, st>>>(p, N, L.gp, L.cell_start, L.counts, L.sxy, L.sorig, L.su,
+                                                  qxy ? nullptr : idx, n);
     const double2* q = qxy ? reinterpret_cast<const double2*>(qxy) : L.sxy;
     const int* qo = qxy ? nullptr : L.sorig;
     const int R0 = block_radius(n);
+    // ranked candidates: a few more than n, in whole warps
+    const int blocks = (int)((Nq + 7) / 8);
+    const bool fast = n <= 112;
+    if (fast) {
+        const double2* fq = reinterpret_cast<const double2*>(qxy);
+        if (n <= 24)
+            knn_fast_kernel<1><<<blocks, 256, 0, st>>>(L.sxy, L.sorig, L.su, L.cell_start, (int)N, L.gp, (int)Nq, fq, n, idx);
+        else if (n <= 56)
+            knn_fast_kernel<2><<<blocks, 256, 0, st>>>(L.sxy, L.sorig, L.su, L.cell_start, (int)N, L.gp, (int)Nq, fq, n, idx);
+        else
+            knn_fast_kernel<4><<<blocks, 256, 0, st>>>(L.sxy, L.sorig, L.su, L.cell_start, (int)N, L.gp, (int)Nq, fq, n, idx);
+    }
+    // queries per warp of the second pass: enough warps to fill the chip
+    const int chunk = fast ? (int)std::min<int64_t>(32, std::max<int64_t>(1, Nq / 16384)) : 0;
+    const int64_t warps = fast ? (Nq + chunk - 1) / chunk : Nq;
+    const int rest = (int)((warps + 7) / 8);
     if (n <= 32)
-        knn_kernel<1><<<blocks, 256, 0, st>>>(L.sxy, L.sorig, L.cell_start, (int)N, L.gp, (int)Nq, q, qo, n, R0, idx);
+        knn_kernel<1><<<rest, 256, 0, st>>>(L.sxy, L.sorig, L.cell_start, (int)N, L.gp, (int)Nq, q, qo, n, R0, idx, chunk);
     else if (n <= 64)
-        knn_kernel<2><<<blocks, 256, 0, st>>>(L.sxy, L.sorig, L.cell_start, (int)N, L.gp, (int)Nq, q, qo, n, R0, idx);
+        knn_kernel<2><<<rest, 256, 0, st>>>(L.sxy, L.sorig, L.cell_start, (int)N, L.gp, (int)Nq, q, qo, n, R0, idx, chunk);
     else
-        knn_kernel<4><<<blocks, 256, 0, st>>>(L.sxy, L.sorig, L.cell_start, (int)N, L.gp, (int)Nq, q, qo, n, R0, idx);
+        knn_kernel<4><<<rest, 256, 0, st>>>(L.sxy, L.sorig, L.cell_start, (int)N, L.gp, (int)Nq, q, qo, n, R0, idx, chunk);
+    note_launches(fast ? 1 : 0);
     note_launches(5);  // bbox, setup, count, scatter, knn (+3 in the scan)
     RBFFD_LAUNCH_CHECK();
     return RBFFD_OK;
