@@ -86,7 +86,7 @@ struct MbTask {
 namespace {
 
 constexpr int kMbT = 256;         // threads per block (8 warps)
-constexpr int kMbTileRows = 256;  // rows per unit
+constexpr int kMbTileRows = 256;  // rows per unit at most (and per task of the persistent kernel)
 constexpr int kMbDenseRows = 16;  // rows per unit of the dense coarsest solves
 enum : int8_t { kOpFirst = 0, kOpSweep = 1, kOpResid = 2, kOpRestrict = 3, kOpProlong = 4, kOpDense = 5 };
 constexpr long long kMbDefaultSpin = 1LL << 26;  // polls of a bounded wait (~seconds with the back-off)
@@ -450,12 +450,27 @@ int64_t coarse_task_bound(int n_inst, int64_t total_nodes) {
 int64_t counter_bound(int n_inst) { return (int64_t)n_inst * (11 * RBFFD_MG_MAX_LEVELS + 2); }
 }  // namespace
 
+// Rows per unit of a launch over `rows` rows: enough units to fill the chip.
+// A warp takes rows one after the other, each a chain of dependent gathers:
+// with 256 rows per unit the restriction into 100k rows ran 390 blocks of 32
+// rows per warp, four times as long as its gathers' bandwidth.
+static int unit_rows(int64_t rows) {
+    constexpr int64_t kUnits = 152 * 16;
+    int per = kMbTileRows;
+    while (per > 8 && rows / per < kUnits) per /= 2;
+    return per;
+}
+
 size_t mg_batch_table_bytes(int n_inst, int64_t total_nodes) {
-    // units of every level (the levels of one instance hold fewer than twice
-    // its nodes; the restriction's sets fewer than its nodes), plus partial
-    // tiles and the dense tiles
-    const int64_t units = 3 * (total_nodes / kMbTileRows + 1) + 3 * (int64_t)n_inst * RBFFD_MG_MAX_LEVELS +
-                          (int64_t)n_inst * (kMgCoarsest / kMbDenseRows + 1);
+    // units: per level l at most total_nodes / 2^l rows, its own and (from the
+    // level above) the restriction's, each with partial tiles per instance;
+    // plus the dense tiles
+    int64_t units = (int64_t)n_inst * (kMgCoarsest / kMbDenseRows + 1);
+    for (int l = 0; l < RBFFD_MG_MAX_LEVELS; ++l) {
+        // (fewer rows only lower the rows per unit, so not the unit count's bound)
+        const int64_t rows = total_nodes >> l;
+        units += 2 * (std::max(rows / kMbTileRows, std::min<int64_t>(rows / 8, 2 * 152 * 16)) + 1 + n_inst);
+    }
     return align_up((size_t)n_inst * RBFFD_MG_MAX_LEVELS * sizeof(MbLevel)) + align_up((size_t)units * sizeof(MbUnit)) +
            align_up((size_t)coarse_task_bound(n_inst, total_nodes) * sizeof(MbTask)) +
            align_up((size_t)(counter_bound(n_inst) + 4) * sizeof(int));
@@ -545,9 +560,15 @@ int mg_batch_build(const MgHierarchy* const* H, const int64_t* node_off, int n_i
         }
     };
     for (int l = 0; l < lmax; ++l) {
+        int64_t rows = 0, rows_next = 0;
+        for (int i = 0; i < n_inst; ++i)
+            if (H[i]->n_levels - 1 > l) {
+                rows += H[i]->lv[l].N;
+                rows_next += H[i]->lv[l + 1].N;
+            }
         B.a_off[l] = (int)units.size();
         for (int i = 0; i < n_inst; ++i)
-            if (H[i]->n_levels - 1 > l) tiles(units, i, l, H[i]->lv[l].N, kMbTileRows);
+            if (H[i]->n_levels - 1 > l) tiles(units, i, l, H[i]->lv[l].N, unit_rows(rows));
         B.a_n[l] = (int)units.size() - B.a_off[l];
         B.d_off[l] = (int)units.size();
         for (int i = 0; i < n_inst; ++i)
@@ -555,7 +576,7 @@ int mg_batch_build(const MgHierarchy* const* H, const int64_t* node_off, int n_i
         B.d_n[l] = (int)units.size() - B.d_off[l];
         B.c_off[l] = (int)units.size();
         for (int i = 0; i < n_inst; ++i)
-            if (H[i]->n_levels - 1 > l) tiles(units, i, l, H[i]->lv[l + 1].N, kMbTileRows);
+            if (H[i]->n_levels - 1 > l) tiles(units, i, l, H[i]->lv[l + 1].N, unit_rows(rows_next));
         B.c_n[l] = (int)units.size() - B.c_off[l];
     }
     // the coarse levels' phases per instance (levels 1 .. L-1): descend --
