@@ -213,40 +213,47 @@ __global__ void __launch_bounds__(kT) mg_restrict_kernel(const int64_t* __restri
     chained_rows<T, TPR, HEAD>(row_ptr, col, val, n, r, nr, flag, [&](int64_t i, T v) { y[i] = v; });
 }
 
-// x += P e (ELL, kMgK entries per row)
+// A row of the prolongation (ELL, kMgK entries), by 16-byte loads.
 template <typename T>
-__global__ void __launch_bounds__(kT) mg_prolong_kernel(int64_t N, const int32_t* __restrict__ pidx,
-                                                        const T* __restrict__ pval, const T* __restrict__ e,
-                                                        int64_t ne, T* __restrict__ x, const int* flag) {
-    (void)ne;  // length of e: bound of the checked build's tests
-    // the first row's entries before the wait (three 16-byte loads of each array)
+struct PRow {
     static_assert(kMgK % 4 == 0, "rows of whole 16-byte loads");
-    int4 c[kMgK / 4];
+    int c[kMgK];
     T v[kMgK];
-    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    auto load = [&](int64_t i) {
+    __device__ __forceinline__ PRow() {}
+    __device__ __forceinline__ PRow(const int32_t* __restrict__ pidx, const T* __restrict__ pval, int64_t i) {
 #pragma unroll
-        for (int j = 0; j < kMgK / 4; ++j) c[j] = __ldg(reinterpret_cast<const int4*>(pidx + i * kMgK) + j);
+        for (int j = 0; j < kMgK / 4; ++j) {
+            const int4 q = __ldg(reinterpret_cast<const int4*>(pidx + i * kMgK) + j);
+            c[4 * j] = q.x;
+            c[4 * j + 1] = q.y;
+            c[4 * j + 2] = q.z;
+            c[4 * j + 3] = q.w;
+        }
 #pragma unroll
         for (int j = 0; j < (int)(kMgK * sizeof(T) / 16); ++j) {
             const float4 q = __ldg(reinterpret_cast<const float4*>(pval + i * kMgK) + j);
             memcpy(reinterpret_cast<char*>(v) + 16 * j, &q, 16);
         }
-    };
-    if (i0 < N) load(i0);
+    }
+};
+
+// x += P e; the first row's entries are loaded before the wait
+template <typename T>
+__global__ void __launch_bounds__(kT) mg_prolong_kernel(int64_t N, const int32_t* __restrict__ pidx,
+                                                        const T* __restrict__ pval, const T* __restrict__ e,
+                                                        int64_t ne, T* __restrict__ x, const int* flag) {
+    (void)ne;  // length of e: bound of the checked build's tests
+    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    PRow<T> p;
+    if (i0 < N) p = PRow<T>(pidx, pval, i0);
     pdl_wait();
     pdl_next();
     if (stopped(flag)) return;
     MG_ELEMS(N, i) {
-        if (i != i0) load(i);
+        if (i != i0) p = PRow<T>(pidx, pval, i);
         T acc = x[i];
 #pragma unroll
-        for (int j = 0; j < kMgK / 4; ++j) {
-            acc = fmaT<T>(v[4 * j], __ldg(&RB_AT(e, c[j].x, ne)), acc);
-            acc = fmaT<T>(v[4 * j + 1], __ldg(&RB_AT(e, c[j].y, ne)), acc);
-            acc = fmaT<T>(v[4 * j + 2], __ldg(&RB_AT(e, c[j].z, ne)), acc);
-            acc = fmaT<T>(v[4 * j + 3], __ldg(&RB_AT(e, c[j].w, ne)), acc);
-        }
+        for (int j = 0; j < kMgK; ++j) acc = fmaT<T>(p.v[j], __ldg(&RB_AT(e, p.c[j], ne)), acc);
         x[i] = acc;
     }
 }
@@ -1181,14 +1188,18 @@ void restrict_to(const MgLevel& L, int64_t nc, const T* r, T* bc, const int* fla
 // memory: a level of some hundred nodes is a few microseconds of launch
 // latency per operation (six per level) and a fraction of one of work.  Every
 // row is summed by the same lanes in the same order as in the kernels above,
-// so the result has the same bits.
-// 845 + 190 + 45 rows: 23 us, 14 launches before.  (A cluster of 16 blocks, up
+// so the result has the same bits.  The operators, read by every sweep, and
+// as many of the transfers as fit are copied to shared memory while the
+// previous kernel of the chain still runs (a batch of rows read from L2 is
+// two or three dependent round trips of ~700 cycles: the restriction alone
+// took 6.5k cycles).
+// 845 + 190 + 45 rows: 15 to 20 us, 14 launches of 3 before.  (A cluster of 16 blocks, up
 // to 20k rows, took 88 us for five levels: its barrier costs 600 to 1,700
 // cycles and a neighbour in another block's shared memory or in L2 500 to
 // 700, once per operation and entry.)
 constexpr int kTailT = 1024;
 constexpr int kTailLevels = 16;
-constexpr int kTailSmem = 64 * 1024;  // leaves the rest of L1 to the matrices
+constexpr int kTailSmem = 208 * 1024;
 
 template <typename T>
 struct TailLevel {
@@ -1205,9 +1216,20 @@ struct TailLevel {
     const T* rval;
 };
 
+// An array that the kernel copies to shared memory first.
+struct TailCopy {
+    const void* src;
+    int bytes, dst;
+};
+constexpr int kTailCopies = 24;
+
 template <typename T>
 struct TailCycle {
-    int levels, nu;
+    int levels, nu, copies;
+    TailCopy copy[kTailCopies];
+    // byte offsets of the copies in shared memory, -1: read from global memory
+    int a_ptr[kTailLevels], a_col[kTailLevels], a_val[kTailLevels];
+    int r_ptr[kTailLevels], r_col[kTailLevels], r_val[kTailLevels];
     const T* minv;
     const T* b;  // right-hand side and result of the first level (not TOP)
     T* x;
@@ -1215,40 +1237,45 @@ struct TailCycle {
 };
 
 // Rows of a CSR matrix by one block, TPR lanes per row: f(i, sum) in one lane.
-template <typename T, int TPR, class F>
-__device__ __forceinline__ void tail_rows(const int64_t* __restrict__ row_ptr, const int* __restrict__ col,
-                                          const T* __restrict__ val, const T* x, int nx, int n, F&& f) {
+template <typename T, int TPR, class RP, class CP, class F>
+__device__ __forceinline__ void tail_rows(const RP* row_ptr, const CP* col, const T* val, const T* x, int nx, int n,
+                                          F&& f) {
     (void)nx;  // length of x: bound of the checked build's tests
     const int sub = threadIdx.x & (TPR - 1), off = (threadIdx.x & 31) / TPR;
     for (int base = (int)threadIdx.x / TPR - off; base < n; base += kTailT / TPR) {
         const int i = base + off;
-        int64_t a = 0, e = 0;
+        int a = 0, e = 0;
         if (i < n) {
-            a = __ldg(row_ptr + i);
-            e = __ldg(row_ptr + i + 1);
+            a = (int)row_ptr[i];
+            e = (int)row_ptr[i + 1];
         }
         T sum = T(0);
-#pragma unroll 4
-        for (int64_t k = a + sub; k < e; k += TPR) sum = fmaT<T>(__ldg(val + k), RB_AT(x, __ldg(col + k), nx), sum);
+        // batches of independent loads; the sum runs in the order of the entries
+        for (int k = a + sub; k < e; k += 6 * TPR) {
+            T v[6], xv[6];
+#pragma unroll
+            for (int u = 0; u < 6; ++u) {
+                const bool in = k + u * TPR < e;
+                v[u] = in ? val[k + u * TPR] : T(0);
+                xv[u] = in ? RB_AT(x, (int)col[k + u * TPR], nx) : T(0);
+            }
+#pragma unroll
+            for (int u = 0; u < 6; ++u)
+                if (k + u * TPR < e) sum = fmaT<T>(v[u], xv[u], sum);
+        }
 #pragma unroll
         for (int o = TPR / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o, TPR);
         if (i < n && sub == 0) f(i, sum);
     }
 }
 
-template <typename T, class F>
-__device__ __forceinline__ void tail_csr(int tpr, const int64_t* row_ptr, const int* col, const T* val, const T* x,
-                                         int nx, int n, F&& f) {
+template <typename T, class RP, class CP, class F>
+__device__ __forceinline__ void tail_csr(int tpr, const RP* row_ptr, const CP* col, const T* val, const T* x, int nx,
+                                         int n, F&& f) {
     if (tpr == 8) tail_rows<T, 8>(row_ptr, col, val, x, nx, n, f);
     else if (tpr == 4) tail_rows<T, 4>(row_ptr, col, val, x, nx, n, f);
     else if (tpr == 2) tail_rows<T, 2>(row_ptr, col, val, x, nx, n, f);
     else tail_rows<T, 1>(row_ptr, col, val, x, nx, n, f);
-}
-
-__device__ __forceinline__ void tail_prefetch(const void* p, int64_t bytes) {
-    const char* c = static_cast<const char*>(p);
-    for (int64_t o = (int64_t)threadIdx.x * 128; o < bytes; o += (int64_t)kTailT * 128)
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(c + o));
 }
 
 // TOP: level 0 is the first one, its right-hand side and result are the
@@ -1260,15 +1287,25 @@ __global__ void __launch_bounds__(kTailT) mg_tail_kernel(const __grid_constant__
     extern __shared__ __align__(16) unsigned char tail_smem[];
     T* vec = reinterpret_cast<T*>(tail_smem);  // per level: two iterates, residual, right-hand side
     const int tid = (int)threadIdx.x, last = c.levels - 1;
-    for (int l = 0; l < last; ++l) {
-        const TailLevel<T>& L = c.lv[l];
-        const int64_t rn = (int64_t)L.n * kMgK;
-        tail_prefetch(L.row_ptr, (L.n + 1) * 8);
-        tail_prefetch(L.col, L.nnz * 4);
-        tail_prefetch(L.val, L.nnz * (int64_t)sizeof(T));
-        tail_prefetch(L.rcol, rn * 4);
-        tail_prefetch(L.rval, rn * (int64_t)sizeof(T));
+    for (int k = 0; k < c.copies; ++k) {
+        const TailCopy& q = c.copy[k];
+        const char* src = static_cast<const char*>(q.src);
+        char* dst = reinterpret_cast<char*>(tail_smem) + q.dst;
+        const int whole = q.bytes & ~15;
+        for (int o = tid * 16; o < whole; o += kTailT * 16)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst + o)),
+                         "l"(src + o));
+        for (int o = whole + tid * 4; o < q.bytes; o += kTailT * 4)
+            *reinterpret_cast<int*>(dst + o) = *reinterpret_cast<const int*>(src + o);
     }
+    auto at = [&](int off, const auto* global) {
+        using P = decltype(global);
+        return off >= 0 ? reinterpret_cast<P>(tail_smem + off) : global;
+    };
+    auto a_ptr = [&](int l) { return at(c.a_ptr[l], c.lv[l].row_ptr); };
+    auto a_col = [&](int l) { return at(c.a_col[l], c.lv[l].col); };
+    auto a_val = [&](int l) { return at(c.a_val[l], c.lv[l].val); };
+    asm volatile("cp.async.wait_all;" ::: "memory");
     pdl_wait();
     pdl_next();
     if (stopped(flag)) return;
@@ -1282,16 +1319,17 @@ __global__ void __launch_bounds__(kTailT) mg_tail_kernel(const __grid_constant__
         for (int i = tid; i < n; i += kTailT) cur[i] = __ldg(L.w + i) * b[i];
         __syncthreads();
         for (int k = 1; k < c.nu; ++k) {
-            tail_csr<T>(L.tpr, L.row_ptr, L.col, L.val, cur, n, n,
+            tail_csr<T>(L.tpr, a_ptr(l), a_col(l), a_val(l), cur, n, n,
                         [&](int i, T ax) { oth[i] = fmaT<T>(__ldg(L.w + i), b[i] - ax, cur[i]); });
             T* s = cur;
             cur = oth;
             oth = s;
             __syncthreads();
         }
-        tail_csr<T>(L.tpr, L.row_ptr, L.col, L.val, cur, n, n, [&](int i, T ax) { r[i] = b[i] - ax; });
+        tail_csr<T>(L.tpr, a_ptr(l), a_col(l), a_val(l), cur, n, n, [&](int i, T ax) { r[i] = b[i] - ax; });
         __syncthreads();
-        tail_csr<T>(L.rtpr, L.rrow, L.rcol, L.rval, r, n, c.lv[l + 1].n, [&](int i, T s) { bc[i] = s; });
+        tail_csr<T>(L.rtpr, at(c.r_ptr[l], L.rrow), at(c.r_col[l], L.rcol), at(c.r_val[l], L.rval), r, n,
+                    c.lv[l + 1].n, [&](int i, T s) { bc[i] = s; });
         __syncthreads();
         v += 4 * n;
     }
@@ -1318,16 +1356,15 @@ __global__ void __launch_bounds__(kTailT) mg_tail_kernel(const __grid_constant__
         T* oth = v + ((c.nu & 1) ? n : 0);
         const T* b = v + 3 * n;
         for (int i = tid; i < n; i += kTailT) {
-            const int32_t* ip = L.pidx + (int64_t)i * kMgK;
-            const T* vp = L.pval + (int64_t)i * kMgK;
+            const PRow<T> p(L.pidx, L.pval, i);
             T acc = cur[i];
 #pragma unroll
-            for (int j = 0; j < kMgK; ++j) acc = fmaT<T>(__ldg(vp + j), RB_AT(e, __ldg(ip + j), nc), acc);
+            for (int j = 0; j < kMgK; ++j) acc = fmaT<T>(p.v[j], RB_AT(e, p.c[j], nc), acc);
             cur[i] = acc;
         }
         for (int k = 0; k < c.nu; ++k) {
             __syncthreads();
-            tail_csr<T>(L.tpr, L.row_ptr, L.col, L.val, cur, n, n,
+            tail_csr<T>(L.tpr, a_ptr(l), a_col(l), a_val(l), cur, n, n,
                         [&](int i, T ax) { oth[i] = fmaT<T>(__ldg(L.w + i), b[i] - ax, cur[i]); });
             T* s = cur;
             cur = oth;
@@ -1344,11 +1381,11 @@ __global__ void __launch_bounds__(kTailT) mg_tail_kernel(const __grid_constant__
 }
 
 // Matrix entries of the first level up to which one block takes it: a sweep
-// then costs about as long as a launch (the block reads ~64 bytes per clock
-// from L2; FP64: 2 multiply-adds per clock).
+// then costs less than a launch, and the operators fit shared memory (FP64: 2
+// multiply-adds per clock).
 template <typename T>
 constexpr int64_t tail_entries() {
-    return sizeof(T) == 8 ? 6144 : 24576;
+    return sizeof(T) == 8 ? 6144 : 12288;
 }
 
 // The cycle of levels [first, n_levels) in one launch; false where it does
@@ -1388,6 +1425,29 @@ bool tail_cycle(const MgHierarchy& h, int first, const double* b, double* x, con
         smem += 4 * (size_t)L.N * sizeof(T);
     }
     if (smem > kTailSmem) return false;
+    // copies while they fit: the operators first, then the restrictions
+    c.copies = 0;
+    auto take = [&](const void* src, size_t bytes) {
+        const size_t at = align_up(smem, 16);
+        if (c.copies >= kTailCopies || at + bytes > kTailSmem || ((uintptr_t)src & 15) != 0) return -1;
+        c.copy[c.copies++] = TailCopy{src, (int)bytes, (int)at};
+        smem = at + bytes;
+        return (int)at;
+    };
+    for (int l = 0; l < kTailLevels; ++l)
+        c.a_ptr[l] = c.a_col[l] = c.a_val[l] = c.r_ptr[l] = c.r_col[l] = c.r_val[l] = -1;
+    for (int l = 0; l + 1 < levels; ++l) {
+        const TailLevel<T>& t = c.lv[l];
+        c.a_val[l] = take(t.val, (size_t)t.nnz * sizeof(T));
+        c.a_col[l] = take(t.col, (size_t)t.nnz * sizeof(int));
+        c.a_ptr[l] = take(t.row_ptr, (size_t)(t.n + 1) * sizeof(int64_t));
+    }
+    for (int l = levels - 2; l >= 0; --l) {
+        const TailLevel<T>& t = c.lv[l];
+        c.r_col[l] = take(t.rcol, (size_t)t.n * kMgK * sizeof(int));
+        c.r_val[l] = take(t.rval, (size_t)t.n * kMgK * sizeof(T));
+        c.r_ptr[l] = take(t.rrow, (size_t)(c.lv[l + 1].n + 1) * sizeof(int64_t));
+    }
     if (cudaFuncSetAttribute(mg_tail_kernel<T, TOP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTailSmem) !=
         cudaSuccess)
         return false;
