@@ -39,6 +39,7 @@
 // and vectors (the mixed-precision solve: the preconditioner needs no FP64
 // accuracy, the outer FP64 BiCGSTAB keeps the residual exact).
 #include "common.cuh"
+#include "csr_rows.cuh"
 #include "internal.cuh"
 #include "scan.cuh"
 
@@ -148,15 +149,23 @@ struct RowHead {
 };
 
 // A chained kernel over the rows of a CSR matrix: f(i, sum) in one lane per
-// row, sum = (A x)_i.  HEAD: the first row's entries are loaded before the
+// row, sum = (A x)_i.  kRowHead: the first row's entries are loaded before the
 // wait (for launches whose lanes have one row each; it costs the registers
-// that hold 64 warps per SM in the large ones).
-template <typename T, int TPR, bool HEAD, class F>
+// that hold 64 warps per SM in the large ones).  kRow32: 32 rows per warp
+// (csr_rows.cuh; for launches of one lane per row that fill the chip).
+enum RowForm { kRowEach = 0, kRowHead = 1, kRow32 = 2 };
+template <typename T, int TPR, int FORM, class F>
 __device__ __forceinline__ void chained_rows(const int64_t* __restrict__ row_ptr, const int* __restrict__ col,
                                              const T* __restrict__ val, int64_t N, const T* __restrict__ x,
                                              int64_t nx, const int* flag, F&& f) {
     const int sub = threadIdx.x & (TPR - 1);
-    if constexpr (HEAD) {
+    if constexpr (FORM == kRow32) {
+        pdl_wait();
+        pdl_next();
+        if (stopped(flag)) return;
+        if constexpr (sizeof(T) == 4 && TPR == 8) rows32_ahead<T, TPR>(row_ptr, col, val, x, nx, N, f);
+        else rows32<T, TPR>(row_ptr, col, val, x, nx, N, f);
+    } else if constexpr (FORM == kRowHead) {
         const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / TPR;  // one row per group of lanes
         RowHead<T, TPR> head;
         head.load(row_ptr, col, val, i, sub, i < N);
@@ -187,30 +196,30 @@ __global__ void __launch_bounds__(kT) mg_first_kernel(int64_t N, const BT* __res
 }
 
 // xo = xi + W (b - A xi)
-template <typename T, typename BT, typename OT, int TPR, bool HEAD>
+template <typename T, typename BT, typename OT, int TPR, int FORM>
 __global__ void __launch_bounds__(kT) mg_jacobi_kernel(const int64_t* __restrict__ row_ptr, const int* __restrict__ col,
                                                        const T* __restrict__ val, int64_t N, const T* __restrict__ xi,
                                                        const BT* __restrict__ b, const T* __restrict__ dinv,
                                                        OT* __restrict__ xo, const int* flag) {
-    chained_rows<T, TPR, HEAD>(row_ptr, col, val, N, xi, N, flag,
+    chained_rows<T, TPR, FORM>(row_ptr, col, val, N, xi, N, flag,
                          [&](int64_t i, T ax) { xo[i] = (OT)fmaT<T>(dinv[i], (T)b[i] - ax, xi[i]); });
 }
 
 // r = b - A x
-template <typename T, typename BT, int TPR, bool HEAD>
+template <typename T, typename BT, int TPR, int FORM>
 __global__ void __launch_bounds__(kT) mg_resid_kernel(const int64_t* __restrict__ row_ptr, const int* __restrict__ col,
                                                       const T* __restrict__ val, int64_t N, const T* __restrict__ x,
                                                       const BT* __restrict__ b, T* __restrict__ r, const int* flag) {
-    chained_rows<T, TPR, HEAD>(row_ptr, col, val, N, x, N, flag, [&](int64_t i, T ax) { r[i] = (T)b[i] - ax; });
+    chained_rows<T, TPR, FORM>(row_ptr, col, val, N, x, N, flag, [&](int64_t i, T ax) { r[i] = (T)b[i] - ax; });
 }
 
 // y = R r (restriction, CSR with n rows)
-template <typename T, int TPR, bool HEAD>
+template <typename T, int TPR, int FORM>
 __global__ void __launch_bounds__(kT) mg_restrict_kernel(const int64_t* __restrict__ row_ptr,
                                                          const int* __restrict__ col, const T* __restrict__ val,
                                                          int64_t n, const T* __restrict__ r, int64_t nr,
                                                          T* __restrict__ y, const int* flag) {
-    chained_rows<T, TPR, HEAD>(row_ptr, col, val, n, r, nr, flag, [&](int64_t i, T v) { y[i] = v; });
+    chained_rows<T, TPR, FORM>(row_ptr, col, val, n, r, nr, flag, [&](int64_t i, T v) { y[i] = v; });
 }
 
 // A row of the prolongation (ELL, kMgK entries), by 16-byte loads.
@@ -1139,17 +1148,38 @@ struct Sel<float> {
     static float* b(const MgLevel& L) { return L.b32; }
 };
 
-// Launches whose rows are at most this many groups' lanes load the rows
-// before the wait for the previous kernel (all lanes resident at once).
-bool head_rows(int64_t rows, int tpr) { return rows * tpr <= (int64_t)sm_count() * 4 * kT; }
+// f(form) with the form of a launch over `rows` rows as a compile-time
+// constant.  Rows are loaded before the wait for the previous kernel where
+// all lanes are resident at once.  Rows of the kernels in csr_rows.cuh, one
+// lane per row, start at a full chip (152 x 2048): 1M rows of 30 entries, FP64
+// cycle 658 -> 619 us; 300k rows, one lane each, lose 2 to 4 %.
+template <int TPR, class F>
+void row_form(int64_t rows, bool wide, F&& f) {
+    if (rows * TPR <= (int64_t)sm_count() * 4 * kT) return f(std::integral_constant<int, kRowHead>());
+    if constexpr (TPR > 1) {
+        if (wide && rows >= (int64_t)sm_count() * 2048) return f(std::integral_constant<int, kRow32>());
+    }
+    f(std::integral_constant<int, kRowEach>());
+}
 
-// f(lanes per row, rows loaded ahead) with both as compile-time constants.
+// f(lanes per row, form) for a level's operator.  Float32 rows of 15 to 40
+// entries: two lanes per row leave L1's wavefronts as the bound, so eight
+// with the loads ahead where the launch is large (1M rows of 30 entries:
+// cycle 458 -> 404 us) and four below (100k rows: 106 -> 97); longer rows stay
+// with four, one row at a time (1M rows of 56 entries: 565 against 569).
+// FP64 rows of that length take four where every lane has one row (100k rows:
+// 157 -> 151; more lanes cost FP64 additions in the larger launches).
+template <typename T>
+int level_tpr(const MgLevel& L) {
+    if (L.tpr != 2 || L.nnz < 15 * L.N) return L.tpr;
+    if (sizeof(T) == 8) return L.N * 4 <= (int64_t)sm_count() * 4 * kT ? 4 : 2;
+    return L.N >= (int64_t)sm_count() * 2048 ? 8 : 4;
+}
 template <class F>
-void row_launch(int64_t rows, int tpr, F&& f) {
-    const bool head = head_rows(rows, tpr);
+void row_launch(int64_t rows, int tpr, bool wide, F&& f) {
     auto go = [&](auto tc) {
-        if (head) f(tc, std::true_type());
-        else f(tc, std::false_type());
+        constexpr int TPR = decltype(tc)::value;
+        row_form<TPR>(rows, wide, [&](auto form) { f(tc, form); });
     };
     switch (tpr) {
         case 8: go(std::integral_constant<int, 8>()); break;
@@ -1158,29 +1188,41 @@ void row_launch(int64_t rows, int tpr, F&& f) {
         default: go(std::integral_constant<int, 1>()); break;
     }
 }
+template <class F>
+int row_blocks(int64_t rows, int tpr, F) {
+    return blocks_for(F::value == kRow32 ? rows : rows * tpr);
+}
+// Whether kRow32 is the better form of a large launch: FP64 rows of two or
+// four lanes, and the float32 rows that level_tpr gives eight.
+template <typename T>
+bool row_wide(int tpr, int base) {
+    return sizeof(T) == 8 ? tpr <= 4 : tpr == 8 && base == 2;
+}
 
 template <typename T, typename BT, typename OT>
 void jacobi(const MgLevel& L, const T* xi, const BT* b, OT* xo, const int* flag, cudaStream_t st) {
-    row_launch(L.N, L.tpr, [&](auto tc, auto hc) {
-        launch_chained(true, mg_jacobi_kernel<T, BT, OT, decltype(tc)::value, decltype(hc)::value>,
-                       blocks_for(L.N * L.tpr), kT, 0, st, L.row_ptr, L.col, Sel<T>::val(L), L.N, xi, b,
+    const int tpr = level_tpr<T>(L);
+    row_launch(L.N, tpr, row_wide<T>(tpr, L.tpr), [&](auto tc, auto form) {
+        launch_chained(true, mg_jacobi_kernel<T, BT, OT, decltype(tc)::value, decltype(form)::value>,
+                       row_blocks(L.N, tpr, form), kT, 0, st, L.row_ptr, L.col, Sel<T>::val(L), L.N, xi, b,
                        Sel<T>::dinv(L), xo, flag);
     });
 }
 
 template <typename T, typename BT>
 void resid(const MgLevel& L, const T* x, const BT* b, T* r, const int* flag, cudaStream_t st) {
-    row_launch(L.N, L.tpr, [&](auto tc, auto hc) {
-        launch_chained(true, mg_resid_kernel<T, BT, decltype(tc)::value, decltype(hc)::value>,
-                       blocks_for(L.N * L.tpr), kT, 0, st, L.row_ptr, L.col, Sel<T>::val(L), L.N, x, b, r, flag);
+    const int tpr = level_tpr<T>(L);
+    row_launch(L.N, tpr, row_wide<T>(tpr, L.tpr), [&](auto tc, auto form) {
+        launch_chained(true, mg_resid_kernel<T, BT, decltype(tc)::value, decltype(form)::value>,
+                       row_blocks(L.N, tpr, form), kT, 0, st, L.row_ptr, L.col, Sel<T>::val(L), L.N, x, b, r, flag);
     });
 }
 
 template <typename T>
 void restrict_to(const MgLevel& L, int64_t nc, const T* r, T* bc, const int* flag, cudaStream_t st) {
-    row_launch(nc, L.rtpr, [&](auto tc, auto hc) {
-        launch_chained(true, mg_restrict_kernel<T, decltype(tc)::value, decltype(hc)::value>,
-                       blocks_for(nc * L.rtpr), kT, 0, st, L.rrow, L.rcol, Sel<T>::rval(L), nc, r, L.N, bc, flag);
+    row_launch(nc, L.rtpr, row_wide<T>(L.rtpr, L.rtpr), [&](auto tc, auto form) {
+        launch_chained(true, mg_restrict_kernel<T, decltype(tc)::value, decltype(form)::value>,
+                       row_blocks(nc, L.rtpr, form), kT, 0, st, L.rrow, L.rcol, Sel<T>::rval(L), nc, r, L.N, bc, flag);
     });
 }
 
@@ -1409,7 +1451,7 @@ bool tail_cycle(const MgHierarchy& h, int first, const double* b, double* x, con
         t = TailLevel<T>{};
         t.n = (int)L.N;
         t.nnz = (int)L.nnz;
-        t.tpr = L.tpr;
+        t.tpr = level_tpr<T>(L);
         t.row_ptr = L.row_ptr;
         t.col = L.col;
         t.val = Sel<T>::val(L);
