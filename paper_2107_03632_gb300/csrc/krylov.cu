@@ -214,8 +214,8 @@ __device__ __forceinline__ double row_dot64(const int64_t* __restrict__ row_ptr,
 // product split exactly by FMA (p + e = a x) and the running sum kept as an
 // unevaluated pair (TwoSum, Knuth), so the residual is accurate to about
 // eps |r_i| instead of eps sum |a x| (the latter reaches 1e-10 of |b| on the
-// finest m = 6 workload).  Used for the explicit residuals that decide
-// convergence and restart every pass; ~10 FP64 operations per entry.
+// finest m = 6 workload).  ~10 FP64 operations per entry: the rows
+// that residual_wide below does not take.
 __device__ __forceinline__ void two_sum64(double a, double b, double& s, double& e) {
     s = __dadd_rn(a, b);
     const double bb = __dadd_rn(s, -a);
@@ -223,7 +223,7 @@ __device__ __forceinline__ void two_sum64(double a, double b, double& s, double&
 }
 
 template <int TPR>
-__device__ __forceinline__ double row_residual64(const int64_t* __restrict__ row_ptr, const int* __restrict__ col,
+__device__ __noinline__ double row_residual_fma(const int64_t* __restrict__ row_ptr, const int* __restrict__ col,
                                                  const double* __restrict__ val, const double* __restrict__ x,
                                                  int64_t nx, int64_t row, int sub, bool valid, double bi) {
     (void)nx;  // length of x: bound of the checked build's tests
@@ -251,6 +251,108 @@ __device__ __forceinline__ double row_residual64(const int64_t* __restrict__ row
         two_sum64(sh, oh, t, te);
         sh = t;
         sl = __dadd_rn(sl, __dadd_rn(ol, te));
+    }
+    double rh, rl;
+    two_sum64(bi, -sh, rh, rl);
+    return __dadd_rn(rh, __dadd_rn(rl, -sl));
+}
+
+// The same residual with the sum in 128-bit integers.  At 2 FP64 lanes per
+// cycle and SM the ten operations per entry above are what such a kernel
+// takes (1M rows of 30 entries: 667 us, a plain product 60); about 60 integer
+// instructions per entry are ten times faster.  A product of two 53-bit
+// mantissas has 106 bits; it is placed six bits up, with the largest exponent
+// of a lane's products so far as the unit's, so a product loses less than
+// 2^-111 of the largest one and 2^14 of them fit.  The sum is then split into
+// two doubles and subtracted from b as above.  Rows with an infinity, a NaN,
+// a product that could overflow or more than 2^14 entries are left to the
+// floating-point form (the whole warp's rows).
+constexpr int kWidePad = 6;
+constexpr int kWideNone = -(1 << 20);  // exponent of a sum without a non-zero product
+
+// acc / 2^d, d >= 0
+__device__ __forceinline__ __int128 wide_down(__int128 acc, int d) { return d < 127 ? acc >> d : (__int128)0; }
+
+// The 53 leading bits of mag 2^e2 (truncated), and mag without them.
+__device__ __forceinline__ double wide_top(unsigned __int128& mag, int e2) {
+    const unsigned long long hi = (unsigned long long)(mag >> 64), lo = (unsigned long long)mag;
+    if ((hi | lo) == 0) return 0.0;
+    const int t = hi ? 127 - __clzll((long long)hi) : 63 - __clzll((long long)lo);  // leading bit
+    const int drop = max(t - 52, 0);
+    const unsigned long long m = (unsigned long long)(mag >> drop);
+    mag -= (unsigned __int128)m << drop;
+    const int field = t + e2 + 1023;
+    if (t >= 52 && field >= 1 && field <= 2046)
+        return __longlong_as_double((long long)((m & 0xfffffffffffffull) | ((unsigned long long)field << 52)));
+    return scalbn((double)m, drop + e2);
+}
+
+template <int TPR>
+__device__ __forceinline__ double row_residual64(const int64_t* __restrict__ row_ptr, const int* __restrict__ col,
+                                                 const double* __restrict__ val, const double* __restrict__ x,
+                                                 int64_t nx, int64_t row, int sub, bool valid, double bi) {
+    constexpr int U = 4;
+    int64_t a = 0, e = 0;
+    if (valid) {
+        a = __ldg(row_ptr + row);
+        e = __ldg(row_ptr + row + 1);
+    }
+    __int128 acc = 0;
+    int unit = kWideNone;
+    bool bad = e - a > 1 << 14;
+    if (!bad) {
+        for (int64_t k = a + sub; k < e; k += U * TPR) {
+            double av[U], xv[U];
+            int ex[U], top = kWideNone;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const bool in = k + u * TPR < e;
+                av[u] = in ? __ldg(val + k + u * TPR) : 0.0;
+                xv[u] = in ? __ldg(&RB_AT(x, __ldg(col + k + u * TPR), nx)) : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int ea = (__double2hiint(av[u]) >> 20) & 0x7ff, eb = (__double2hiint(xv[u]) >> 20) & 0x7ff;
+                ex[u] = max(ea, 1) + max(eb, 1);
+                bad |= ea == 0x7ff || eb == 0x7ff || ex[u] > 2044 + 1022;
+                if ((__double_as_longlong(av[u]) << 1) != 0 && (__double_as_longlong(xv[u]) << 1) != 0)
+                    top = max(top, ex[u]);
+            }
+            if (top > unit) {
+                acc = wide_down(acc, top - unit);
+                unit = top;
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const unsigned long long ba = (unsigned long long)__double_as_longlong(av[u]);
+                const unsigned long long bx = (unsigned long long)__double_as_longlong(xv[u]);
+                const unsigned long long ma = (ba & 0xfffffffffffffull) | ((ba << 1) >> 53 ? 1ull << 52 : 0);
+                const unsigned long long mx = (bx & 0xfffffffffffffull) | ((bx << 1) >> 53 ? 1ull << 52 : 0);
+                const unsigned __int128 p = (unsigned __int128)(ma << kWidePad) * mx;
+                const int d = unit - ex[u];  // (a zero product may be above the unit)
+                const __int128 q = (__int128)(d > 0 ? (d < 127 ? p >> d : (unsigned __int128)0) : p);
+                acc += (long long)(ba ^ bx) < 0 ? -q : q;
+            }
+        }
+    }
+    if (__any_sync(0xffffffffu, bad)) return row_residual_fma<TPR>(row_ptr, col, val, x, nx, row, sub, valid, bi);
+#pragma unroll
+    for (int o = TPR / 2; o > 0; o >>= 1) {
+        const int ou = __shfl_xor_sync(0xffffffffu, unit, o, TPR);
+        const unsigned long long oh = __shfl_xor_sync(0xffffffffu, (unsigned long long)(acc >> 64), o, TPR);
+        const unsigned long long ol = __shfl_xor_sync(0xffffffffu, (unsigned long long)acc, o, TPR);
+        const __int128 other = (__int128)(((unsigned __int128)oh << 64) | ol);
+        const int nu = max(unit, ou);
+        acc = wide_down(acc, nu - unit) + wide_down(other, nu - ou);
+        unit = nu;
+    }
+    const bool neg = acc < 0;
+    unsigned __int128 mag = neg ? (unsigned __int128)(-acc) : (unsigned __int128)acc;
+    const int e2 = unit - 2150 - kWidePad;
+    double sh = wide_top(mag, e2), sl = wide_top(mag, e2);
+    if (neg) {
+        sh = -sh;
+        sl = -sl;
     }
     double rh, rl;
     two_sum64(bi, -sh, rh, rl);
