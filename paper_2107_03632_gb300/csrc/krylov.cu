@@ -93,7 +93,7 @@ struct KState {
     unsigned int counter[kSlots];
 };
 
-__device__ __forceinline__ double* part_at(double* part, int slot, int q) {
+__host__ __device__ __forceinline__ double* part_at(double* part, int slot, int q) {
     return part + ((size_t)slot * kQ + q) * kMaxBlocks;
 }
 
@@ -632,6 +632,298 @@ __global__ void __launch_bounds__(kThreads) update_xr64_kernel(int64_t N, double
         finish_iteration(st, tot[0], tot[1], tot[2]);
 }
 
+// ---- whole iterations of a small system in one launch ------------------------
+// An iteration of five launches over 10k rows is 30 us, of which the work is
+// two or three: each launch is a few microseconds of latency and a reduction
+// that its last block finishes alone.  Here one block per SM keeps its rows
+// (entries, vectors) in shared memory for all the iterations of a launch and
+// the blocks exchange vectors through L2.  Two of the five steps need no
+// exchange of their own: A p gathers r, p and v of the iteration before and
+// forms p = r + beta (p - omega v) per entry, A s forms s = r - alpha v (the
+// bits of the stored vectors); what is left is one exchange per reduction,
+// three per iteration.  What bounds it: the chain of each exchange (stores
+// fenced, arrivals counted, the blocks' sums read back at 1,000 to 1,500
+// cycles per trip, FP64 additions in a tree) and, for larger systems, the
+// three FP64 operations more per entry.  Microseconds per iteration, separate
+// kernels and here, rows of 15 entries: 2k rows 31 and 17, 10k 30 and 19, 40k
+// 41 and 30, 80k 64 and 41.  The line is where a block's mean share of the
+// entries fills what it holds in shared memory.
+constexpr int kPassT = 512;
+constexpr int kPassTpr = 4;
+constexpr int kPassRows = 32;          // fewest rows per block
+constexpr int kPassBlocks = 160;       // most blocks
+constexpr int kPassEntries = 8192;     // mean entries per block up to which the kernel is used
+constexpr int kPassSmemEntries = 10240;  // entries per block held in shared memory (the rest: global)
+constexpr int kPassSlot = 4;           // slots of `part` for the three reductions: 4, 5, 6
+constexpr int kPassFlagSlot = 7;       // the blocks' arrivals so far
+constexpr int kPassVecs = 9;
+static_assert(kPassFlagSlot < kSlots && kPassSlot + 3 <= kPassFlagSlot, "partial-sum slots");
+
+inline size_t pass_smem(int rows) {
+    return (size_t)kPassSmemEntries * 12 + (size_t)rows * 8 * kPassVecs + (size_t)(rows + 2) * 8;
+}
+
+// A value that another block has written before the last exchange (the
+// compiler may move or merge plain and __ldcg loads).
+__device__ __forceinline__ double load_exchanged(const double* p) {
+    double v;
+    asm volatile("ld.relaxed.gpu.global.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// then(sums over all blocks) in thread 0 of every block, before any thread
+// returns; also the exchange: what any thread wrote before is visible (through
+// L2) to every thread after.  Only the first `warps` warps hold values, in the
+// lanes that are multiples of LANES.  An FP64 instruction is 16 cycles of the
+// SM's unit per warp, so warps without values take no part, one warp adds the
+// blocks' sums and one thread works out the scalars (with every thread working
+// them out an iteration of 10k rows was 22 us, now 19).  False when a block
+// did not arrive within the limit.
+template <int NQ, int LANES, class F>
+__device__ __forceinline__ bool pass_sums(double (&v)[NQ], int warps, double* part, int slot, unsigned int* count,
+                                          unsigned int target, F&& then) {
+    constexpr int W = kPassT / 32;
+    __shared__ double sh[NQ][W];
+    __shared__ int arrived;
+    const int tid = (int)threadIdx.x, lane = tid & 31, wid = tid >> 5, nb = (int)gridDim.x;
+    if (wid < warps) {
+#pragma unroll
+        for (int o = 16; o >= LANES; o >>= 1)
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+        if (lane == 0)
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) sh[q][wid] = v[q];
+    }
+    __syncthreads();
+    if (wid == 0) {
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) v[q] = lane < warps ? sh[q][lane] : 0.0;
+#pragma unroll
+        for (int o = W / 2; o > 0; o >>= 1)
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+        int ok = 1;
+        if (lane == 0) {
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) RB_AT(part_at(part, slot, q), blockIdx.x, kMaxBlocks) = v[q];
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
+            unsigned int seen;
+            int polls = 0;
+            do {
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(count) : "memory");
+            } while (seen < target && ++polls < (1 << 21));
+            ok = seen >= target;
+        }
+        __syncwarp();  // the other lanes' loads follow the acquire
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+        // all of a lane's loads in flight at once: a value another SM has just
+        // written is 1,000 to 1,500 cycles away
+        double w[NQ][kPassBlocks / 32];
+#pragma unroll
+        for (int u = 0; u < kPassBlocks / 32; ++u)
+#pragma unroll
+            for (int q = 0; q < NQ; ++q)
+                w[q][u] = load_exchanged(part_at(part, slot, q) + min(u * 32 + lane, nb - 1));
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) v[q] = 0.0;
+#pragma unroll
+        for (int u = 0; u < kPassBlocks / 32; ++u)
+            if (u * 32 < nb)
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) v[q] += u * 32 + lane < nb ? w[q][u] : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+        if (lane == 0) {
+            arrived = ok;
+            then(v);
+        }
+    }
+    __syncthreads();
+    return arrived != 0;
+}
+
+// `iters` iterations from the state the other kernels leave (see
+// update_p64_kernel ... update_xr64_kernel), rows_per_block rows per block.
+// p2, v2: second buffers of p and v (a block writes its new values while
+// others still gather the old ones).
+__global__ void __launch_bounds__(kPassT) pass64_kernel(const int64_t* __restrict__ row_ptr,
+                                                        const int* __restrict__ col,
+                                                        const double* __restrict__ val, int64_t N,
+                                                        int rows_per_block, int iters, double* x, double* r,
+                                                        const double* rh, double* p, double* v, double* p2,
+                                                        double* v2, const double* __restrict__ d,
+                                                        const double* __restrict__ dinv, KState* st, double* part) {
+    extern __shared__ __align__(16) unsigned char pass_smem_base[];
+    constexpr int U = 4, G = kPassT / kPassTpr;
+    const int tid = (int)threadIdx.x, sub = tid & (kPassTpr - 1), grp = tid / kPassTpr;
+    const unsigned int nb = gridDim.x;
+    const int64_t row0 = (int64_t)blockIdx.x * rows_per_block;
+    const int R = (int)max((int64_t)0, min((int64_t)rows_per_block, N - row0));
+    double* sval = reinterpret_cast<double*>(pass_smem_base);
+    double* sx = sval + kPassSmemEntries;
+    double *srh = sx + rows_per_block, *sd = srh + rows_per_block, *sdi = sd + rows_per_block,
+           *sr = sdi + rows_per_block, *sp = sr + rows_per_block, *sv = sp + rows_per_block,
+           *ss = sv + rows_per_block, *stt = ss + rows_per_block;
+    int64_t* srow = reinterpret_cast<int64_t*>(stt + rows_per_block);  // entries relative to the block's first
+    int* scol = reinterpret_cast<int*>(srow + rows_per_block + 2);
+    unsigned int* count = reinterpret_cast<unsigned int*>(part_at(part, kPassFlagSlot, 0));
+    double *const p_out = p, *const v_out = v;
+    if (st->flag != kRunning) return;  // (the same in every block: written after the last exchange)
+    const int64_t base = R > 0 ? __ldg(row_ptr + row0) : 0;
+    for (int i = tid; i < R; i += kPassT) {
+        sx[i] = x[row0 + i];
+        srh[i] = rh[row0 + i];
+        sd[i] = d[row0 + i];
+        sdi[i] = dinv[row0 + i];
+        sr[i] = r[row0 + i];
+        sp[i] = p[row0 + i];
+        sv[i] = v[row0 + i];
+    }
+    for (int i = tid; i <= R; i += kPassT) srow[i] = R > 0 ? __ldg(row_ptr + row0 + i) - base : 0;
+    __syncthreads();
+    const int held = (int)min(srow[R], (int64_t)kPassSmemEntries);
+    for (int k = tid; k < held; k += kPassT) {
+        sval[k] = __ldg(val + base + k);
+        scol[k] = __ldg(col + base + k);
+    }
+    __shared__ KState k;  // the scalars, kept by thread 0
+    __shared__ double beta;
+    if (tid == 0) {
+        k = *st;
+        beta = (k.rho_new / k.rho) * (k.alpha / k.omega);
+    }
+    unsigned int arrivals = 0;
+    bool late = false;  // a block did not arrive
+    const int row_warps = (min(R, G) * kPassTpr + 31) / 32, own_warps = min(kPassT / 32, (R + 31) / 32);
+    __syncthreads();
+
+    // sum of a row's entries times g(column), in every lane of the group
+    auto row_sum = [&](int i, bool valid, auto&& g) {
+        double sum = 0.0;
+        const int64_t a = valid ? srow[i] : 0, e = valid ? srow[i + 1] : 0;
+        for (int64_t k = a + sub; k < e; k += U * kPassTpr) {
+            double av[U];
+            int c[U];
+            bool in[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t ku = k + u * kPassTpr;
+                in[u] = ku < e;
+                const bool near = ku < held;
+                av[u] = !in[u] ? 0.0 : near ? sval[ku] : __ldg(val + base + ku);
+                c[u] = !in[u] ? 0 : near ? scol[ku] : __ldg(col + base + ku);
+            }
+            g(c, in, av, sum);
+        }
+#pragma unroll
+        for (int o = kPassTpr / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o, kPassTpr);
+        return sum;
+    };
+
+    while (iters-- > 0) {
+        // p = r + beta (p - omega v), v = D^-1 A p, (rh, v)
+        const double be = beta, om = k.omega;
+        double one[1] = {0.0};
+        for (int i0 = 0; i0 < R; i0 += G) {
+            const int i = i0 + grp;
+            const double ap = row_sum(i, i < R, [&](int (&c)[U], bool (&in)[U], double (&av)[U], double& sum) {
+                double gr[U], gp[U], gv[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    gr[u] = in[u] ? load_exchanged(&RB_AT(r, c[u], N)) : 0.0;
+                    gp[u] = in[u] ? load_exchanged(&RB_AT(p, c[u], N)) : 0.0;
+                    gv[u] = in[u] ? load_exchanged(&RB_AT(v, c[u], N)) : 0.0;
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (in[u]) sum = fma(av[u], fma(be, fma(-om, gv[u], gp[u]), gr[u]), sum);
+            });
+            if (i < R && sub == 0) {
+                const double pi = fma(be, fma(-om, sv[i], sp[i]), sr[i]), vi = ap * sdi[i];
+                sp[i] = pi;
+                sv[i] = vi;
+                p2[row0 + i] = pi;
+                v2[row0 + i] = vi;
+                one[0] = fma(srh[i], vi, one[0]);
+            }
+        }
+        {
+            double* q = p;
+            p = p2;
+            p2 = q;
+            q = v;
+            v = v2;
+            v2 = q;
+        }
+        auto alpha_of = [&](const double (&sum)[1]) { set_alpha(&k, sum[0]); };
+        if (!pass_sums<1, kPassTpr>(one, row_warps, part, kPassSlot, count, arrivals += nb, alpha_of)) late = true;
+        if (late || k.flag != kRunning) break;
+        const double al = k.alpha;
+        // s = r - alpha v, t = D^-1 A s, (t, s), (t, t)
+        double two[2] = {0.0, 0.0};
+        for (int i0 = 0; i0 < R; i0 += G) {
+            const int i = i0 + grp;
+            const double as = row_sum(i, i < R, [&](int (&c)[U], bool (&in)[U], double (&av)[U], double& sum) {
+                double gr[U], gv[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    gr[u] = in[u] ? load_exchanged(&RB_AT(r, c[u], N)) : 0.0;
+                    gv[u] = in[u] ? load_exchanged(&RB_AT(v, c[u], N)) : 0.0;
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (in[u]) sum = fma(av[u], fma(-al, gv[u], gr[u]), sum);
+            });
+            if (i < R && sub == 0) {
+                const double ti = as * sdi[i], si = fma(-al, sv[i], sr[i]);
+                stt[i] = ti;
+                ss[i] = si;
+                two[0] = fma(ti, si, two[0]);
+                two[1] = fma(ti, ti, two[1]);
+            }
+        }
+        auto omega_of = [&](const double (&sum)[2]) { set_omega(&k, sum[0], sum[1], 0.0); };
+        if (!pass_sums<2, kPassTpr>(two, row_warps, part, kPassSlot + 1, count, arrivals += nb, omega_of)) late = true;
+        if (late || k.flag != kRunning) break;
+        const double om2 = k.omega;
+        // x += alpha p + omega s, r = s - omega t
+        double acc[3] = {0.0, 0.0, 0.0};
+        for (int i = tid; i < R; i += kPassT) {
+            const double si = ss[i], ri = fma(-om2, stt[i], si), ru = ri * sd[i];
+            sx[i] = fma(om2, si, fma(al, sp[i], sx[i]));
+            sr[i] = ri;
+            r[row0 + i] = ri;
+            acc[0] = fma(ru, ru, acc[0]);
+            acc[1] = fma(srh[i], ri, acc[1]);
+            acc[2] = fma(ri, ri, acc[2]);
+        }
+        auto finish = [&](const double (&sum)[3]) {
+            finish_iteration(&k, sum[0], sum[1], sum[2]);
+            beta = (k.rho_new / k.rho) * (k.alpha / k.omega);
+        };
+        if (!pass_sums<3, 1>(acc, own_warps, part, kPassSlot + 2, count, arrivals += nb, finish)) late = true;
+        if (late || k.flag != kRunning) break;
+    }
+    // (every block is past its last gather: it left the loop behind the same exchange)
+    for (int i = tid; i < R; i += kPassT) {
+        x[row0 + i] = sx[i];
+        p_out[row0 + i] = sp[i];
+        v_out[row0 + i] = sv[i];
+    }
+    if (blockIdx.x == 0 && tid == 0) {
+        st->rho = k.rho;
+        st->rho_new = k.rho_new;
+        st->alpha = k.alpha;
+        st->omega = k.omega;
+        st->rnorm2 = k.rnorm2;
+        st->iter = k.iter;
+        st->flag = late ? (int)kBreakdown : k.flag;
+    }
+}
+
 // ============================================================ double-float ==
 // sum_j a_ij (d_j - d_i) over one row with float a_ij; TPR lanes, df32
 // accumulation (result in every lane).
@@ -1094,6 +1386,40 @@ void iter64(int tpr, const rbffd_csr& A, double* x, const Work& w, cudaStream_t 
     }
 }
 
+// `count` iterations by pass64_kernel; false where it does not apply.
+// (Profiling times the products, so it takes the separate kernels.)
+bool pass64(const rbffd_csr& A, double* x, const Work& w, int count, cudaStream_t st) {
+    const int sms = std::min(sm_count(), kPassBlocks);
+    if (w.mg || profiling() || A.nnz > (int64_t)sms * kPassEntries) return false;
+    const int rows = (int)std::max<int64_t>(kPassRows, (A.n_rows + sms - 1) / sms);
+    const size_t smem = pass_smem(rows);
+    if (smem > 220 * 1024) return false;
+    if (cudaFuncSetAttribute(pass64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaMemsetAsync(part_at(w.part, kPassFlagSlot, 0), 0, sizeof(unsigned int), st) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)((A.n_rows + rows - 1) / rows));
+    cfg.blockDim = dim3(kPassT);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeCooperative;  // the blocks wait on one another
+    attr.val.cooperative = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, pass64_kernel, A.row_ptr, A.col, static_cast<const double*>(A.val), A.n_rows, rows,
+                           count, x, w.r, static_cast<const double*>(w.rh), w.p, w.v, w.s, w.t,
+                           static_cast<const double*>(w.d), static_cast<const double*>(w.dinv), w.st,
+                           w.part) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    note_launches(1);
+    return true;
+}
+
 void iter_df(int tpr, const rbffd_csr& A32, const Work& w, cudaStream_t st, std::vector<int>& ev, bool chained) {
     switch (tpr) {
         case 2: OpsDf<2>::iteration(A32, w, st, ev, chained); break;
@@ -1205,7 +1531,7 @@ int run_chunks(const Work& w, KState* hs, cudaStream_t st, ChunkPlan& plan, Iter
         const int chunk = plan.chunk;
         const auto t0 = std::chrono::steady_clock::now();
         ev.clear();
-        for (int c = 0; c < chunk; ++c) iter(ev, c > 0);
+        iter(ev, chunk);
         RBFFD_LAUNCH_CHECK();
         const int rc = read_state(w, hs, st);
         if (rc != RBFFD_OK) return -rc;
@@ -1368,7 +1694,10 @@ int solve_fp64(const rbffd_csr& A, const double* b, double* x, const rbffd_solve
             if ((rc = read_state(w, &hs, st)) != RBFFD_OK) return rc;
         }
         const int f = run_chunks(
-            w, &hs, st, chunk, [&](std::vector<int>& ev, bool chained) { iter64(tpr, A, x, w, st, ev, chained); }, &mon,
+            w, &hs, st, chunk, [&](std::vector<int>& ev, int count) {
+                if (pass64(A, x, w, count, st)) return;
+                for (int c = 0; c < count; ++c) iter64(tpr, A, x, w, st, ev, c > 0);
+            }, &mon,
             rel, total);
         if (f < 0) return -f;
         if (w.left && (rc = mg_dirichlet_fix(w.mg, b, x, nullptr, st)) != RBFFD_OK) return rc;
@@ -1468,7 +1797,9 @@ int solve_mixed(const rbffd_csr& A, const rbffd_csr& A32, const double* b, doubl
         if ((rc = read_state(w, &hs, st)) != RBFFD_OK) return rc;
         const double start2 = hs.rmax2;
         const int f = run_chunks(
-            w, &hs, st, chunk, [&](std::vector<int>& ev, bool chained) { iter_df(tpr32, A32, w, st, ev, chained); },
+            w, &hs, st, chunk, [&](std::vector<int>& ev, int count) {
+                for (int c = 0; c < count; ++c) iter_df(tpr32, A32, w, st, ev, c > 0);
+            },
             &mon, rel, total);
         if (f < 0) return -f;
         total += hs.iter;
