@@ -80,3 +80,35 @@ def test_repeats_bit_for_bit():
     for _ in range(50):
         x, i = r.rbffd_solve(A, bd, None, opts)
         assert i["iters"] == i0["iters"] and torch.equal(x, x0)
+
+
+def test_solves_from_several_threads_and_streams():
+    """Launches whose blocks wait on one another, from four streams at once."""
+    import threading
+
+    from paper_2107_03632_gb300 import rbffd as r
+
+    dev = lambda a: torch.from_numpy(a).cuda()
+    systems = []
+    for seed in range(4):
+        rp, col, val, b = _system(10_007, 15, 20 + seed)
+        A, bd = r.CsrMatrix(dev(rp), dev(col), dev(val)), dev(b)
+        x, info = r.rbffd_solve(A, bd, None, r.make_opts(tol=1e-13))
+        systems.append((A, bd, x, info["iters"]))
+    torch.cuda.synchronize()
+    wrong = []
+
+    def work(A, bd, x0, iters):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            for _ in range(25):
+                x, info = r.rbffd_solve(A, bd, None, r.make_opts(tol=1e-13))
+                torch.cuda.current_stream().synchronize()
+                if info["iters"] != iters or not torch.equal(x, x0):
+                    wrong.append((info["iters"], iters))
+
+    threads = [threading.Thread(target=work, args=s) for s in systems]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong
