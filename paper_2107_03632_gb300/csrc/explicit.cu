@@ -14,7 +14,7 @@
 // one thread per interior row, ping-pong between two u buffers (both hold
 // the Dirichlet values, which no step writes); the steps are captured once
 // into a CUDA graph of kGraphSteps launches and replayed, so a step costs
-// its memory traffic and not a host launch, and each launch is a
+// its memory traffic and not a host launch; in small sets each launch is a
 // programmatic dependent of the one before (launch_chained).
 #include "common.cuh"
 #include "scan.cuh"
@@ -81,13 +81,31 @@ __global__ void __launch_bounds__(kT) explicit_pack_kernel(const int32_t* __rest
     if (nb) atomicOr(bad, 1);
 }
 
-// One forward-Euler step on the interior rows.  The entries go in groups of
+// One forward-Euler step on the interior rows.
+__global__ void __launch_bounds__(kT) explicit_step_kernel(const int32_t* __restrict__ rows,
+                                                           const int32_t* __restrict__ idxT,
+                                                           const double* __restrict__ wT, int64_t Ni, int n,
+                                                           const double* __restrict__ f, double dt,
+                                                           const double* __restrict__ u1, double* __restrict__ u2,
+                                                           int64_t N) {
+    (void)N;  // nodes: bound of the checked build's tests
+    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < Ni; r += (int64_t)gridDim.x * blockDim.x) {
+        double lap = 0.0;
+        for (int j = 0; j < n; ++j)
+            lap = fma(__ldg(wT + (int64_t)j * Ni + r), __ldg(&RB_AT(u1, __ldg(idxT + (int64_t)j * Ni + r), N)), lap);
+        const int i = __ldg(rows + r);
+        RB_AT(u2, i, N) = fma(dt, __ldg(&RB_AT(f, i, N)) + lap, RB_AT(u1, i, N));
+    }
+}
+
+// The same for small sets (one row per thread).  The entries go in groups of
 // U: indices and weights first, then the gathers, all in flight at once (one
 // at a time, a launch that leaves the chip idle spends its 4 us on dependent
-// L2 round trips); the first row's first group and source are loaded before
-// the previous step has completed.  30k rows, n = 12: 3.9 -> 3.1 us per step.
+// L2 round trips); the first group and the source are loaded before the
+// previous step has completed.  30k rows, n = 12: 4.0 -> 2.9 us per step.
+constexpr int kSmallT = 64;
 template <int U>
-__global__ void __launch_bounds__(kT) explicit_step_kernel(const int32_t* __restrict__ rows,
+__global__ void __launch_bounds__(kSmallT) explicit_step_small_kernel(const int32_t* __restrict__ rows,
                                                            const int32_t* __restrict__ idxT,
                                                            const double* __restrict__ wT, int64_t Ni, int n,
                                                            const double* __restrict__ f, double dt,
@@ -104,31 +122,29 @@ __global__ void __launch_bounds__(kT) explicit_step_kernel(const int32_t* __rest
             w[j] = in ? __ldg(wT + (int64_t)(j0 + j) * Ni + r) : 0.0;
         }
     };
-    const int64_t r0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int i0 = 0;
-    double f0 = 0.0;
-    if (r0 < Ni) {
-        load(r0, 0);
-        i0 = __ldg(rows + r0);
-        f0 = __ldg(&RB_AT(f, i0, N));
+    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    int i = 0;
+    double fi = 0.0;
+    if (r < Ni) {
+        load(r, 0);
+        i = __ldg(rows + r);
+        fi = __ldg(&RB_AT(f, i, N));
     }
     pdl_wait();
     pdl_next();
-    for (int64_t r = r0; r < Ni; r += (int64_t)gridDim.x * blockDim.x) {
-        const int i = r == r0 ? i0 : __ldg(rows + r);
-        const double fi = r == r0 ? f0 : __ldg(&RB_AT(f, i, N)), ui = RB_AT(u1, i, N);
-        double lap = 0.0;
-        for (int j0 = 0; j0 < n; j0 += U) {
-            if (j0 > 0 || r != r0) load(r, j0);
-            double u[U];
+    if (r >= Ni) return;
+    const double ui = RB_AT(u1, i, N);
+    double lap = 0.0;
+    for (int j0 = 0; j0 < n; j0 += U) {
+        if (j0 > 0) load(r, j0);
+        double u[U];
 #pragma unroll
-            for (int j = 0; j < U; ++j) u[j] = j0 + j < n ? __ldg(&RB_AT(u1, c[j], N)) : 0.0;
+        for (int j = 0; j < U; ++j) u[j] = j0 + j < n ? __ldg(&RB_AT(u1, c[j], N)) : 0.0;
 #pragma unroll
-            for (int j = 0; j < U; ++j)
-                if (j0 + j < n) lap = fma(w[j], u[j], lap);
-        }
-        RB_AT(u2, i, N) = fma(dt, fi + lap, ui);
+        for (int j = 0; j < U; ++j)
+            if (j0 + j < n) lap = fma(w[j], u[j], lap);
     }
+    RB_AT(u2, i, N) = fma(dt, fi + lap, ui);
 }
 
 int step_blocks(int64_t Ni) {
@@ -136,18 +152,19 @@ int step_blocks(int64_t Ni) {
     return (int)std::max<int64_t>(1, std::min<int64_t>(b, (int64_t)sm_count() * 32));
 }
 
-// Entries per group: all of a common support where there are fewer rows than
-// the chip has lanes, 8 (fewer registers, more warps) where HBM is the limit.
-// (Small blocks there too: the rows spread evenly over the SMs, whose FP64
-// units do 2 multiply-adds per clock.)
+// The small form where the rows leave most of the chip idle (all of a common
+// support in one group; blocks of 64, so that the rows spread evenly over the
+// SMs, whose FP64 units do 2 multiply-adds per clock), the plain loop, with
+// more warps, where L2 or HBM is the limit.  The line is one wave of the small
+// form.  Microseconds per step, plain and small, n = 12: 30k rows 4.0 and 2.9,
+// 60k 4.3 and 3.5, 75k 4.2 and 5.2; n = 45: 60k 9.3 and 8.4, 75k 9.3 and 13.3.
 void explicit_step(bool chained, const ExplicitLayout& L, int64_t Ni, int n, const double* f, double dt,
                    const double* u1, double* u2, int64_t N, cudaStream_t st) {
-    if (Ni <= (int64_t)sm_count() * 1024)
-        launch_chained(chained, explicit_step_kernel<16>, (unsigned)((Ni + 63) / 64), 64, 0, st, L.rows, L.idx, L.w,
-                       Ni, n, f, dt, u1, u2, N);
+    if (Ni <= (int64_t)sm_count() * 400)
+        launch_chained(chained, explicit_step_small_kernel<16>, (unsigned)((Ni + kSmallT - 1) / kSmallT), kSmallT, 0,
+                       st, L.rows, L.idx, L.w, Ni, n, f, dt, u1, u2, N);
     else
-        launch_chained(chained, explicit_step_kernel<8>, step_blocks(Ni), kT, 0, st, L.rows, L.idx, L.w, Ni, n, f, dt,
-                       u1, u2, N);
+        explicit_step_kernel<<<step_blocks(Ni), kT, 0, st>>>(L.rows, L.idx, L.w, Ni, n, f, dt, u1, u2, N);
 }
 
 }  // namespace
