@@ -177,21 +177,27 @@ SPMV_DF_TRAFFIC = {"source_sha256_16": "ea63d4b54b1529b9", "traffic_over_algorit
                    / 279652728.0}
 
 
-# DRAM traffic of the FP64 weight solve from one ncu capture of
-# weights_ns_kernel<128, NsF64> (four warps per stencil) at 1M nodes, m = 6,
-# n = 56: dram read + write per stencil (idx read, w written; the gathered
-# coordinates come from L2).  Valid only at that (n, m) and while the
-# kernel's sources are the ones captured.
-WEIGHTS_F64_TRAFFIC = {"source_sha256_16": "5a541d3a57e1eb7e", "n": 56, "m": 6,
-                       "bytes_per_node": (259.903744e6 + 406.790144e6) / 1001697.0}
+# The refined FP64 weight solve (weights_refined_kernel) at 1M nodes, m = 6,
+# n = 56, from one ncu capture: DRAM read + write and warp instructions per
+# stencil.  Valid only at that (n, m) and while the kernel's sources are the
+# ones captured.
+WEIGHTS_F64_TRAFFIC = {"source_sha256_16": "12f4cc266207f88f", "n": 56, "m": 6,
+                       "bytes_per_node": (249.541632e6 + 406.857984e6) / 1000870.0,
+                       "warp_instr_per_node": 34599512456 / 1000870.0}
 
 
 def weights_source_hash():
     import hashlib
 
     d = os.path.join(ROOT, "paper_2107_03632_gb300", "csrc")
-    seg = "".join(open(os.path.join(d, f)).read() for f in ("weights.cu", "common.cuh", "checked.cuh"))
+    seg = "".join(open(os.path.join(d, f)).read() for f in ("refined.cu", "fixed.cuh", "common.cuh", "checked.cuh"))
     return hashlib.sha256(seg.encode()).hexdigest()[:16]
+
+
+def weights_refined(n: int, m: int) -> bool:
+    """Whether the FP64 weights come from the refined float32 solve (the
+    library's rule; RBFFD_WEIGHTS=ns64 asks for the elimination)."""
+    return 1 <= m <= 6 and n <= 64 and os.environ.get("RBFFD_WEIGHTS", "") != "ns64"
 
 
 def spmv_df_source_hash():
@@ -263,8 +269,9 @@ def weights_df_instr(n: int, m: int) -> float:
 
 
 def weights_roofline(kernel_name: str, n: int, m: int, N: int, ms: float, extra: dict) -> dict:
-    """Roofline of the weight solve: FP64 kernels against the FP64 units'
-    peak (counted flops); double-float kernels against the FP32 pipe's peak
+    """Roofline of the weight solve: FP64 elimination against the FP64 units'
+    peak (counted flops), its refined form against the FP32 pipe's; double-float
+    kernels against the FP32 pipe's peak
     (FP32 instructions of the df operations), with the FP64-equivalent rate
     beside it."""
     fl = weights_flops(n, m)
@@ -278,6 +285,17 @@ def weights_roofline(kernel_name: str, n: int, m: int, N: int, ms: float, extra:
                "peak_kind": "FP32 lanes x max clock (152 SMs x 128 lanes x 2070 MHz)",
                "instr_per_node": ins, "df_ops_per_node": weights_df_ops(n, m),
                "fp64_equivalent_tflops": f64_equiv, "fp64_equivalent_frac_of_fp64_units": f64_equiv / FP64_PEAK_TFLOPS_UNITS}
+    elif kernel_name.startswith("null-space") and weights_refined(n, m):
+        # the float32 elimination's multiply-adds (the steps weights_flops
+        # counts) on the FP32 pipe; the residuals' integer work is not counted
+        ins = fl / 2.0
+        ach = ins * N / (ms * 1e-3) / 1e12
+        out = {"kernel": f"weights_refined_kernel, FP64 weights by refinement ({kernel_name} for the stencils it "
+                         f"leaves), m={m}, n={n}", "bound": "alu",
+               "achieved": ach, "peak": FP32_PEAK_TINSTR_UNITS, "unit": "T FP32 lane-instr/s",
+               "frac": ach / FP32_PEAK_TINSTR_UNITS,
+               "peak_kind": "FP32 lanes x max clock (152 SMs x 128 lanes x 2070 MHz)",
+               "fp64_equivalent_tflops": f64_equiv, "fp64_equivalent_frac_of_fp64_units": f64_equiv / FP64_PEAK_TFLOPS_UNITS}
     else:
         out = {"kernel": f"weights_ns_kernel, FP64 ({kernel_name}), m={m}, n={n}", "bound": "alu",
                "achieved": f64_equiv, "peak": FP64_PEAK_TFLOPS_UNITS, "unit": "TFLOP/s",
@@ -285,8 +303,11 @@ def weights_roofline(kernel_name: str, n: int, m: int, N: int, ms: float, extra:
                "peak_kind": "FP64 units x max clock (152 SMs x 2 FMA/clk x 2070 MHz)"}
     traffic = None
     t = WEIGHTS_F64_TRAFFIC
-    if "df" not in kernel_name and (n, m) == (t["n"], t["m"]) and weights_source_hash() == t["source_sha256_16"]:
+    if out["kernel"].startswith("weights_refined") and (n, m) == (t["n"], t["m"]) \
+            and weights_source_hash() == t["source_sha256_16"]:
         traffic = t["bytes_per_node"] * N
+        # issue slots: 4 warp instructions per SM and clock
+        out["issue_frac"] = t["warp_instr_per_node"] * N / (ms * 1e-3) / (152 * 4 * 2070e6)
     out.update({"traffic": traffic, "traffic_unit": "bytes per launch (ncu dram read + write, scaled by N)",
                 "flops_per_node": fl, "ms_per_launch": ms, "launches": 1})
     out.update(extra)
@@ -1427,8 +1448,10 @@ def run_gpu(args):
                   "measured_in": "separate profiled loop (events around every sweep)"}
     roof_weights = weights_roofline(wcfg["kernel"], n, m, N, st_ms[1],
                                     {"cublas_dgemm_tflops": fp64_peak,
-                                     "frac_of_dgemm": (weights_flops(n, m) * N / (st_ms[1] * 1e-3) / 1e12
-                                                       / fp64_peak if fp64_peak == fp64_peak else None),
+                                     # (the refined form does not run these flops in FP64)
+                                     "fp64_equivalent_frac_of_dgemm": (weights_flops(n, m) * N / (st_ms[1] * 1e-3)
+                                                                       / 1e12 / fp64_peak
+                                                                       if fp64_peak == fp64_peak else None),
                                      "lu_equivalent_tflops": lu_equiv,
                                      "measured_in": "timed region (events around the weights launch)"})
     weights_dominate = st_ms[1] > roof_solve["ms_per_step"]
@@ -1440,7 +1463,8 @@ def run_gpu(args):
                    "tol": args.tol,
                    "precision_by_stage": {
                        "stencils": "f64 distance keys (f32 pruning bounds)",
-                       "weights": "f64 (null-space elimination + L D L^T, FP64 throughout)",
+                       "weights": "f64 (float32 null-space solve refined with 64-bit fixed-point residuals, f64 "
+                                  "elimination of the stencils it leaves)",
                        "assembly": "f64 values (+ f32 copy for the preconditioner)",
                        "krylov": "f64 BiCGSTAB, f64 residual and updates",
                        "preconditioner": ("float32 multigrid V-cycle (coarse weights in double-float)" if use_mg
