@@ -712,7 +712,7 @@ __device__ __forceinline__ bool pass_sums(double (&v)[NQ], int warps, double* pa
             int polls = 0;
             do {
                 asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(count) : "memory");
-            } while (seen < target && ++polls < (1 << 21));
+            } while (seen < target && ++polls < (1 << 24));
             ok = seen >= target;
         }
         __syncwarp();  // the other lanes' loads follow the acquire
