@@ -43,12 +43,13 @@ struct GridParams {
     double margin;      // absolute slack for the geometric pruning tests
     double inv_fix;     // kFix / cell
     int G;              // cells per axis (G x G cells)
-    int fast;           // every coordinate is finite: the fixed-point search applies
+    int fast;           // the fixed-point search applies (see grid_setup_kernel)
 };
 
 // Fixed-point grid coordinates: units per cell.
 constexpr int kFixBits = 12;
 constexpr int kFix = 1 << kFixBits;
+constexpr double kFastMinCell = 1e-140, kFastMaxSpan = 1e150;  // where it is used
 
 struct Box {
     double mnx, mny, mxx, mxy;
@@ -120,7 +121,12 @@ __global__ void __launch_bounds__(kBoxBlocks) grid_setup_kernel(const Box* __res
     }
     double x0 = r.mnx, y0 = r.mny;
     double span = fmax(r.mxx - r.mnx, r.mxy - r.mny);
-    const bool finite_box = r.odd == 0.0 && x0 <= r.mxx && y0 <= r.mxy;
+    // The fixed-point search takes the nearest points of the plane, the order
+    // of a stencil is that of the rounded d^2.  The two agree while every d^2
+    // it can meet is far inside the normal range: from the square of one unit
+    // (cell / kFix), where an underflow would turn the geometry's order into
+    // ties that the index decides, to that of the whole span.
+    const bool in_range = r.odd == 0.0 && x0 <= r.mxx && y0 <= r.mxy && span < kFastMaxSpan;
     if (!(x0 > -INFINITY && x0 < INFINITY)) x0 = 0.0;  // no finite point
     if (!(y0 > -INFINITY && y0 < INFINITY)) y0 = 0.0;
     if (!(span > 0.0 && span < INFINITY)) span = 1.0;    // single point / degenerate
@@ -132,11 +138,12 @@ __global__ void __launch_bounds__(kBoxBlocks) grid_setup_kernel(const Box* __res
     p.margin = 1e-12 * (span + fabs(x0) + fabs(y0));
     p.inv_fix = p.inv_cell * kFix;
     p.G = G;
-    p.fast = finite_box && p.cell > 0.0 && p.inv_fix < INFINITY ? 1 : 0;
+    p.fast = in_range && p.cell > kFastMinCell ? 1 : 0;
     *gp = p;
 }
 
-// Coordinate in units of cell / kFix, rounded down (NaN: 0; saturating).
+// Coordinate in units of cell / kFix, rounded down and saturating (fix_cell
+// clamps whatever a NaN becomes).
 __device__ __forceinline__ int fix_coord(double v, double v0, double inv_fix) {
     return __double2int_rd((v - v0) * inv_fix);
 }
