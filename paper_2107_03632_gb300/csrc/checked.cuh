@@ -33,6 +33,8 @@
 
 #include <type_traits>
 
+#include "live.cuh"
+
 namespace rbffd {
 
 // FNV-1a (32-bit) hash of the base name of a path: identifies the source
@@ -81,6 +83,11 @@ __device__ __forceinline__ T& rb_chk_at(T* p, I i, long long n, uint32_t file, i
     if ((unsigned long long)k < (unsigned long long)n) return p[k];
     rb_chk_fail(file, line, k, n);
     return *reinterpret_cast<T*>(rb_chk_sink);
+}
+
+template <class T, class I>
+__device__ __forceinline__ T rb_chk_at(::rbffd::Live<T> v, I i, long long n, uint32_t file, int line) {
+    return rb_chk_at(v.p, i, n, file, line);
 }
 
 __device__ __forceinline__ void rb_chk_span(long long off, long long len, long long n, uint32_t file, int line) {

@@ -70,7 +70,10 @@ inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s
 // chain calls pdl_wait() in every thread before it touches anything the chain
 // writes and before it may return, and pdl_next() only after that (so at most
 // two kernels overlap); the first kernel of a chain is not `chained`, so what
-// is read before the wait was written by kernels that had completed.
+// is read before the wait was written by kernels that had completed; what the
+// chain writes is read through Live<T> and written through plain pointers
+// (live.cuh), and __ldg and __restrict__ are for what no kernel of the chain
+// writes (matrices, indices, scalings, the source).
 template <class... P, class... A>
 inline cudaError_t launch_chained(bool chained, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem,
                                   cudaStream_t st, A&&... args) {

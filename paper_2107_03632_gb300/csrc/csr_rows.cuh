@@ -39,8 +39,7 @@ __device__ __forceinline__ T rows32_exchange(T (&s)[TPR], int sub) {
 // per row, or fewer and several passes).
 template <typename T, int TPR, class F>
 __device__ __forceinline__ void rows32(const int64_t* __restrict__ row_ptr, const int* __restrict__ col,
-                                       const T* __restrict__ val, const T* __restrict__ x, int64_t nx, int64_t N,
-                                       F&& f) {
+                                       const T* __restrict__ val, Live<T> x, int64_t nx, int64_t N, F&& f) {
     (void)nx;  // length of x: bound of the checked build's tests
     constexpr int G = 32 / TPR;
     const int lane = (int)(threadIdx.x & 31), sub = lane & (TPR - 1), g = lane / TPR;
@@ -58,7 +57,7 @@ __device__ __forceinline__ void rows32(const int64_t* __restrict__ row_ptr, cons
             T t = T(0);
 #pragma unroll 4
             for (int64_t k = a + sub; k < e; k += TPR)
-                t = fma_of(__ldg(val + k), __ldg(&RB_AT(x, __ldg(col + k), nx)), t);
+                t = fma_of(__ldg(val + k), RB_AT(x, __ldg(col + k), nx), t);
             s[j] = t;
         }
         const T t = rows32_exchange<T, TPR>(s, sub);
@@ -74,8 +73,7 @@ __device__ __forceinline__ void rows32(const int64_t* __restrict__ row_ptr, cons
 // entries.  For float32: in FP64 the 64 registers more cost what it gives.
 template <typename T, int TPR, class F>
 __device__ __forceinline__ void rows32_ahead(const int64_t* __restrict__ row_ptr, const int* __restrict__ col,
-                                             const T* __restrict__ val, const T* __restrict__ x, int64_t nx,
-                                             int64_t N, F&& f) {
+                                             const T* __restrict__ val, Live<T> x, int64_t nx, int64_t N, F&& f) {
     (void)nx;  // length of x: bound of the checked build's tests
     constexpr int G = 32 / TPR, U = 4;
     const int lane = (int)(threadIdx.x & 31), sub = lane & (TPR - 1), g = lane / TPR;
@@ -116,7 +114,7 @@ __device__ __forceinline__ void rows32_ahead(const int64_t* __restrict__ row_ptr
             const int64_t kj = k, cj = cnt;
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                xv[u] = u * TPR < cj ? __ldg(&RB_AT(x, c[u], nx)) : T(0);
+                xv[u] = u * TPR < cj ? RB_AT(x, c[u], nx) : T(0);
                 w[u] = v[u];
             }
             if (j + 1 == TPR) {
@@ -129,7 +127,7 @@ __device__ __forceinline__ void rows32_ahead(const int64_t* __restrict__ row_ptr
             for (int u = 0; u < U; ++u)
                 if (u * TPR < cj) t = fma_of(w[u], xv[u], t);
             for (int64_t o = U * TPR; o < cj; o += TPR)
-                t = fma_of(__ldg(val + kj + o), __ldg(&RB_AT(x, __ldg(col + kj + o), nx)), t);
+                t = fma_of(__ldg(val + kj + o), RB_AT(x, __ldg(col + kj + o), nx), t);
             s[j] = t;
         }
         const T t = rows32_exchange<T, TPR>(s, sub);

@@ -92,14 +92,8 @@ __device__ __forceinline__ df df_from_double(double v) {
 __device__ __forceinline__ double df_to_double(df a) { return (double)a.hi + (double)a.lo; }
 
 // float2 storage of a df value (hi in .x, lo in .y): 8 bytes, like a double.
-__device__ __forceinline__ df df_load(const float2* p) {
-    const float2 v = *p;
-    return df_make(v.x, v.y);
-}
-__device__ __forceinline__ df df_ldg(const float2* p) {
-    const float2 v = __ldg(p);
-    return df_make(v.x, v.y);
-}
+__device__ __forceinline__ df df_of(float2 v) { return df_make(v.x, v.y); }
+__device__ __forceinline__ df df_load(const float2* p) { return df_of(*p); }
 __device__ __forceinline__ void df_store(float2* p, df a) { *p = make_float2(a.hi, a.lo); }
 
 __device__ __forceinline__ df df_shfl_xor(df a, int o, int width) {

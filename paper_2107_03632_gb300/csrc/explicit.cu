@@ -106,11 +106,10 @@ __global__ void __launch_bounds__(kT) explicit_step_kernel(const int32_t* __rest
 constexpr int kSmallT = 64;
 template <int U>
 __global__ void __launch_bounds__(kSmallT) explicit_step_small_kernel(const int32_t* __restrict__ rows,
-                                                           const int32_t* __restrict__ idxT,
-                                                           const double* __restrict__ wT, int64_t Ni, int n,
-                                                           const double* __restrict__ f, double dt,
-                                                           const double* __restrict__ u1, double* __restrict__ u2,
-                                                           int64_t N) {
+                                                                      const int32_t* __restrict__ idxT,
+                                                                      const double* __restrict__ wT, int64_t Ni, int n,
+                                                                      const double* __restrict__ f, double dt,
+                                                                      Live<double> u1, double* u2, int64_t N) {
     (void)N;  // nodes: bound of the checked build's tests
     int c[U];
     double w[U];
@@ -139,7 +138,7 @@ __global__ void __launch_bounds__(kSmallT) explicit_step_small_kernel(const int3
         if (j0 > 0) load(r, j0);
         double u[U];
 #pragma unroll
-        for (int j = 0; j < U; ++j) u[j] = j0 + j < n ? __ldg(&RB_AT(u1, c[j], N)) : 0.0;
+        for (int j = 0; j < U; ++j) u[j] = j0 + j < n ? RB_AT(u1, c[j], N) : 0.0;
 #pragma unroll
         for (int j = 0; j < U; ++j)
             if (j0 + j < n) lap = fma(w[j], u[j], lap);

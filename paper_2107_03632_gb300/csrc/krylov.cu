@@ -194,8 +194,8 @@ __device__ __forceinline__ void set_omega(KState* st, double ts, double tt, doub
 // sum_k a_k x[col_k] over one row, TPR lanes (result in every lane).
 template <int TPR>
 __device__ __forceinline__ double row_dot64(const int64_t* __restrict__ row_ptr, const int* __restrict__ col,
-                                            const double* __restrict__ val, const double* __restrict__ x,
-                                            int64_t nx, int64_t row, int sub, bool valid) {
+                                            const double* __restrict__ val, Live<double> x, int64_t nx, int64_t row,
+                                            int sub, bool valid) {
     (void)nx;  // length of x: bound of the checked build's tests
     int64_t a = 0, e = 0;
     if (valid) {
@@ -204,7 +204,7 @@ __device__ __forceinline__ double row_dot64(const int64_t* __restrict__ row_ptr,
     }
     double sum = 0.0;
 #pragma unroll 4
-    for (int64_t k = a + sub; k < e; k += TPR) sum = fma(__ldg(val + k), __ldg(&RB_AT(x, __ldg(col + k), nx)), sum);
+    for (int64_t k = a + sub; k < e; k += TPR) sum = fma(__ldg(val + k), RB_AT(x, __ldg(col + k), nx), sum);
 #pragma unroll
     for (int o = TPR / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o, TPR);
     return sum;
@@ -463,8 +463,7 @@ __global__ void __launch_bounds__(kThreads) resid64_kernel(const int64_t* __rest
     }
 }
 
-__global__ void __launch_bounds__(kThreads) update_p64_kernel(int64_t N, const double* __restrict__ r,
-                                                              const double* __restrict__ v, double* __restrict__ p,
+__global__ void __launch_bounds__(kThreads) update_p64_kernel(int64_t N, Live<double> r, Live<double> v, double* p,
                                                               const KState* st) {
     pdl_wait();
     pdl_next();
@@ -480,12 +479,10 @@ __global__ void __launch_bounds__(kThreads) update_p64_kernel(int64_t N, const d
 // (dotv); dotv NULL: xin.
 template <int TPR, int MODE>
 __global__ void __launch_bounds__(kThreads) spmv64_kernel(const int64_t* __restrict__ row_ptr,
-                                                          const int* __restrict__ col,
-                                                          const double* __restrict__ val, int64_t N,
-                                                          const double* __restrict__ xin,
-                                                          const double* __restrict__ dinv, double* __restrict__ y,
-                                                          const double* __restrict__ rh, KState* st, double* part,
-                                                          const double* __restrict__ dotv) {
+                                                          const int* __restrict__ col, const double* __restrict__ val,
+                                                          int64_t N, Live<double> xin, const double* __restrict__ dinv,
+                                                          double* y, Live<double> rh, KState* st, double* part,
+                                                          Live<double> dotv) {
     pdl_wait();
     pdl_next();
     if (st->flag != kRunning) return;
@@ -494,12 +491,13 @@ __global__ void __launch_bounds__(kThreads) spmv64_kernel(const int64_t* __restr
     RBFFD_ROW_LOOP(TPR, N, i, valid, {
         const double ax = row_dot64<TPR>(row_ptr, col, val, xin, N, i, sub, valid);
         if (valid && sub == 0) {
+            // (loads first: a store may alias them)
+            const double si = MODE == 0 ? rh[i] : MODE == 1 ? (dotv ? dotv[i] : xin[i]) : 0.0;
             const double yi = ax * dinv[i];
             y[i] = yi;
             if (MODE == 0) {
-                acc[0] = fma(rh[i], yi, acc[0]);
+                acc[0] = fma(si, yi, acc[0]);
             } else if (MODE == 1) {
-                const double si = dotv ? dotv[i] : xin[i];
                 acc[0] = fma(yi, si, acc[0]);
                 acc[1] = fma(yi, yi, acc[1]);
                 acc[2] = fma(si, si, acc[2]);
@@ -521,8 +519,8 @@ __global__ void __launch_bounds__(kThreads) spmv64_kernel(const int64_t* __restr
 // SpMV kernels fuse in the right-preconditioned form.  MODE 0: (rh, v) ->
 // alpha.  MODE 1: (t, s), (t, t), (s, s) -> omega.
 template <int MODE>
-__global__ void __launch_bounds__(kThreads) dot64_kernel(int64_t N, const double* __restrict__ a,
-                                                         const double* __restrict__ b, KState* st, double* part) {
+__global__ void __launch_bounds__(kThreads) dot64_kernel(int64_t N, Live<double> a, Live<double> b, KState* st,
+                                                         double* part) {
     pdl_wait();
     pdl_next();
     if (st->flag != kRunning) return;
@@ -575,8 +573,7 @@ __global__ void __launch_bounds__(kThreads) left_init_kernel(int64_t N, const do
     }
 }
 
-__global__ void __launch_bounds__(kThreads) update_s64_kernel(int64_t N, const double* __restrict__ r,
-                                                              const double* __restrict__ v, double* __restrict__ s,
+__global__ void __launch_bounds__(kThreads) update_s64_kernel(int64_t N, Live<double> r, Live<double> v, double* s,
                                                               const KState* st) {
     pdl_wait();
     pdl_next();
@@ -605,26 +602,23 @@ __device__ __forceinline__ void finish_iteration(KState* st, double rn2, double 
 
 // x += alpha p + omega sx (sx = M^-1 s with right preconditioning, else s),
 // r = s - omega t.
-__global__ void __launch_bounds__(kThreads) update_xr64_kernel(int64_t N, double* __restrict__ x,
-                                                               const double* __restrict__ p,
-                                                               const double* __restrict__ s,
-                                                               const double* __restrict__ t, double* __restrict__ r,
-                                                               const double* __restrict__ rh,
-                                                               const double* __restrict__ d, KState* st,
-                                                               double* part, const double* __restrict__ sx) {
+__global__ void __launch_bounds__(kThreads) update_xr64_kernel(int64_t N, double* x, Live<double> p, Live<double> s,
+                                                               Live<double> t, double* r, Live<double> rh,
+                                                               const double* __restrict__ d, KState* st, double* part,
+                                                               Live<double> sx) {
     pdl_wait();
     pdl_next();
     if (st->flag != kRunning) return;
     const double alpha = st->alpha, omega = st->omega;
     double acc[3] = {0.0, 0.0, 0.0};
     RBFFD_ELEM_LOOP(N, i) {
-        const double si = s[i];
-        x[i] = fma(omega, sx ? sx[i] : si, fma(alpha, p[i], x[i]));
-        const double ri = fma(-omega, t[i], si);
+        // (loads first: a store may alias them)
+        const double si = s[i], ti = t[i], pi = p[i], hi = rh[i], xi = x[i], mi = sx ? sx[i] : si;
+        const double ri = fma(-omega, ti, si), ru = ri * d[i];
+        x[i] = fma(omega, mi, fma(alpha, pi, xi));
         r[i] = ri;
-        const double ru = ri * d[i];
         acc[0] = fma(ru, ru, acc[0]);
-        acc[1] = fma(rh[i], ri, acc[1]);
+        acc[1] = fma(hi, ri, acc[1]);
         acc[2] = fma(ri, ri, acc[2]);
     }
     double tot[3];
@@ -929,8 +923,8 @@ __global__ void __launch_bounds__(kPassT) pass64_kernel(const int64_t* __restric
 // accumulation (result in every lane).
 template <int TPR>
 __device__ __forceinline__ df row_apply_df(const int64_t* __restrict__ row_ptr, const int* __restrict__ col,
-                                           const float* __restrict__ val, const float2* __restrict__ x,
-                                           int64_t nx, int64_t row, int sub, bool valid, df xi) {
+                                           const float* __restrict__ val, Live<float2> x, int64_t nx, int64_t row,
+                                           int sub, bool valid, df xi) {
     (void)nx;  // length of x: bound of the checked build's tests
     int64_t a = 0, e = 0;
     if (valid) {
@@ -941,7 +935,7 @@ __device__ __forceinline__ df row_apply_df(const int64_t* __restrict__ row_ptr, 
 #pragma unroll 4
     for (int64_t k = a + sub; k < e; k += TPR) {
         const float w = __ldg(val + k);
-        const df xj = df_ldg(&RB_AT(x, __ldg(col + k), nx));
+        const df xj = df_of(RB_AT(x, __ldg(col + k), nx));
         // d_j - d_i as an unnormalised pair: the rounding of the leading
         // difference is at most eps_32 of that difference (exact when the
         // two values are within a factor 2), so no cancellation is lost
@@ -1002,17 +996,16 @@ __global__ void __launch_bounds__(kThreads) load_df_kernel(int64_t N, const doub
     }
 }
 
-__global__ void __launch_bounds__(kThreads) update_p_df_kernel(int64_t N, const float2* __restrict__ r,
-                                                               const float2* __restrict__ v,
-                                                               float2* __restrict__ p, const KState* st) {
+__global__ void __launch_bounds__(kThreads) update_p_df_kernel(int64_t N, Live<float2> r, Live<float2> v, float2* p,
+                                                               const KState* st) {
     pdl_wait();
     pdl_next();
     if (st->flag != kRunning) return;
     const df beta = df_from_double((st->rho_new / st->rho) * (st->alpha / st->omega));
     const df nomega = df_from_double(-st->omega);
     RBFFD_ELEM_LOOP(N, i) {
-        const df t = df_fma(nomega, df_load(v + i), df_load(p + i));
-        df_store(p + i, df_fma(beta, t, df_load(r + i)));
+        const df t = df_fma(nomega, df_of(v[i]), df_load(p + i));
+        df_store(p + i, df_fma(beta, t, df_of(r[i])));
     }
 }
 
@@ -1020,12 +1013,9 @@ __global__ void __launch_bounds__(kThreads) update_p_df_kernel(int64_t N, const 
 // (y, xin), (y, y) -> omega.
 template <int TPR, int MODE>
 __global__ void __launch_bounds__(kThreads) spmv_df_kernel(const int64_t* __restrict__ row_ptr,
-                                                           const int* __restrict__ col,
-                                                           const float* __restrict__ val, int64_t N,
-                                                           const float2* __restrict__ xin,
-                                                           const float* __restrict__ sigma,
-                                                           const float* __restrict__ dinv,
-                                                           float2* __restrict__ y, const float2* __restrict__ rh,
+                                                           const int* __restrict__ col, const float* __restrict__ val,
+                                                           int64_t N, Live<float2> xin, const float* __restrict__ sigma,
+                                                           const float* __restrict__ dinv, float2* y, Live<float2> rh,
                                                            KState* st, double* part) {
     pdl_wait();
     pdl_next();
@@ -1033,14 +1023,15 @@ __global__ void __launch_bounds__(kThreads) spmv_df_kernel(const int64_t* __rest
     const int sub = threadIdx.x & (TPR - 1);
     DfAcc a0, a1, a2;
     RBFFD_ROW_LOOP(TPR, N, i, valid, {
-        const df xi = valid ? df_ldg(xin + i) : df_make(0.f, 0.f);
+        const df xi = valid ? df_of(xin[i]) : df_make(0.f, 0.f);
         df ax = row_apply_df<TPR>(row_ptr, col, val, xin, N, i, sub, valid, xi);
         if (valid && sub == 0) {
             ax = df_add(ax, df_mul_f(xi, sigma[i]));
             const df yi = df_mul_f(ax, dinv[i]);
+            const df hi = MODE == 0 ? df_of(rh[i]) : xi;  // (before the store, which may alias it)
             df_store(y + i, yi);
             if (MODE == 0) {
-                a0.add(df_mul(df_load(rh + i), yi));
+                a0.add(df_mul(hi, yi));
             } else {
                 a0.add(df_mul(yi, xi));
                 a1.add(df_mul(yi, yi));
@@ -1066,22 +1057,17 @@ __global__ void __launch_bounds__(kThreads) spmv_df_kernel(const int64_t* __rest
     }
 }
 
-__global__ void __launch_bounds__(kThreads) update_s_df_kernel(int64_t N, const float2* __restrict__ r,
-                                                               const float2* __restrict__ v,
-                                                               float2* __restrict__ s, const KState* st) {
+__global__ void __launch_bounds__(kThreads) update_s_df_kernel(int64_t N, Live<float2> r, Live<float2> v, float2* s,
+                                                               const KState* st) {
     pdl_wait();
     pdl_next();
     if (st->flag != kRunning) return;
     const df nalpha = df_from_double(-st->alpha);
-    RBFFD_ELEM_LOOP(N, i) df_store(s + i, df_fma(nalpha, df_load(v + i), df_load(r + i)));
+    RBFFD_ELEM_LOOP(N, i) df_store(s + i, df_fma(nalpha, df_of(v[i]), df_of(r[i])));
 }
 
-__global__ void __launch_bounds__(kThreads) update_xr_df_kernel(int64_t N, float2* __restrict__ x,
-                                                                const float2* __restrict__ p,
-                                                                const float2* __restrict__ s,
-                                                                const float2* __restrict__ t,
-                                                                float2* __restrict__ r,
-                                                                const float2* __restrict__ rh,
+__global__ void __launch_bounds__(kThreads) update_xr_df_kernel(int64_t N, float2* x, Live<float2> p, Live<float2> s,
+                                                                Live<float2> t, float2* r, Live<float2> rh,
                                                                 const float* __restrict__ d, KState* st,
                                                                 double* part) {
     pdl_wait();
@@ -1091,13 +1077,13 @@ __global__ void __launch_bounds__(kThreads) update_xr_df_kernel(int64_t N, float
     const df nomega = df_from_double(-st->omega);
     DfAcc a0, a1, a2;
     RBFFD_ELEM_LOOP(N, i) {
-        const df si = df_load(s + i);
-        df_store(x + i, df_fma(omega, si, df_fma(alpha, df_load(p + i), df_load(x + i))));
-        const df ri = df_fma(nomega, df_load(t + i), si);
+        // (loads first: a store may alias them)
+        const df si = df_of(s[i]), ti = df_of(t[i]), pi = df_of(p[i]), hi = df_of(rh[i]), xi = df_load(x + i);
+        const df ri = df_fma(nomega, ti, si), ru = df_mul_f(ri, d[i]);
+        df_store(x + i, df_fma(omega, si, df_fma(alpha, pi, xi)));
         df_store(r + i, ri);
-        const df ru = df_mul_f(ri, d[i]);
         a0.add(df_mul(ru, ru));
-        a1.add(df_mul(df_load(rh + i), ri));
+        a1.add(df_mul(hi, ri));
         a2.add(df_mul(ri, ri));
     }
     double acc[3] = {df_to_double(a0.value()), df_to_double(a1.value()), df_to_double(a2.value())}, tot[3];

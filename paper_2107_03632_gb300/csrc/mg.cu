@@ -89,8 +89,8 @@ __device__ __forceinline__ float fmaT<float>(float a, float b, float c) {
 
 template <typename T, int TPR>
 __device__ __forceinline__ T row_sum(const int64_t* __restrict__ row_ptr, const int* __restrict__ col,
-                                     const T* __restrict__ val, const T* __restrict__ x, int64_t nx, int64_t row,
-                                     int sub, bool valid) {
+                                     const T* __restrict__ val, Live<T> x, int64_t nx, int64_t row, int sub,
+                                     bool valid) {
     (void)nx;  // length of x: bound of the checked build's tests
     int64_t a = 0, e = 0;
     if (valid) {
@@ -99,7 +99,7 @@ __device__ __forceinline__ T row_sum(const int64_t* __restrict__ row_ptr, const 
     }
     T sum = T(0);
 #pragma unroll 4
-    for (int64_t k = a + sub; k < e; k += TPR) sum = fmaT<T>(__ldg(val + k), __ldg(&RB_AT(x, __ldg(col + k), nx)), sum);
+    for (int64_t k = a + sub; k < e; k += TPR) sum = fmaT<T>(__ldg(val + k), RB_AT(x, __ldg(col + k), nx), sum);
 #pragma unroll
     for (int o = TPR / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o, TPR);
     return sum;
@@ -129,19 +129,19 @@ struct RowHead {
             v[u] = k < e ? __ldg(val + k) : T(0);
         }
     }
-    __device__ __forceinline__ T sum(const int* __restrict__ col, const T* __restrict__ val,
-                                     const T* __restrict__ x, int64_t nx, int sub) const {
+    __device__ __forceinline__ T sum(const int* __restrict__ col, const T* __restrict__ val, Live<T> x, int64_t nx,
+                                     int sub) const {
         (void)nx;  // length of x: bound of the checked build's tests
         T xv[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) xv[u] = a + sub + u * TPR < e ? __ldg(&RB_AT(x, c[u], nx)) : T(0);
+        for (int u = 0; u < U; ++u) xv[u] = a + sub + u * TPR < e ? RB_AT(x, c[u], nx) : T(0);
         T s = T(0);
 #pragma unroll
         for (int u = 0; u < U; ++u)
             if (a + sub + u * TPR < e) s = fmaT<T>(v[u], xv[u], s);
 #pragma unroll 4
         for (int64_t k = a + sub + U * TPR; k < e; k += TPR)
-            s = fmaT<T>(__ldg(val + k), __ldg(&RB_AT(x, __ldg(col + k), nx)), s);
+            s = fmaT<T>(__ldg(val + k), RB_AT(x, __ldg(col + k), nx), s);
 #pragma unroll
         for (int o = TPR / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, TPR);
         return s;
@@ -156,8 +156,8 @@ struct RowHead {
 enum RowForm { kRowEach = 0, kRowHead = 1, kRow32 = 2 };
 template <typename T, int TPR, int FORM, class F>
 __device__ __forceinline__ void chained_rows(const int64_t* __restrict__ row_ptr, const int* __restrict__ col,
-                                             const T* __restrict__ val, int64_t N, const T* __restrict__ x,
-                                             int64_t nx, const int* flag, F&& f) {
+                                             const T* __restrict__ val, int64_t N, Live<T> x, int64_t nx,
+                                             const int* flag, F&& f) {
     const int sub = threadIdx.x & (TPR - 1);
     if constexpr (FORM == kRow32) {
         pdl_wait();
@@ -187,8 +187,8 @@ __device__ __forceinline__ void chained_rows(const int64_t* __restrict__ row_ptr
 
 // x = W b (the first sweep from x = 0); dinv holds W = Omega D^-1
 template <typename T, typename BT>
-__global__ void __launch_bounds__(kT) mg_first_kernel(int64_t N, const BT* __restrict__ b, const T* __restrict__ dinv,
-                                                      T* __restrict__ x, const int* flag) {
+__global__ void __launch_bounds__(kT) mg_first_kernel(int64_t N, Live<BT> b, const T* __restrict__ dinv, T* x,
+                                                      const int* flag) {
     pdl_wait();
     pdl_next();
     if (stopped(flag)) return;
@@ -198,9 +198,8 @@ __global__ void __launch_bounds__(kT) mg_first_kernel(int64_t N, const BT* __res
 // xo = xi + W (b - A xi)
 template <typename T, typename BT, typename OT, int TPR, int FORM>
 __global__ void __launch_bounds__(kT) mg_jacobi_kernel(const int64_t* __restrict__ row_ptr, const int* __restrict__ col,
-                                                       const T* __restrict__ val, int64_t N, const T* __restrict__ xi,
-                                                       const BT* __restrict__ b, const T* __restrict__ dinv,
-                                                       OT* __restrict__ xo, const int* flag) {
+                                                       const T* __restrict__ val, int64_t N, Live<T> xi, Live<BT> b,
+                                                       const T* __restrict__ dinv, OT* xo, const int* flag) {
     chained_rows<T, TPR, FORM>(row_ptr, col, val, N, xi, N, flag,
                          [&](int64_t i, T ax) { xo[i] = (OT)fmaT<T>(dinv[i], (T)b[i] - ax, xi[i]); });
 }
@@ -208,8 +207,8 @@ __global__ void __launch_bounds__(kT) mg_jacobi_kernel(const int64_t* __restrict
 // r = b - A x
 template <typename T, typename BT, int TPR, int FORM>
 __global__ void __launch_bounds__(kT) mg_resid_kernel(const int64_t* __restrict__ row_ptr, const int* __restrict__ col,
-                                                      const T* __restrict__ val, int64_t N, const T* __restrict__ x,
-                                                      const BT* __restrict__ b, T* __restrict__ r, const int* flag) {
+                                                      const T* __restrict__ val, int64_t N, Live<T> x, Live<BT> b, T* r,
+                                                      const int* flag) {
     chained_rows<T, TPR, FORM>(row_ptr, col, val, N, x, N, flag, [&](int64_t i, T ax) { r[i] = (T)b[i] - ax; });
 }
 
@@ -217,8 +216,7 @@ __global__ void __launch_bounds__(kT) mg_resid_kernel(const int64_t* __restrict_
 template <typename T, int TPR, int FORM>
 __global__ void __launch_bounds__(kT) mg_restrict_kernel(const int64_t* __restrict__ row_ptr,
                                                          const int* __restrict__ col, const T* __restrict__ val,
-                                                         int64_t n, const T* __restrict__ r, int64_t nr,
-                                                         T* __restrict__ y, const int* flag) {
+                                                         int64_t n, Live<T> r, int64_t nr, T* y, const int* flag) {
     chained_rows<T, TPR, FORM>(row_ptr, col, val, n, r, nr, flag, [&](int64_t i, T v) { y[i] = v; });
 }
 
@@ -249,8 +247,8 @@ struct PRow {
 // x += P e; the first row's entries are loaded before the wait
 template <typename T>
 __global__ void __launch_bounds__(kT) mg_prolong_kernel(int64_t N, const int32_t* __restrict__ pidx,
-                                                        const T* __restrict__ pval, const T* __restrict__ e,
-                                                        int64_t ne, T* __restrict__ x, const int* flag) {
+                                                        const T* __restrict__ pval, Live<T> e, int64_t ne, T* x,
+                                                        const int* flag) {
     (void)ne;  // length of e: bound of the checked build's tests
     const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     PRow<T> p;
@@ -262,15 +260,15 @@ __global__ void __launch_bounds__(kT) mg_prolong_kernel(int64_t N, const int32_t
         if (i != i0) p = PRow<T>(pidx, pval, i);
         T acc = x[i];
 #pragma unroll
-        for (int j = 0; j < kMgK; ++j) acc = fmaT<T>(p.v[j], __ldg(&RB_AT(e, p.c[j], ne)), acc);
+        for (int j = 0; j < kMgK; ++j) acc = fmaT<T>(p.v[j], RB_AT(e, p.c[j], ne), acc);
         x[i] = acc;
     }
 }
 
 // x = Minv b, one warp per row
 template <typename T, typename BT, typename OT>
-__global__ void __launch_bounds__(kT) mg_dense_kernel(int n, const T* __restrict__ minv, const BT* __restrict__ b,
-                                                      OT* __restrict__ x, const int* flag) {
+__global__ void __launch_bounds__(kT) mg_dense_kernel(int n, const T* __restrict__ minv, Live<BT> b, OT* x,
+                                                      const int* flag) {
     pdl_wait();
     pdl_next();
     if (stopped(flag)) return;
@@ -394,7 +392,7 @@ __global__ void __launch_bounds__(kT) mg_gather_kernel(const double2* __restrict
 __global__ void __launch_bounds__(kT) mg_bfix_kernel(const int64_t* __restrict__ row_ptr, const int* __restrict__ col,
                                                      const double* __restrict__ val, int64_t N,
                                                      const uint8_t* __restrict__ mask, const double* __restrict__ w,
-                                                     const double* __restrict__ r, double* y, const int* flag) {
+                                                     Live<double> r, double* y, const int* flag) {
     pdl_wait();
     pdl_next();
     if (stopped(flag)) return;
@@ -1273,7 +1271,7 @@ struct TailCycle {
     int a_ptr[kTailLevels], a_col[kTailLevels], a_val[kTailLevels];
     int r_ptr[kTailLevels], r_col[kTailLevels], r_val[kTailLevels];
     const T* minv;
-    const T* b;  // right-hand side and result of the first level (not TOP)
+    Live<T> b;  // right-hand side and result of the first level (not TOP)
     T* x;
     TailLevel<T> lv[kTailLevels];
 };
@@ -1323,9 +1321,8 @@ __device__ __forceinline__ void tail_csr(int tpr, const RP* row_ptr, const CP* c
 // TOP: level 0 is the first one, its right-hand side and result are the
 // caller's FP64 vectors.
 template <typename T, bool TOP>
-__global__ void __launch_bounds__(kTailT) mg_tail_kernel(const __grid_constant__ TailCycle<T> c,
-                                                         const double* __restrict__ b64, double* __restrict__ x64,
-                                                         const int* flag) {
+__global__ void __launch_bounds__(kTailT) mg_tail_kernel(const __grid_constant__ TailCycle<T> c, Live<double> b64,
+                                                         double* x64, const int* flag) {
     extern __shared__ __align__(16) unsigned char tail_smem[];
     T* vec = reinterpret_cast<T*>(tail_smem);  // per level: two iterates, residual, right-hand side
     const int tid = (int)threadIdx.x, last = c.levels - 1;
@@ -1621,8 +1618,8 @@ int mg_dirichlet_fix(const MgHierarchy* h, const double* r, double* y, const int
     return RBFFD_OK;
 }
 
-__global__ void __launch_bounds__(kT) mg_zero_dirichlet_kernel(int64_t N, const uint8_t* __restrict__ mask,
-                                                               double* __restrict__ y, const int* flag) {
+__global__ void __launch_bounds__(kT) mg_zero_dirichlet_kernel(int64_t N, const uint8_t* __restrict__ mask, double* y,
+                                                               const int* flag) {
     pdl_wait();
     pdl_next();
     if (stopped(flag)) return;
