@@ -90,6 +90,21 @@ inline cudaError_t launch_chained(bool chained, void (*kernel)(P...), unsigned g
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
+// Allows a kernel all the dynamic shared memory that its static part leaves.
+// The attribute belongs to the kernel, not to a launch, so it never takes the
+// size of the launch at hand: two threads that launch the same kernel with
+// different sizes would take each other's permission away between setting it
+// and launching.
+template <class K>
+inline cudaError_t allow_dynamic_smem(K* kernel) {
+    constexpr int kBlockSmem = 227 * 1024;
+    cudaFuncAttributes a{};
+    const cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                kBlockSmem - (int)a.sharedSizeBytes);
+}
+
 // Number of SMs of the current device (cached per device).
 int sm_count();
 

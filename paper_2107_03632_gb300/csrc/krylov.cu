@@ -651,6 +651,7 @@ constexpr int kPassSmemEntries = 10240;  // entries per block held in shared mem
 constexpr int kPassSlot = 4;           // slots of `part` for the three reductions: 4, 5, 6
 constexpr int kPassFlagSlot = 7;       // the blocks' arrivals so far
 constexpr int kPassVecs = 9;
+constexpr int kPassMaxSmem = 220 * 1024;  // (beside the kernel's static shared memory)
 static_assert(kPassFlagSlot < kSlots && kPassSlot + 3 <= kPassFlagSlot, "partial-sum slots");
 
 inline size_t pass_smem(int rows) {
@@ -1379,8 +1380,8 @@ bool pass64(const rbffd_csr& A, double* x, const Work& w, int count, cudaStream_
     if (w.mg || profiling() || A.nnz > (int64_t)sms * kPassEntries) return false;
     const int rows = (int)std::max<int64_t>(kPassRows, (A.n_rows + sms - 1) / sms);
     const size_t smem = pass_smem(rows);
-    if (smem > 220 * 1024) return false;
-    if (cudaFuncSetAttribute(pass64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+    if (smem > kPassMaxSmem) return false;
+    if (allow_dynamic_smem(pass64_kernel) != cudaSuccess ||
         cudaMemsetAsync(part_at(w.part, kPassFlagSlot, 0), 0, sizeof(unsigned int), st) != cudaSuccess) {
         (void)cudaGetLastError();
         return false;

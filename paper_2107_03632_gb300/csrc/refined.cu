@@ -886,7 +886,7 @@ int launch(const double2* xy, const int32_t* idx, int64_t N, int n, double* w, i
         }
     }
     const size_t smem = (size_t)spb * g.bytes;
-    RBFFD_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    RBFFD_CUDA_TRY(allow_dynamic_smem(kern));
     RBFFD_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
     int per_sm = 0;
     RBFFD_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, TT * spb, smem));

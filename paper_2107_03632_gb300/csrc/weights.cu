@@ -1156,7 +1156,7 @@ int launch_ns(const WCfg& c, const double2* xy, const int32_t* idx, int64_t N, i
     const int spb = stencils_per_block(c);
     const size_t smem = block_smem(c, n, m);
     auto kern = weights_ns_kernel<NT, R, MARKED>;
-    RBFFD_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    RBFFD_CUDA_TRY(allow_dynamic_smem(kern));
     RBFFD_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
     int per_sm = 0;
     RBFFD_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT * spb, smem));
@@ -1188,7 +1188,7 @@ int launch_weights(const WCfg& c, const double* xy, const int32_t* idx, int64_t 
         WeightsGeom g = weights_geom(n, m);
         const int wpb = c.wpb;
         const size_t smem = block_smem(c, n, m);
-        RBFFD_CUDA_TRY(cudaFuncSetAttribute(weights_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        RBFFD_CUDA_TRY(allow_dynamic_smem(weights_kernel));
         RBFFD_CUDA_TRY(cudaFuncSetAttribute(weights_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
         int per_sm = 0;
         RBFFD_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, weights_kernel, 32 * wpb, smem));
@@ -1414,7 +1414,7 @@ int rbffd::interp_weights(const double* xy, int64_t Nd, const double* qxy, int64
     size_t smem = 0;
     const int wpb = weights_warps_per_block(g, &smem);
     if (smem > 227 * 1024) return RBFFD_ERR_INVALID_ARG;
-    RBFFD_CUDA_TRY(cudaFuncSetAttribute(weights_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    RBFFD_CUDA_TRY(allow_dynamic_smem(weights_kernel));
     int per_sm = 0;
     RBFFD_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, weights_kernel, 32 * wpb, smem));
     if (per_sm < 1) return RBFFD_ERR_INVALID_ARG;
