@@ -15,8 +15,8 @@ from fixtures import disk_nodes
 pytestmark = pytest.mark.gpu
 
 
-def _run(jobs, repeats):
-    """Each job () -> tensors from its own thread and stream, `repeats` times."""
+def _run(jobs, repeats, burst):
+    """Each job () -> tensors from its own thread and stream, `repeats` bursts of calls."""
     alone = [job() for job in jobs]
     torch.cuda.synchronize()
     wrong = []
@@ -25,7 +25,8 @@ def _run(jobs, repeats):
         try:
             with torch.cuda.stream(torch.cuda.Stream()):
                 for _ in range(repeats):
-                    got = job()
+                    for _ in range(burst):
+                        got = job()
                     torch.cuda.current_stream().synchronize()
                     if not all(torch.equal(a, b) for a, b in zip(got, ref)):
                         wrong.append("bits")
@@ -49,7 +50,7 @@ def test_weights_of_two_sizes_from_several_threads(lib, a, b):
     for m, n in (a, b):
         idx = rbffd.rbffd_stencils(xy, n)
         jobs.append(lambda m=m, idx=idx: rbffd.rbffd_weights(xy, idx, m))
-    _run(jobs, 1000)
+    _run(jobs, 40, 150)
 
 
 def test_one_launch_solves_of_two_sizes_from_several_threads(lib):
@@ -64,4 +65,4 @@ def test_one_launch_solves_of_two_sizes_from_several_threads(lib):
                                                                val.ravel())))
         b = torch.from_numpy(np.random.default_rng(N).standard_normal(N)).cuda()
         jobs.append(lambda A=A, b=b: (r.rbffd_solve(A, b, None, r.make_opts(tol=1e-12))[0],))
-    _run(jobs, 40)
+    _run(jobs, 40, 1)
