@@ -156,13 +156,14 @@ int rbffd_weights(const double* xy, const int32_t* idx, int64_t N, int32_t n, in
 /* double-float (warps_per_block 1..4: 2..8 stencils per block); 9 / 10:    */
 /* a quarter of a warp (8 threads), four stencils per warp (4..16 per      */
 /* block).                                                                  */
-/* Where 1 <= m <= 6 and n <= 64 every FP64 null-space configuration (0, 2, */
-/* 3, 7, 9) first runs the refined solve -- float32 elimination, then       */
-/* residuals and sums in 64-bit fixed point, to at least the accuracy of   */
-/* the FP64 elimination -- and the elimination, one warp per stencil, only */
-/* for the stencils whose refinement does not converge fast enough or that */
-/* may be singular; the configurations then give the same bits and take    */
-/* the same time, and autotuning times the default one for all of them.     */
+/* Where 1 <= m <= 6 and 6 < n <= 64 (n = s: sets of N s >= 81,920) every   */
+/* FP64 null-space configuration (0, 2, 3, 7, 9) first runs the refined     */
+/* solve -- float32 elimination, then residuals and sums in 64-bit fixed   */
+/* point -- and its elimination only for the stencils whose refinement     */
+/* does not converge fast enough or that may be singular; the              */
+/* configurations give the same bits and differ in the time of those       */
+/* stencils, and autotuning keeps the default one unless another is        */
+/* clearly faster.                                                          */
 /* The default is FP64: 2 (two warps per stencil) for m >= 5 when it fits,  */
 /* 9 (a quarter warp, warps_per_block 2) for m <= 2 with n <= 16, 7 (half a */
 /* warp, warps_per_block 2) for other m <= 4 with n <= 32, 0 for other     */

@@ -913,7 +913,12 @@ int launch_m(const double2* xy, const int32_t* idx, int64_t N, int n, double* w,
 
 }  // namespace
 
-bool refined_applies(int n, int m) { return m >= 1 && m <= 6 && n <= 64 && n >= (m + 1) * (m + 2) / 2; }
+// (n <= 6, m <= 2: the elimination is as short as the second launch.  100k even
+// nodes, elimination / refined solve: m = 1, n = 6 0.233 / 0.233 ms, m = 2,
+// n = 6 0.239 / 0.263, m = 2, n = 7 0.33 / 0.28.)
+bool refined_applies(int n, int m) {
+    return m >= 1 && m <= 6 && n <= 64 && n >= (m + 1) * (m + 2) / 2 && n > 6;
+}
 
 int refined_weights(const double* xy, const int32_t* idx, int64_t N, int32_t n, int32_t m, double* w,
                     int32_t* node_status, cudaStream_t st) {

@@ -542,8 +542,12 @@ struct NsDF {
 // and handed to the others through shared memory: computed by every thread
 // of the group they cost as many FP64 lane-operations as a full row update.
 //
-// MARKED (NT = 32 only): solves just the stencils whose first weight is
-// kWeightsMark; a warp looks at 32 stencils at a time.
+// MARKED: solves just the stencils whose first weight is kWeightsMark.  A
+// group owns the same stencils as without MARKED (every total_warps-th one),
+// so that marks spread over all groups however they lie and whatever N is,
+// and looks at one per lane (32 at most) at a time.  (32 consecutive stencils
+// per warp instead: 2,000 stencils, m = 6, n = 56, all marked: 8.9 ms; the
+// elimination of every stencil 0.57.)
 template <int NT, class R, bool MARKED = false>
 __global__ void __launch_bounds__(128) weights_ns_kernel(const double2* __restrict__ xy, const int* __restrict__ idx,
                                                          int N, int n, int m, int s, int LDQ, int LDS,
@@ -591,29 +595,38 @@ __global__ void __launch_bounds__(128) weights_ns_kernel(const double2* __restri
     auto ldc = [&](const S* p) -> V { return R::ld(&RB_PT(p, Phi, region)); };
     auto stc = [&](S* p, V v) { R::st(&RB_PT(p, Phi, region), v); };
 
-    static_assert(!MARKED || NT == 32, "marked stencils are found by whole warps");
-    int64_t ahead = (int64_t)(blockIdx.x * wpb + wib) * (MARKED ? 32 : 1);  // next stencil, or group of 32
-    unsigned found = 0;  // marked stencils not yet solved of the 32 from `from` on
-    int from = 0;
+    int64_t ahead = blockIdx.x * wpb + wib;  // next stencil
+    unsigned found = 0;  // marked stencils not yet solved: bit k for from + k total_warps
+    int64_t from = 0;
     auto next = [&](int& node) -> bool {
         if constexpr (!MARKED) {
             node = (int)ahead;
             ahead += total_warps;
             return node < N && node >= 0;
         } else {
-            while (found == 0) {
-                if (ahead >= N) return false;
-                from = (int)ahead;
-                found = __ballot_sync(0xffffffffu, ahead + lane < N && (unsigned long long)__double_as_longlong(
-                                                                           w[(ahead + lane) * n]) == kWeightsMark);
-                ahead += (int64_t)total_warps * 32;
+            // the groups of a warp look and solve together (-1: none left for this group)
+            constexpr int LOOK = NT < 32 ? NT : 32;
+            const int at = lane & (LOOK - 1), bit0 = (int)(threadIdx.x & 31) & ~(LOOK - 1);
+            for (;;) {
+                const bool look = found == 0 && ahead < N;
+                if (!__any_sync(0xffffffffu, look)) break;
+                const int64_t k = ahead + (int64_t)at * total_warps;
+                const bool mark = look && k < N &&
+                                  (unsigned long long)__double_as_longlong(w[k * n]) == kWeightsMark;
+                const unsigned b = __ballot_sync(0xffffffffu, mark) >> bit0;
+                if (look) {
+                    found = LOOK < 32 ? b & ((1u << (LOOK & 31)) - 1u) : b;
+                    from = ahead;
+                    ahead += (int64_t)total_warps * LOOK;
+                }
             }
-            node = from + __ffs(found) - 1;
+            node = found ? (int)(from + (int64_t)(__ffs(found) - 1) * total_warps) : -1;
             found &= found - 1;
-            return true;
+            return __any_sync(0xffffffffu, node >= 0) != 0;
         }
     };
     for (int node; next(node);) {
+        if (MARKED && node < 0) continue;
         const int* sten = idx + (int64_t)node * n;
         const double2 c = cxy[node];
 
@@ -1061,6 +1074,16 @@ bool cfg_is_ns64(const WCfg& c) {
     return c.kernel == 0 || c.kernel == 2 || c.kernel == 3 || c.kernel == 7 || c.kernel == 9;
 }
 
+// Whether a call runs the refined solve first.  At n = s small sets do not: an
+// elimination without a reduced matrix is short, a few of their stencils are
+// always left, and the call then takes the time of both (elimination / with
+// the refined solve, us: m = 4, n = 15 2k nodes 65 / 85, 8k 112 / 106; m = 6,
+// n = 28 1k 90 / 115, 4k 216 / 198).
+bool cfg_refines(const WCfg& c, int64_t N, int n, int m) {
+    const int s = (m + 1) * (m + 2) / 2;
+    return cfg_is_ns64(c) && !c.direct && refined_applies(n, m) && (n > s || N * s >= 81920);
+}
+
 bool cfg_is_df(const WCfg& c) { return (c.kernel >= 4 && c.kernel <= 6) || c.kernel == 8 || c.kernel == 10; }
 
 // The double-float null-space kernels: 1 <= m <= 6 (accuracy, see NsDF).
@@ -1079,7 +1102,8 @@ bool cfg_valid(const WCfg& c, int n, int m) {
 }
 
 // (The figures are of the elimination alone: it solves every stencil for
-// n > 64 or m > 6, and under RBFFD_WEIGHTS=ns64.)
+// n > 64 or m > 6 and under RBFFD_WEIGHTS=ns64, else those that the refined
+// solve leaves.)
 WCfg default_cfg(int n, int m) {
     WCfg c;
     // FP64 by default: null-space elimination (m >= 1: the form needs r^3
@@ -1161,8 +1185,7 @@ int launch_ns(const WCfg& c, const double2* xy, const int32_t* idx, int64_t N, i
     int per_sm = 0;
     RBFFD_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT * spb, smem));
     if (per_sm < 1) return RBFFD_ERR_INVALID_ARG;
-    const int64_t per_block = (int64_t)spb * (MARKED ? 32 : 1);
-    const int64_t need = (N + per_block - 1) / per_block;
+    const int64_t need = (N + spb - 1) / spb;
     const int blocks = (int)std::min<int64_t>(need, (int64_t)per_sm * sm_count());
     kern<<<blocks, NT * spb, smem, st>>>(xy, idx, (int)N, n, m, g.s, g.LDQ, g.LDS, g.bytes, w, node_status, cxy,
                                          (int)Nd, op);
@@ -1174,16 +1197,17 @@ int launch_weights(const WCfg& c, const double* xy, const int32_t* idx, int64_t 
     if (!cfg_valid(c, n, m)) return RBFFD_ERR_INVALID_ARG;
     const double2* p = reinterpret_cast<const double2*>(xy);
     int rc = RBFFD_OK;
-    if (cfg_is_ns64(c) && !c.direct && refined_applies(n, m)) {
+    if (cfg_refines(c, N, n, m)) {
         // every FP64 null-space configuration: the refined solve, then the
-        // elimination (one warp per stencil) of the stencils it left
+        // configuration's elimination of the stencils it left
         rc = refined_weights(xy, idx, N, n, m, w, node_status, st);
         if (rc != RBFFD_OK) return rc;
         note_launches(1);
-        WCfg left{0, 1};
-        size_t smem = 0;
-        left.wpb = warps_per_block_for(smem_per_stencil(0, n, m), &smem);
-        rc = launch_ns<32, NsF64, true>(left, p, idx, N, n, m, w, node_status, st);
+        rc = c.kernel == 2   ? launch_ns<64, NsF64, true>(c, p, idx, N, n, m, w, node_status, st)
+             : c.kernel == 3 ? launch_ns<128, NsF64, true>(c, p, idx, N, n, m, w, node_status, st)
+             : c.kernel == 7 ? launch_ns<16, NsF64, true>(c, p, idx, N, n, m, w, node_status, st)
+             : c.kernel == 9 ? launch_ns<8, NsF64, true>(c, p, idx, N, n, m, w, node_status, st)
+                             : launch_ns<32, NsF64, true>(c, p, idx, N, n, m, w, node_status, st);
     } else if (c.kernel == 1) {
         WeightsGeom g = weights_geom(n, m);
         const int wpb = c.wpb;
@@ -1269,12 +1293,16 @@ extern "C" int rbffd_weights_autotune(const double* xy, const int32_t* idx, int6
         all.push_back(WCfg{10, wpb});
     }
     std::vector<WCfg> cands;
+    // Where the refined solve applies, the FP64 null-space configurations
+    // differ only in the elimination of the stencils it leaves: the default
+    // one is timed first and another has to be clearly faster.
     const WCfg def = default_cfg(n, m);
+    const bool shared = refined_applies(n, m);
+    if (shared) std::stable_partition(all.begin(), all.end(), [&](const WCfg& c) {
+        return c.kernel == def.kernel && c.wpb == def.wpb;
+    });
     for (const WCfg& c : all) {
         if (!cfg_valid(c, n, m)) continue;
-        // the FP64 null-space configurations share the refined solve where it
-        // applies: the default one stands for them
-        if (cfg_is_ns64(c) && refined_applies(n, m) && (c.kernel != def.kernel || c.wpb != def.wpb)) continue;
         if (precision == RBFFD_WEIGHTS_FP64 && cfg_is_df(c)) continue;
         if (precision == RBFFD_WEIGHTS_DF && !cfg_is_df(c)) continue;
         cands.push_back(c);
@@ -1302,7 +1330,8 @@ extern "C" int rbffd_weights_autotune(const double* xy, const int32_t* idx, int6
         }
         if (rc != RBFFD_OK) break;
         const double per = best_ms * 1e6 / (double)S;  // ms per 1e6 stencils
-        if (per < win_ms) {
+        const bool tie = shared && cfg_is_ns64(c) && cfg_is_ns64(win) && per > 0.97 * win_ms;
+        if (per < win_ms && !tie) {
             win_ms = per;
             win = c;
         }
