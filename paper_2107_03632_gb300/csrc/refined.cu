@@ -182,6 +182,12 @@ __device__ __forceinline__ uint64_t fx_scale(int64_t hi, int64_t lo, int sh) {
 constexpr float kRefPivot = 1e-5f;   // smaller pivots of P: the FP64 elimination decides
 constexpr float kRefRate = 0.125f;   // slowest accepted reduction per refinement step
 constexpr int kRefMaxSolves = 10;
+// Exponents of the corrections' scales: every power of two that the kernel
+// forms from one (2^(25 - e), 2^(e - 49), 2^(e0 - 60), 2^(el - 49), with
+// el <= e0 + kRefLambda) is a normal float.  Smaller corrections take the
+// lowest scale: they are below the unit of the sums anyway.
+constexpr int kRefMinExp = -66, kRefMaxExp = 60, kRefLambda = 12;
+static_assert(kRefMinExp - 60 >= -126 && 25 - kRefMinExp <= 127, "scales of the smallest corrections");
 // Predicted error at which refinement stops, relative to max |w|: about a
 // tenth of the FP64 elimination's median error (3e-15, 2e-14, 8e-14 at m = 2,
 // 4, 6), and full accuracy near n = s, where the elimination is as accurate.
@@ -727,8 +733,9 @@ __global__ void __launch_bounds__(NT * H > 32 ? NT * H : 128, ref_min_blocks<NT,
                 const unsigned um = ref_max<TT>(bad ? 0x7f800000u : __float_as_uint(fabsf(dj)), red, it & 1);
                 if (um == 0u && it > 0) break;  // the residual is zero
                 const float m = __uint_as_float(um);
-                const int e = (int)(um >> 23) - 126;  // 2^e > m
-                if (um >= 0x7f800000u || e < -100 || e > 60) {  // not finite, a failed check, or out of scale
+                const int em = (int)(um >> 23) - 126, e = max(em, kRefMinExp);  // 2^e > m
+                // not finite, a failed check, or out of scale
+                if (um >= 0x7f800000u || e > kRefMaxExp || (it == 0 && em < kRefMinExp)) {
                     ok = false;
                     break;
                 }
@@ -829,8 +836,8 @@ __global__ void __launch_bounds__(NT * H > 32 ? NT * H : 128, ref_min_blocks<NT,
                     rg = (float)rgi * fx_pow2f(e0 - 60);
                 }
                 const unsigned ul = ref_max<TT>(__float_as_uint(fabsf(dl)), red, 2 + (it & 1));
-                const int el = max((int)(ul >> 23) - 126, -100);
-                if (ul >= 0x7f800000u || el > e0 + 12) {  // (e0 + 12: l in the range of the sums)
+                const int el = max((int)(ul >> 23) - 126, kRefMinExp);
+                if (ul >= 0x7f800000u || el > e0 + kRefLambda) {  // (l in the range of the sums)
                     ok = false;
                     break;
                 }
