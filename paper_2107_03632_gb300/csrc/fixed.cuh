@@ -9,7 +9,8 @@
 //   coordinate  X = x 2^61            |x| <= 1
 //   r^2         q = r^2 2^58          r <= 2
 //   r           s = r 2^60
-//   r^3, p_k    v = value 2^56        r^3 <= 8, |p_k| <= 1
+//   r^3         v = value 2^56        r^3 <= 8
+//   p_k         v = value 2^61        |p_k| <= 1
 //
 // A 64-bit value is split into two signed 32-bit digits v = hi 2^32 + lo, so
 // that every partial product is a signed 32 x 32 -> 64 multiply-add.
@@ -119,10 +120,10 @@ __host__ __device__ __forceinline__ int64_t fx_cube(int64_t q, int64_t s) {
     return (int64_t)((uint64_t)h << 2) + (c >> 30);
 }
 
-// x p 2^56 of a coordinate (2^61) and a value (2^56), |x p| <= 1.
+// x p 2^61 of a coordinate and a monomial (2^61 both), |x p| <= 1.
 __host__ __device__ __forceinline__ int64_t fx_mono(const Digits& x, const Digits& p) {
-    const int64_t h = fx_mul32(x.hi, p.hi);                               // unit 2^-53
-    const int64_t c = fx_mul32(x.hi, p.lo) + fx_mul32(x.lo, p.hi);        // unit 2^-85
+    const int64_t h = fx_mul32(x.hi, p.hi);                               // unit 2^-58
+    const int64_t c = fx_mul32(x.hi, p.lo) + fx_mul32(x.lo, p.hi);        // unit 2^-90
     return (int64_t)((uint64_t)h << 3) + (c >> 29);
 }
 

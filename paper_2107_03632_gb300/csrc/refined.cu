@@ -4,17 +4,21 @@
 // The saddle-point system of a stencil (weights.cu: [Phi P; P^T 0] [w; l] =
 // [f; g] in scaled coordinates) is eliminated once in float32 by the
 // null-space method, and the solution is refined: the residual of the
-// current (w, l) is formed in 64-bit fixed point from kernel values and
-// monomials known to 2^-54 (fixed.cuh), the float32 factors solve for a
-// correction, and the sum is kept in 64-bit fixed point.  Each step reduces
-// the error by the float32 elimination's relative error (1e-3 to 1e-6 on
-// node sets of even density), so three to five solves reach the accuracy of
+// current (w, l) is formed in 64-bit fixed point from kernel values known to
+// 2^-54 and monomials known to 2^-59 (fixed.cuh), the float32 factors solve
+// for a correction, and the sum is kept in 64-bit fixed point.  Each step
+// reduces the error by the float32 elimination's relative error (1e-3 to 1e-6
+// on node sets of even density), so three to five solves reach the accuracy of
 // the residual, which is that of the kernel values: more bits than FP64
-// elimination carries.  Largest error per stencil relative to its largest
-// weight, against extended precision (disk of 1,321 nodes, 50 sampled rows;
-// here / FP64 elimination): m = 2, n = 12 1.3e-15 / 1.6e-14; m = 4, n = 30
-// 8.8e-15 / 1.7e-13; m = 6, n = 56 5.2e-13 / 3.5e-12.  A stencil whose corrections do not fall by 8x per step,
-// whose pivots are small, or whose values leave the fixed-point ranges is
+// elimination carries.  (The monomials need more than the kernel values: near
+// n = s they determine the weights alone, and everywhere the multipliers l, up
+// to 2^12 times the weights, carry their errors into the residual.  With units
+// of 2^-56 for both, m = 5, n = 22 had 3.7e-14 below.)  Largest error per
+// stencil relative to its largest weight, against 180-bit fixed point (disk of
+// 2,000 nodes, 15 sampled rows; here / FP64 elimination): m = 2, n = 12 8.3e-16
+// / 1.6e-14; m = 4, n = 30 6.6e-15 / 4.5e-13; m = 5, n = 22 2.7e-15 / 1.6e-14;
+// m = 6, n = 56 4.4e-14 / 8.4e-13.  A stencil whose corrections do not fall by
+// 8x per step, whose pivots are small, or whose values leave the fixed-point ranges is
 // marked and solved by the FP64 elimination kernel (weights.cu) in a second
 // launch, which also decides every singular case.
 //
@@ -51,7 +55,7 @@ __host__ __device__ constexpr int ref_ks(int s) { return s <= 4 ? 4 : s <= 8 ? 8
 //   phi   digits of |x_j - x_k|^3 2^56, entry [t - 1][j] for k = j + t mod n,
 //         t = 1 .. n/2: every pair once (t = n/2 twice for even n), and both
 //         of a thread's accesses in the residual are unit-stride
-//   pd    digits of the monomials 2^56, [j][k], odd stride.  Before they are
+//   pd    digits of the monomials 2^61, [j][k], odd stride.  Before they are
 //         formed the region holds W^T at its start and Phi11 at its end
 //   F1    [Phi11; Phi21], n rows of LS (pivot nodes first): rows S.. become
 //         T^T = (Phi12 - Phi11 X^T)^T, rows 0..S are inside pd
@@ -183,7 +187,7 @@ constexpr float kRefPivot = 1e-5f;   // smaller pivots of P: the FP64 eliminatio
 constexpr float kRefRate = 0.125f;   // slowest accepted reduction per refinement step
 constexpr int kRefMaxSolves = 10;
 // Exponents of the corrections' scales: every power of two that the kernel
-// forms from one (2^(25 - e), 2^(e - 49), 2^(e0 - 60), 2^(el - 49), with
+// forms from one (2^(25 - e), 2^(e - 54), 2^(e0 - 60), 2^(el - 54), with
 // el <= e0 + kRefLambda) is a normal float.  Smaller corrections take the
 // lowest scale: they are below the unit of the sums anyway.
 constexpr int kRefMinExp = -66, kRefMaxExp = 60, kRefLambda = 12;
@@ -652,7 +656,7 @@ __global__ void __launch_bounds__(NT * H > 32 ? NT * H : 128, ref_min_blocks<NT,
                 const Digits xd = fx_digits(at.x), yd = fx_digits(at.y);
                 int2* pr = pd + nd * LP;
                 Digits up[M + 1];  // the previous degree's digits
-                up[0].hi = 1 << 24;
+                up[0].hi = 1 << 29;
                 up[0].lo = 0;
                 pr[0] = make_int2(up[0].hi, up[0].lo);
                 int cur = 1;
@@ -764,7 +768,8 @@ __global__ void __launch_bounds__(NT * H > 32 ? NT * H : 128, ref_min_blocks<NT,
                 // residual: r -= Phi d, rg -= P^T d, exact sums of the digits'
                 // products, of unit 2^(e - 49) (H) and 2^(e - 81) (L).  The 64-bit
                 // wrap of r is harmless while the true residual is below 2^(e0 + 2)
-                const float hs = fx_pow2f(e - 49);
+                // (the monomials' digits have units 2^-5 of the kernel values')
+                const float hs = fx_pow2f(e - 49), gs = fx_pow2f(e - 54);
                 float check = rf;
                 int64_t HH = 0, LL = 0;
                 if (nd < n) {
@@ -831,8 +836,8 @@ __global__ void __launch_bounds__(NT * H > 32 ? NT * H : 128, ref_min_blocks<NT,
                         GL += part[k * S + t].y;
                     }
                     if (it == 0) rgi = grhs != 0.f && 61 - e0 < 64 ? (int64_t)(1ull << (61 - e0)) : 0;
-                    rgi = (int64_t)((uint64_t)rgi - fx_scale(GH, GL, 11 - (e0 - e)));
-                    bad |= !(fabsf(rg - (float)GH * hs) < fx_pow2f(e0));
+                    rgi = (int64_t)((uint64_t)rgi - fx_scale(GH, GL, 6 - (e0 - e)));
+                    bad |= !(fabsf(rg - (float)GH * gs) < fx_pow2f(e0));
                     rg = (float)rgi * fx_pow2f(e0 - 60);
                 }
                 const unsigned ul = ref_max<TT>(__float_as_uint(fabsf(dl)), red, 2 + (it & 1));
@@ -853,8 +858,8 @@ __global__ void __launch_bounds__(NT * H > 32 ? NT * H : 128, ref_min_blocks<NT,
                         PH += fx_mul32(a.x, d);
                         PL += fx_mul32(a.y, d);
                     }
-                    ri = (int64_t)((uint64_t)ri - fx_scale(PH, PL, 11 - (e0 - el)));
-                    check -= (float)PH * fx_pow2f(el - 49);
+                    ri = (int64_t)((uint64_t)ri - fx_scale(PH, PL, 6 - (e0 - el)));
+                    check -= (float)PH * fx_pow2f(el - 54);
                     bad |= !(fabsf(check) < fx_pow2f(e0));
                     rf = (float)ri * fx_pow2f(e0 - 60);
                 }
