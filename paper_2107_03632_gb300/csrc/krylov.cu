@@ -1442,10 +1442,19 @@ double rel_of(const KState& s) {
 // the measured time per iteration: early BiCGSTAB iterations often reduce
 // the residual slowly and would make the prediction far too long.  Without
 // a measurement: 4, doubling, within the same time cap.
+// Iterations in one launch that ends itself (pass64_kernel) cost nothing past
+// the end of the pass and have a fixed number per round trip instead, whatever
+// the clock says: such a launch needs a place on every SM at once, and beside
+// another stream's kernels each round trip can be a wait for one of them.
+// (Sized by the time per iteration, which then holds that wait, chunks shrank
+// to two: 10k rows beside weight solves of 16 ms took 2.8 s, now 0.1; alone
+// 9.9 ms, now 9.5.)
 constexpr double kChunkMs = 4.0;
+constexpr int kOneLaunch = 512;
 
 struct ChunkPlan {
     int chunk = 4;
+    bool one_launch = false;
     double rate2 = 0.0;
     double ms_per_iter = 0.0;
     int cap() const {
@@ -1460,10 +1469,12 @@ struct ChunkPlan {
     }
     // first chunk of a pass starting at |r|^2 = start2 that ends at target2
     void start(double start2, double target2) {
+        if (one_launch) return;
         const int n = need(start2, target2, rate2);
         if (n > 0) chunk = std::min(std::max(n, 1), cap());
     }
     void update(const KState& hs, double start2, int ran, double ms) {
+        if (one_launch) return;
         if (ran > 0 && ms > 0.0) ms_per_iter = ms_per_iter > 0.0 ? 0.5 * (ms_per_iter + ms / ran) : ms / ran;
         const double target2 = std::max(hs.tol2, hs.repl2 * hs.rmax2);
         if (hs.iter > 0 && hs.rnorm2 > 0.0 && start2 > 0.0) {
@@ -1506,7 +1517,8 @@ struct StagMonitor {
 // error.  rel_start: the relative residual at the pass start, it_base: the
 // iterations before this pass.  With profiling on, only the SpMV launches of
 // iterations that ran are accounted (launches after the pass ended return at
-// once and are dropped).
+// once and are dropped).  iter(events, n): enqueues n iterations, or kOneLaunch
+// of them in one launch, which it says by setting plan.one_launch.
 template <class IterFn>
 int run_chunks(const Work& w, KState* hs, cudaStream_t st, ChunkPlan& plan, IterFn iter, StagMonitor* mon = nullptr,
                double rel_start = 0.0, long long it_base = 0) {
@@ -1682,7 +1694,8 @@ int solve_fp64(const rbffd_csr& A, const double* b, double* x, const rbffd_solve
         }
         const int f = run_chunks(
             w, &hs, st, chunk, [&](std::vector<int>& ev, int count) {
-                if (pass64(A, x, w, count, st)) return;
+                chunk.one_launch = pass64(A, x, w, kOneLaunch, st);
+                if (chunk.one_launch) return;
                 for (int c = 0; c < count; ++c) iter64(tpr, A, x, w, st, ev, c > 0);
             }, &mon,
             rel, total);
