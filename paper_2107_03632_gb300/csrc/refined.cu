@@ -356,7 +356,8 @@ __global__ void __launch_bounds__(NT * H > 32 ? NT * H : 128, ref_min_blocks<NT,
     const bool mine = t < n;  // holds a node's row, residual and weight
     const int spb = blockDim.x / TT;
 
-    for (int node = blockIdx.x * spb + threadIdx.x / TT; node < N; node += gridDim.x * spb) {
+    // (unsigned: past 2^31 - 1 the index ends the loop instead of turning negative)
+    for (unsigned node = blockIdx.x * spb + threadIdx.x / TT; node < (unsigned)N; node += gridDim.x * spb) {
         bool ok = true;  // uniform over the stencil's threads
         // ---- shift and scale (FP64) ------------------------------------------
         const double2 c = xy[node];

@@ -91,7 +91,8 @@ __global__ void __launch_bounds__(128) weights_kernel(const double2* __restrict_
     auto a = [&](size_t i) -> double& { return RB_AT(A, i, smem_doubles); };
     const int total_warps = gridDim.x * wpb;
 
-    for (int node = blockIdx.x * wpb + wib; node < N; node += total_warps) {
+    // (unsigned: past 2^31 - 1 the index ends the loop instead of turning negative)
+    for (unsigned node = blockIdx.x * wpb + wib; node < (unsigned)N; node += total_warps) {
         const int* sten = idx + (int64_t)node * n;
         const double2 c = cxy[node];
 
