@@ -221,20 +221,4 @@ __device__ __forceinline__ double sqrt64(double a) {
     return fma(fma(-s, s, a), hy, s);
 }
 
-// Block-wide sum; every thread gets the result.  `sh` needs 32 doubles.
-template <int BLOCK>
-__device__ __forceinline__ double block_sum(double v, double* sh) {
-    constexpr int W = BLOCK / 32;
-    v = warp_sum(v);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) sh[wid] = v;
-    __syncthreads();
-    double t = (lane < W) ? sh[lane] : 0.0;
-    if (wid == 0) t = warp_sum(t);
-    if (threadIdx.x == 0) sh[0] = t;
-    __syncthreads();
-    return sh[0];
-}
-
 }  // namespace rbffd

@@ -215,7 +215,7 @@ __device__ __forceinline__ double row_dot64(const int64_t* __restrict__ row_ptr,
 // unevaluated pair (TwoSum, Knuth), so the residual is accurate to about
 // eps |r_i| instead of eps sum |a x| (the latter reaches 1e-10 of |b| on the
 // finest m = 6 workload).  ~10 FP64 operations per entry: the rows
-// that residual_wide below does not take.
+// that row_residual64 below does not take.
 __device__ __forceinline__ void two_sum64(double a, double b, double& s, double& e) {
     s = __dadd_rn(a, b);
     const double bb = __dadd_rn(s, -a);
