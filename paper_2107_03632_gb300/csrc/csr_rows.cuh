@@ -71,6 +71,9 @@ __device__ __forceinline__ void rows32(const int64_t* __restrict__ row_ptr, cons
 // L1 wavefronts of two: 16-byte pieces of 16 rows are 16 lines per load of 32
 // entries, 64-byte pieces of 4 rows are 4) are not a round trip per four
 // entries.  For float32: in FP64 the 64 registers more cost what it gives.
+// The gathers are unconditional (x_0 past a row's end, not used): as
+// conditional ordinary loads they are not all in flight before the next row's
+// loads (1M rows of 30 entries: a sweep 72 us, now 60; mixed solve 20.6 -> 19.7).
 template <typename T, int TPR, class F>
 __device__ __forceinline__ void rows32_ahead(const int64_t* __restrict__ row_ptr, const int* __restrict__ col,
                                              const T* __restrict__ val, Live<T> x, int64_t nx, int64_t N, F&& f) {
@@ -114,7 +117,7 @@ __device__ __forceinline__ void rows32_ahead(const int64_t* __restrict__ row_ptr
             const int64_t kj = k, cj = cnt;
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                xv[u] = u * TPR < cj ? RB_AT(x, c[u], nx) : T(0);
+                xv[u] = RB_AT(x, c[u], nx);
                 w[u] = v[u];
             }
             if (j + 1 == TPR) {

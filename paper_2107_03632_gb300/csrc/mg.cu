@@ -134,7 +134,7 @@ struct RowHead {
         (void)nx;  // length of x: bound of the checked build's tests
         T xv[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) xv[u] = a + sub + u * TPR < e ? RB_AT(x, c[u], nx) : T(0);
+        for (int u = 0; u < U; ++u) xv[u] = RB_AT(x, c[u], nx);  // (x_0 past the row's end, not used)
         T s = T(0);
 #pragma unroll
         for (int u = 0; u < U; ++u)
