@@ -181,9 +181,9 @@ SPMV_DF_TRAFFIC = {"source_sha256_16": "ea63d4b54b1529b9", "traffic_over_algorit
 # n = 56, from one ncu capture: DRAM read + write and warp instructions per
 # stencil.  Valid only at that (n, m) and while the kernel's sources are the
 # ones captured.
-WEIGHTS_F64_TRAFFIC = {"source_sha256_16": "12f4cc266207f88f", "n": 56, "m": 6,
-                       "bytes_per_node": (249.541632e6 + 406.857984e6) / 1000870.0,
-                       "warp_instr_per_node": 34599512456 / 1000870.0}
+WEIGHTS_F64_TRAFFIC = {"source_sha256_16": "30217bca79a7bc84", "n": 56, "m": 6,
+                       "bytes_per_node": (250.715136e6 + 407.757312e6) / 1001767.0,
+                       "warp_instr_per_node": 34685612020 / 1001767.0}
 
 
 def weights_source_hash():
@@ -197,7 +197,7 @@ def weights_source_hash():
 def weights_refined(n: int, m: int) -> bool:
     """Whether the FP64 weights come from the refined float32 solve (the
     library's rule; RBFFD_WEIGHTS=ns64 asks for the elimination)."""
-    return 1 <= m <= 6 and n <= 64 and os.environ.get("RBFFD_WEIGHTS", "") != "ns64"
+    return 1 <= m <= 6 and 6 < n <= 64 and os.environ.get("RBFFD_WEIGHTS", "") != "ns64"
 
 
 def spmv_df_source_hash():

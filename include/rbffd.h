@@ -592,6 +592,9 @@ int rbffd_solve_batched(const rbffd_batch_desc* desc, int32_t n_inst, const doub
 /* V-cycle, 118 B per (node, rhs) + 4 passes x 8 nnz on the finest level.   */
 /* Profiling is process-wide, off by default, and meant for one thread and   */
 /* one device.  rbffd_profile_read waits for bracketed launches to finish.   */
+/* With profiling on, FP64 solves of small systems without multigrid run    */
+/* the separate kernels instead of whole iterations in one launch, so their */
+/* times are not those of a run without it.                                  */
 /* ------------------------------------------------------------------------ */
 typedef struct rbffd_profile {
     int64_t launches;         /* kernels launched since the last reset */
