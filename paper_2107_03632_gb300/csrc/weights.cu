@@ -2,7 +2,7 @@
 // held in shared memory and solved by one, two or four warps (sm_103a), in
 // FP64 or in double-float arithmetic (opt-in).  The FP64 null-space
 // configurations run the refined solve of refined.cu first where it applies
-// (n <= 64, 1 <= m <= 6) and the elimination here for the stencils it leaves.
+// (6 < n <= 64, 1 <= m <= 6) and the elimination here for the stencils it leaves.
 //
 // Sec. II, Eq. 1: (L u)(x_c) ~ sum_j w_j u(x_j) over the stencil of x_c.
 // Sec. V: Phi(r) = r^3 augmented with the monomials of degree <= m, L = lap.
